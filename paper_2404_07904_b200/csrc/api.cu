@@ -26,6 +26,7 @@ cudaError_t launch_span_compose(const float *X_all, const float *lam_all, const 
 int         gate_bwd_slices(long long U, int N);
 cudaError_t launch_gate_fwd(const SeqArgs &a, const float *beta, void *o_out, void *k_out, void *i_out);
 cudaError_t launch_gate_bwd(const SeqArgs &a, const float *beta, float *partial, float *d_beta);
+cudaError_t launch_gate_reduce_beta(const float *partial, float *d_beta, int B, int H, int P, int dk, cudaStream_t stream);
 cudaError_t launch_alu_fwd_gated(const SeqArgs &a, const float *beta);
 cudaError_t launch_alu_bwd_gated(const SeqArgs &a, const float *beta, float *partial, float *d_beta);
 cudaError_t launch_tc_fwd(const SeqArgs &a);
@@ -103,6 +104,7 @@ void fill_args(SeqArgs &a, const hgrn2_desc *d, int C, void *stream, void *ws, c
     // float matrix per unit for units redone on the exact path
     a.seg_scratch = nullptr;
     a.exact_scratch = nullptr;
+    a.room = reinterpret_cast<float *>(static_cast<char *>(ws) + sizeof(StatusBlock));
     if (use_tc(d)) {
         char *p = static_cast<char *>(ws) + sizeof(StatusBlock) + saved_bytes_for(d, C, cu != nullptr);
         const size_t seg = cu ? tc_segment_scratch_bytes_packed(d) : tc_segment_scratch_bytes(d, C);
@@ -193,10 +195,10 @@ hgrn2_status fwd_impl(const hgrn2_desc *desc, const void *o, const void *f, cons
     a.o = o; a.f = f; a.i = i; a.S0 = S0; a.y = y; a.SN = SN;
     a.states = static_cast<float *>(saved);
     a.status = static_cast<StatusBlock *>(ws);
-    // The status word starts every call at zero.  On the tensor-core path the first kernel of the call does that
-    // itself (a separate clear between two kernels of a stream costs a microsecond of idle GPU each time);
-    // everywhere else, and when no kernel will run, it is a small asynchronous memset.
-    a.clear_status = use_tc(desc) && !empty;
+    // The status word starts every call at zero.  The first kernel of the call does that itself (a separate clear
+    // between two kernels of a stream costs a microsecond of idle GPU each time); when no kernel will run, and in
+    // front of the serial fp32 kernels, it is a small asynchronous memset.
+    a.clear_status = !empty;
     if (!a.clear_status && cudaMemsetAsync(ws, 0, sizeof(StatusBlock), a.stream) != cudaSuccess) return HGRN2_ERR_CUDA;
     if ((size_t)desc->B * desc->H == 0) return HGRN2_OK;
     if (desc->N == 0) {
@@ -207,7 +209,7 @@ hgrn2_status fwd_impl(const hgrn2_desc *desc, const void *o, const void *f, cons
         }
         return HGRN2_OK;
     }
-    cudaError_t e = use_tc(desc) ? launch_tc_fwd(a) : launch_alu_fwd(a);
+    cudaError_t e = use_tc(desc) ? launch_tc_fwd(a) : launch_fp32_fwd(a);
     return e == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
 }
 
@@ -230,7 +232,10 @@ hgrn2_status bwd_impl(const hgrn2_desc *desc, const void *o, const void *f, cons
     a.o = o; a.f = f; a.i = i; a.S0 = S0; a.dy = dy; a.dSN = dSN;
     a.d_o = d_o; a.d_f = d_f; a.d_i = d_i; a.dS0 = dS0;
     a.status = static_cast<StatusBlock *>(ws);
-    a.clear_status = use_tc(desc) && !empty;                     // see hgrn2_fwd
+    const bool tc = use_tc(desc);
+    a.states = const_cast<float *>(static_cast<const float *>(saved));
+    const bool serial = !tc && !empty && !fp32_bwd_supported(a);
+    a.clear_status = !empty && !serial;                          // see hgrn2_fwd
     if (!a.clear_status && cudaMemsetAsync(ws, 0, sizeof(StatusBlock), a.stream) != cudaSuccess) return HGRN2_ERR_CUDA;
     if ((size_t)desc->B * desc->H == 0) return HGRN2_OK;
     if (desc->N == 0) {
@@ -241,14 +246,12 @@ hgrn2_status bwd_impl(const hgrn2_desc *desc, const void *o, const void *f, cons
         }
         return HGRN2_OK;
     }
-    const bool tc = use_tc(desc);
-    if (saved) {
-        a.states = const_cast<float *>(static_cast<const float *>(saved));
-    } else {
+    if (!tc && !serial) return launch_fp32_bwd(a) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
+    if (!saved) {
         // re-create the chunk-start states inside the workspace with a states-only forward
         SeqArgs r = a;
         r.y = nullptr; r.SN = nullptr;
-        r.states = reinterpret_cast<float *>(static_cast<char *>(ws) + sizeof(StatusBlock));
+        r.states = a.room;
         cudaError_t e = tc ? launch_tc_fwd(r) : launch_alu_fwd(r);
         if (e != cudaSuccess) return HGRN2_ERR_CUDA;
         a.states = r.states;
@@ -282,7 +285,7 @@ namespace {
 // Gated entry points.  Tensor-core path: `saved` = [o | encoded gate | i] (bf16, what the element-wise kernel in front wrote)
 // followed by the ordinary saved data; the workspace = status block | room for all of that when saved is NULL |
 // segment scratch | exact-path scratch | partial sums of d_beta.  fp32 path: the ordinary saved data and workspace
-// plus one row of partial sums per unit.
+// plus one row of partial sums per unit and chunk.
 size_t gate_tensor_bytes(const hgrn2_desc *d) { return (size_t)d->B * d->H * d->N * d->dk * 2; }
 
 size_t saved_bytes_gated(const hgrn2_desc *d, int C)
@@ -293,7 +296,7 @@ size_t saved_bytes_gated(const hgrn2_desc *d, int C)
 size_t beta_partial_bytes(const hgrn2_desc *d)
 {
     const long long U = (long long)d->B * d->H;
-    const int P = use_tc(d) ? gate_bwd_slices(U, d->N) : 1;
+    const int P = use_tc(d) ? gate_bwd_slices(U, d->N) : fp32_dbeta_rows(d->N);
     return (((size_t)U * P * d->dk * sizeof(float)) + 255) & ~(size_t)255;
 }
 
@@ -354,7 +357,7 @@ hgrn2_status hgrn2_fwd_gated(const hgrn2_desc *desc, const void *zo, const void 
     a.o = zo; a.f = zf; a.i = zi; a.S0 = S0; a.y = y; a.SN = SN;
     a.status = static_cast<StatusBlock *>(ws);
     const bool tc = use_tc(desc);
-    a.clear_status = tc && !empty;
+    a.clear_status = !empty;
     if (!a.clear_status && cudaMemsetAsync(ws, 0, sizeof(StatusBlock), a.stream) != cudaSuccess) return HGRN2_ERR_CUDA;
     if ((size_t)desc->B * desc->H == 0) return HGRN2_OK;
     if (desc->N == 0) {
@@ -367,7 +370,7 @@ hgrn2_status hgrn2_fwd_gated(const hgrn2_desc *desc, const void *zo, const void 
     }
     if (!tc) {
         a.states = static_cast<float *>(saved);
-        return launch_alu_fwd_gated(a, beta) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
+        return launch_fp32_fwd_gated(a, beta) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
     }
     // the gates go to the head of `saved` (kept for the backward) or, for inference, of the workspace's room for it
     char *gates = saved ? static_cast<char *>(saved) : static_cast<char *>(ws) + sizeof(StatusBlock);
@@ -401,7 +404,9 @@ hgrn2_status hgrn2_bwd_gated(const hgrn2_desc *desc, const void *zo, const void 
     a.d_o = d_zo; a.d_f = d_zf; a.d_i = d_zi; a.dS0 = dS0;
     a.status = static_cast<StatusBlock *>(ws);
     const bool tc = use_tc(desc);
-    a.clear_status = tc && !empty;
+    if (!tc) a.states = const_cast<float *>(static_cast<const float *>(saved));
+    const bool serial = !tc && !empty && !fp32_bwd_supported(a);
+    a.clear_status = !empty && !serial;
     if (!a.clear_status && cudaMemsetAsync(ws, 0, sizeof(StatusBlock), a.stream) != cudaSuccess) return HGRN2_ERR_CUDA;
     const size_t beta_bytes = (size_t)desc->H * desc->dk * sizeof(float);
     if (empty) {                                 // no token: nothing depends on beta; the state gradient passes through
@@ -414,16 +419,18 @@ hgrn2_status hgrn2_bwd_gated(const hgrn2_desc *desc, const void *zo, const void 
         return HGRN2_OK;
     }
     if (!tc) {
-        if (saved) {
-            a.states = const_cast<float *>(static_cast<const float *>(saved));
-        } else {
+        if (serial) {                            // one unit, states re-created: see fp32_bwd_supported
             SeqArgs r = a;
             r.y = nullptr; r.SN = nullptr;
-            r.states = reinterpret_cast<float *>(static_cast<char *>(ws) + sizeof(StatusBlock));
+            r.states = a.room;
             if (launch_alu_fwd_gated(r, beta) != cudaSuccess) return HGRN2_ERR_CUDA;
-            a.states = r.states;
+            a.states = a.room;
+            return launch_alu_bwd_gated(a, beta, partial, d_beta) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
         }
-        return launch_alu_bwd_gated(a, beta, partial, d_beta) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
+        if (launch_fp32_bwd_gated(a, beta, d_beta ? partial : nullptr) != cudaSuccess) return HGRN2_ERR_CUDA;
+        if (!d_beta) return HGRN2_OK;
+        return launch_gate_reduce_beta(partial, d_beta, desc->B, desc->H, fp32_dbeta_rows(desc->N), desc->dk, a.stream) ==
+                       cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
     }
     const size_t gb = gate_tensor_bytes(desc);
     char *gates;

@@ -1,11 +1,9 @@
-// Chunkwise forward and backward of the HGRN2 recurrence on fp32 CUDA cores.
+// Serial fp32 kernels: one CTA per (batch, head) unit walks the chunks in order (forward) or in reverse (backward)
+// with the running state S (forward) or state gradient dS (backward) resident in shared memory.
 //
-// This is the path for float32 I/O (a single-pass bf16/tf32 tensor-core product cannot hold
-// a 1e-4 error bound) and for every shape the tensor-core kernels do not cover.  One CTA per
-// (batch, head) unit walks the chunks in order (forward) or in reverse (backward) with the
-// running state S (forward) or state gradient dS (backward) resident in shared memory.
-//
-// The per-unit bodies (and the chunk-local formulas they follow) are in chunk_alu.cuh.
+// Left for one case only, the backward of a single unit without saved states: its workspace holds one set of
+// boundary states, and the chunk-parallel kernels (chunk_fp32.cu) need two.  The per-unit bodies (chunk_alu.cuh)
+// are also the exact path of the tensor-core kernels.
 #include "chunk_alu.cuh"
 
 namespace hgrn2 {

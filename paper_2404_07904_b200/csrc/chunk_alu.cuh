@@ -1,9 +1,5 @@
-// Chunkwise forward and backward of the HGRN2 recurrence on fp32 CUDA cores.
-//
-// This is the path for float32 I/O (a single-pass bf16/tf32 tensor-core product cannot hold
-// a 1e-4 error bound) and for every shape the tensor-core kernels do not cover.  One CTA per
-// (batch, head) unit walks the chunks in order (forward) or in reverse (backward) with the
-// running state S (forward) or state gradient dS (backward) resident in shared memory.
+// Chunkwise forward and backward of one (batch, head) unit on fp32 CUDA cores, chunk after chunk, with the running
+// state S (forward) or state gradient dS (backward) resident in shared memory.
 //
 // Chunk-local form, derived from Eq. 3 by unrolling C steps.  Per chunk, q = o, k = 1 - f,
 // v = i, b_j = sum_{r<=j} log f_r (inclusive, per key dimension), Lam_j = exp(b_j):

@@ -86,10 +86,11 @@ struct SeqArgs {
     void *d_o, *d_f, *d_i;        // bwd out
     float *dS0;                   // nullable
     StatusBlock *status;
+    float *room = nullptr;        // fp32 path: the workspace's room for one set of boundary states
     void *seg_scratch;            // tensor-core path: scratch for sequences split into segments (nullable)
     float *exact_scratch = nullptr;   // tensor-core backward: [B*H][dk][dv] floats for units redone on the exact path
     float *totals = nullptr;      // tensor-core path: per-chunk decay totals inside the saved data (set by its launchers)
-    bool clear_status = false;    // tensor-core path: the first kernel of the call zeroes the status word itself
+    bool clear_status = false;    // the first kernel of the call zeroes the status word itself
     int start_aborted = 0;        // tensor-core path, debugging: every CTA starts as if its first wait had run out
     bool gate_enc = false;         // the f tensor holds the signed gate encoding (gated entry points)
     const int *cu = nullptr;      // packed batch: device array of B + 1 row offsets (B = sequences, N = total rows per head)
@@ -171,5 +172,12 @@ int         alu_default_chunk(int dk, int dv);
 bool        alu_chunk_supported(int dk, int dv, int C);
 cudaError_t launch_alu_fwd(const SeqArgs &a);
 cudaError_t launch_alu_bwd(const SeqArgs &a);
+// fp32 kernels, parallel over chunks (chunk_fp32.cu)
+bool        fp32_bwd_supported(const SeqArgs &a);
+int         fp32_dbeta_rows(int N);          // rows of partial sums per unit (gated backward)
+cudaError_t launch_fp32_fwd(const SeqArgs &a);
+cudaError_t launch_fp32_bwd(const SeqArgs &a);
+cudaError_t launch_fp32_fwd_gated(const SeqArgs &a, const float *beta);
+cudaError_t launch_fp32_bwd_gated(const SeqArgs &a, const float *beta, float *partial);
 
 }  // namespace hgrn2

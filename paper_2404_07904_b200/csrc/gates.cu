@@ -239,6 +239,12 @@ cudaError_t launch_gate_bwd(const SeqArgs &a, const float *beta, float *partial,
     return cudaGetLastError();
 }
 
+cudaError_t launch_gate_reduce_beta(const float *partial, float *d_beta, int B, int H, int P, int dk, cudaStream_t stream)
+{
+    gate_reduce_beta_kernel<<<H, 128, 0, stream>>>(partial, d_beta, B, H, P, dk);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_alu_fwd_gated(const SeqArgs &a, const float *beta)
 {
     if ((long long)a.B * a.H == 0 || a.N == 0) return cudaSuccess;
