@@ -2,7 +2,8 @@
 
 Tensors are ``torch`` CUDA tensors used purely as device memory; every step of the
 recurrence runs inside ``libhgrn2.so``.  There is no CPU or eager fallback: if the library
-is missing or fails to load, importing this module's functions raises.
+is missing or fails to load, importing this module's functions raises.  The calls of a training step and of a decode
+loop marshal their arguments in C++ (``native/marshal.cpp``), the rest through ctypes.
 """
 from __future__ import annotations
 
@@ -110,6 +111,24 @@ def load() -> ctypes.CDLL:
     return lib
 
 
+_marshal = None
+
+
+def _calls():
+    """The C++ marshalling module (built in-tree next to the library); raises if it is absent."""
+    global _marshal
+    if _marshal is None:
+        load()
+        from . import _marshal as m
+        m.setup(Desc, Hgrn2Error)
+        _marshal = m
+    return _marshal
+
+
+def _handle(stream: Optional[torch.cuda.Stream]):
+    return None if stream is None else stream.cuda_stream
+
+
 def status_string(code: int) -> str:
     return load().hgrn2_status_string(int(code)).decode()
 
@@ -177,91 +196,30 @@ def hgrn2_fwd(o, f, i, S0=None, *, y=None, SN=None, saved=None, ws=None, want_fi
               save_for_backward=True, chunk=0, flags=0, stream=None):
     """Forward over [B, H, N, d] tensors.  Returns (y, SN, saved, ws, desc); buffers that are not passed in
     are allocated with torch (device memory only)."""
-    B, H, N, dk = o.shape
-    dv = i.shape[-1]
-    desc = make_desc(B, H, N, dk, dv, _io_code(o), chunk, flags)
-    dev = o.device
-    if y is None:
-        y = torch.empty((B, H, N, dv), dtype=o.dtype, device=dev)
-    if SN is None and want_final_state:
-        SN = torch.empty((B, H, dk, dv), dtype=torch.float32, device=dev)
-    if saved is None and save_for_backward:
-        saved = alloc_saved(desc, dev)
-    if ws is None:
-        ws = alloc_workspace(desc, dev)
-    code = load().hgrn2_fwd(ctypes.byref(desc), _ptr(o), _ptr(f), _ptr(i), _ptr(S0), _ptr(y), _ptr(SN),
-                            _ptr(saved), _ptr(ws), _stream(stream))
-    _check(code, "hgrn2_fwd")
-    return y, SN, saved, ws, desc
+    return _calls().fwd(0, o, f, i, None, S0, y, SN, saved, ws, want_final_state, save_for_backward, chunk, flags,
+                        _handle(stream))
 
 
 def hgrn2_bwd(o, f, i, S0, dy, dSN=None, saved=None, *, d_o=None, d_f=None, d_i=None, dS0=None, ws=None,
               want_dS0=True, chunk=0, flags=0, stream=None):
     """Backward of hgrn2_fwd.  Returns (d_o, d_f, d_i, dS0, ws)."""
-    B, H, N, dk = o.shape
-    dv = i.shape[-1]
-    desc = make_desc(B, H, N, dk, dv, _io_code(o), chunk, flags)
-    dev = o.device
-    d_o = torch.empty_like(o) if d_o is None else d_o
-    d_f = torch.empty_like(f) if d_f is None else d_f
-    d_i = torch.empty_like(i) if d_i is None else d_i
-    if dS0 is None and want_dS0:
-        dS0 = torch.empty((B, H, dk, dv), dtype=torch.float32, device=dev)
-    if ws is None:
-        ws = alloc_workspace(desc, dev)
-    code = load().hgrn2_bwd(ctypes.byref(desc), _ptr(o), _ptr(f), _ptr(i), _ptr(S0), _ptr(dy), _ptr(dSN),
-                            _ptr(saved), _ptr(d_o), _ptr(d_f), _ptr(d_i), _ptr(dS0), _ptr(ws), _stream(stream))
-    _check(code, "hgrn2_bwd")
-    return d_o, d_f, d_i, dS0, ws
+    return _calls().bwd(0, o, f, i, None, S0, dy, dSN, saved, d_o, d_f, d_i, None, dS0, ws, want_dS0, False, chunk, flags,
+                        _handle(stream))
 
 
 def hgrn2_fwd_varlen(o, f, i, cu_seqlens, S0=None, *, y=None, SN=None, saved=None, ws=None, want_final_state=True,
                      save_for_backward=True, chunk=0, flags=0, stream=None):
     """Forward over a packed batch: o, f [H, T, dk], i [H, T, dv]; cu_seqlens int32 [B + 1] on the device; states
     [B, H, dk, dv].  Returns (y, SN, saved, ws, desc)."""
-    H, T, dk = o.shape
-    dv = i.shape[-1]
-    B = cu_seqlens.numel() - 1
-    if cu_seqlens.dtype != torch.int32:
-        raise TypeError("cu_seqlens must be int32")
-    desc = make_desc(B, H, T, dk, dv, _io_code(o), chunk, flags)
-    dev = o.device
-    if y is None:
-        y = torch.empty((H, T, dv), dtype=o.dtype, device=dev)
-    if SN is None and want_final_state:
-        SN = torch.empty((B, H, dk, dv), dtype=torch.float32, device=dev)
-    lib = load()
-    if saved is None and save_for_backward:
-        saved = torch.empty(max(int(lib.hgrn2_saved_bytes_varlen(ctypes.byref(desc))), 16), dtype=torch.uint8, device=dev)
-    if ws is None:
-        ws = torch.empty(int(lib.hgrn2_workspace_bytes_varlen(ctypes.byref(desc))), dtype=torch.uint8, device=dev)
-    code = lib.hgrn2_fwd_varlen(ctypes.byref(desc), _ptr(o), _ptr(f), _ptr(i), _ptr(cu_seqlens), _ptr(S0), _ptr(y),
-                                _ptr(SN), _ptr(saved), _ptr(ws), _stream(stream))
-    _check(code, "hgrn2_fwd_varlen")
-    return y, SN, saved, ws, desc
+    return _calls().fwd(1, o, f, i, cu_seqlens, S0, y, SN, saved, ws, want_final_state, save_for_backward, chunk, flags,
+                        _handle(stream))
 
 
 def hgrn2_bwd_varlen(o, f, i, cu_seqlens, S0, dy, dSN=None, saved=None, *, d_o=None, d_f=None, d_i=None, dS0=None,
                      ws=None, want_dS0=True, chunk=0, flags=0, stream=None):
     """Backward of hgrn2_fwd_varlen.  Returns (d_o, d_f, d_i, dS0, ws)."""
-    H, T, dk = o.shape
-    dv = i.shape[-1]
-    B = cu_seqlens.numel() - 1
-    desc = make_desc(B, H, T, dk, dv, _io_code(o), chunk, flags)
-    dev = o.device
-    d_o = torch.empty_like(o) if d_o is None else d_o
-    d_f = torch.empty_like(f) if d_f is None else d_f
-    d_i = torch.empty_like(i) if d_i is None else d_i
-    if dS0 is None and want_dS0:
-        dS0 = torch.empty((B, H, dk, dv), dtype=torch.float32, device=dev)
-    lib = load()
-    if ws is None:
-        ws = torch.empty(int(lib.hgrn2_workspace_bytes_varlen(ctypes.byref(desc))), dtype=torch.uint8, device=dev)
-    code = lib.hgrn2_bwd_varlen(ctypes.byref(desc), _ptr(o), _ptr(f), _ptr(i), _ptr(cu_seqlens), _ptr(S0), _ptr(dy),
-                                _ptr(dSN), _ptr(saved), _ptr(d_o), _ptr(d_f), _ptr(d_i), _ptr(dS0), _ptr(ws),
-                                _stream(stream))
-    _check(code, "hgrn2_bwd_varlen")
-    return d_o, d_f, d_i, dS0, ws
+    return _calls().bwd(1, o, f, i, cu_seqlens, S0, dy, dSN, saved, d_o, d_f, d_i, None, dS0, ws, want_dS0, False, chunk,
+                        flags, _handle(stream))
 
 
 def span_summary_fwd(f, i, *, ws=None, chunk=0, flags=0, stream=None):
@@ -305,47 +263,15 @@ def hgrn2_fwd_gated(zo, zf, zi, beta, S0=None, *, y=None, SN=None, saved=None, w
                     save_for_backward=True, chunk=0, flags=0, stream=None):
     """Forward from the pre-activations: o = sigmoid(zo), f = beta + (1 - beta) sigmoid(zf), i = silu(zi), then the
     recurrence.  zo, zf [B, H, N, dk], zi [B, H, N, dv], beta [H, dk] float32.  Returns (y, SN, saved, ws, desc)."""
-    B, H, N, dk = zo.shape
-    dv = zi.shape[-1]
-    desc = make_desc(B, H, N, dk, dv, _io_code(zo), chunk, flags)
-    dev = zo.device
-    lib = load()
-    if y is None:
-        y = torch.empty((B, H, N, dv), dtype=zo.dtype, device=dev)
-    if SN is None and want_final_state:
-        SN = torch.empty((B, H, dk, dv), dtype=torch.float32, device=dev)
-    if saved is None and save_for_backward:
-        saved = torch.empty(max(int(lib.hgrn2_saved_bytes_gated(ctypes.byref(desc))), 16), dtype=torch.uint8, device=dev)
-    if ws is None:
-        ws = torch.empty(int(lib.hgrn2_workspace_bytes_gated(ctypes.byref(desc))), dtype=torch.uint8, device=dev)
-    code = lib.hgrn2_fwd_gated(ctypes.byref(desc), _ptr(zo), _ptr(zf), _ptr(zi), _ptr(beta), _ptr(S0), _ptr(y), _ptr(SN),
-                               _ptr(saved), _ptr(ws), _stream(stream))
-    _check(code, "hgrn2_fwd_gated")
-    return y, SN, saved, ws, desc
+    return _calls().fwd(2, zo, zf, zi, beta, S0, y, SN, saved, ws, want_final_state, save_for_backward, chunk, flags,
+                        _handle(stream))
 
 
 def hgrn2_bwd_gated(zo, zf, zi, beta, S0, dy, dSN=None, saved=None, *, d_zo=None, d_zf=None, d_zi=None, d_beta=None,
                     dS0=None, ws=None, want_dS0=True, want_d_beta=True, chunk=0, flags=0, stream=None):
     """Backward of hgrn2_fwd_gated.  Returns (d_zo, d_zf, d_zi, d_beta, dS0, ws)."""
-    B, H, N, dk = zo.shape
-    dv = zi.shape[-1]
-    desc = make_desc(B, H, N, dk, dv, _io_code(zo), chunk, flags)
-    dev = zo.device
-    lib = load()
-    d_zo = torch.empty_like(zo) if d_zo is None else d_zo
-    d_zf = torch.empty_like(zf) if d_zf is None else d_zf
-    d_zi = torch.empty_like(zi) if d_zi is None else d_zi
-    if d_beta is None and want_d_beta:
-        d_beta = torch.empty((H, dk), dtype=torch.float32, device=dev)
-    if dS0 is None and want_dS0:
-        dS0 = torch.empty((B, H, dk, dv), dtype=torch.float32, device=dev)
-    if ws is None:
-        ws = torch.empty(int(lib.hgrn2_workspace_bytes_gated(ctypes.byref(desc))), dtype=torch.uint8, device=dev)
-    code = lib.hgrn2_bwd_gated(ctypes.byref(desc), _ptr(zo), _ptr(zf), _ptr(zi), _ptr(beta), _ptr(S0), _ptr(dy),
-                               _ptr(dSN), _ptr(saved), _ptr(d_zo), _ptr(d_zf), _ptr(d_zi), _ptr(d_beta), _ptr(dS0),
-                               _ptr(ws), _stream(stream))
-    _check(code, "hgrn2_bwd_gated")
-    return d_zo, d_zf, d_zi, d_beta, dS0, ws
+    return _calls().bwd(2, zo, zf, zi, beta, S0, dy, dSN, saved, d_zo, d_zf, d_zi, d_beta, dS0, ws, want_dS0,
+                        want_d_beta, chunk, flags, _handle(stream))
 
 
 def hgrn2_bwd_static_scratch(o, f, i, S0, dy, dSN, d_o, d_f, d_i, dS0=None, status_out=None, *, chunk=0, flags=0,
@@ -366,27 +292,13 @@ def hgrn2_bwd_static_scratch(o, f, i, S0, dy, dSN, d_o, d_f, d_i, dS0=None, stat
 
 def hgrn2_step(o, f, i, S, *, y=None, stream=None):
     """One decode step on [B, H, d] gates; S [B, H, dk, dv] float32 is updated in place.  Returns y."""
-    B, H, dk = o.shape
-    dv = i.shape[-1]
-    desc = make_desc(B, H, 1, dk, dv, _io_code(o))
-    if y is None:
-        y = torch.empty((B, H, dv), dtype=o.dtype, device=o.device)
-    code = load().hgrn2_step(ctypes.byref(desc), _ptr(o), _ptr(f), _ptr(i), _ptr(S), _ptr(y), _stream(stream))
-    _check(code, "hgrn2_step")
-    return y
+    return _calls().step(o, f, i, S, y, _handle(stream), False)
 
 
 def hgrn2_step_multi(o, f, i, S, *, y=None, stream=None):
     """T successive decode steps in one launch on [B, H, T, d] gates; S [B, H, dk, dv] float32 is updated in
     place to the state after the last token.  Returns y [B, H, T, dv]."""
-    B, H, T, dk = o.shape
-    dv = i.shape[-1]
-    desc = make_desc(B, H, T, dk, dv, _io_code(o))
-    if y is None:
-        y = torch.empty((B, H, T, dv), dtype=o.dtype, device=o.device)
-    code = load().hgrn2_step_multi(ctypes.byref(desc), _ptr(o), _ptr(f), _ptr(i), _ptr(S), _ptr(y), _stream(stream))
-    _check(code, "hgrn2_step_multi")
-    return y
+    return _calls().step(o, f, i, S, y, _handle(stream), True)
 
 
 def exact_path_units(ws: torch.Tensor) -> int:
