@@ -77,18 +77,6 @@ __device__ __forceinline__ Where packed_where(const Args &a, int b, long long h)
     return Where{h * a.N + start, n, (n + kL - 1) / kL, (h - a.g0) * a.spp + start / kL + b, b * (long long)a.H + h};
 }
 
-template <typename T> __device__ __forceinline__ void load4(const T *p, float (&x)[4]);
-template <> __device__ __forceinline__ void load4<float>(const float *p, float (&x)[4])
-{
-    const float4 v = *reinterpret_cast<const float4 *>(p);
-    x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-}
-template <> __device__ __forceinline__ void load4<__nv_bfloat16>(const __nv_bfloat16 *p, float (&x)[4])
-{
-    const uint2 v = *reinterpret_cast<const uint2 *>(p);
-    x[0] = __uint_as_float(v.x << 16); x[1] = __uint_as_float(v.x & 0xFFFF0000u);
-    x[2] = __uint_as_float(v.y << 16); x[3] = __uint_as_float(v.y & 0xFFFF0000u);
-}
 template <typename T> __device__ __forceinline__ void store4(T *p, float a, float b, float c, float d);
 template <> __device__ __forceinline__ void store4<float>(float *p, float a, float b, float c, float d)
 {

@@ -36,6 +36,20 @@ template <> __device__ __forceinline__ float load_f<__nv_bfloat16>(const __nv_bf
     return __bfloat162float(*p);
 }
 
+// four consecutive elements, aligned to their own size
+template <typename T> __device__ __forceinline__ void load4(const T *p, float (&x)[4]);
+template <> __device__ __forceinline__ void load4<float>(const float *p, float (&x)[4])
+{
+    const float4 v = *reinterpret_cast<const float4 *>(p);
+    x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+}
+template <> __device__ __forceinline__ void load4<__nv_bfloat16>(const __nv_bfloat16 *p, float (&x)[4])
+{
+    const uint2 v = *reinterpret_cast<const uint2 *>(p);
+    x[0] = __uint_as_float(v.x << 16); x[1] = __uint_as_float(v.x & 0xFFFF0000u);
+    x[2] = __uint_as_float(v.y << 16); x[3] = __uint_as_float(v.y & 0xFFFF0000u);
+}
+
 template <typename T> __device__ __forceinline__ void store_f(T *p, float x);
 template <> __device__ __forceinline__ void store_f<float>(float *p, float x) { *p = x; }
 template <> __device__ __forceinline__ void store_f<__nv_bfloat16>(__nv_bfloat16 *p, float x)
@@ -138,6 +152,7 @@ struct SegPlan {
     uint64_t tail_units;   // units [main_units, main_units + tail_units) are split into G segments each
     int G;
 };
+int         sm_count();        // SMs of the current device (0: no device)
 SegPlan     tc_seg_plan(uint64_t U, int N, int NC);
 // Sequences that are NOT whole chunks, few or left-over units (as SegPlan): those units' sequences are cut into G
 // segments of Lc chunks (the last one shorter), which run through the packed-batch geometry (per-CTA rows from an
