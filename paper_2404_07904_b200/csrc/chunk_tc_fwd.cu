@@ -20,6 +20,8 @@
 // Tensor-memory plan (512 columns): S' at [0,128) (lane = key dim, column = value dim); Y, double
 // buffered, at [128,384) and A, double buffered, at [384,512) in the M = 64 accumulator layout
 // (row r -> lane 32 * (r / 16) + r % 16).
+#include <atomic>
+
 #include "chunk_alu.cuh"
 #include "tc_chunk.cuh"
 
@@ -629,11 +631,15 @@ __global__ void seg_combine_kernel(const float *__restrict__ S0, const float *__
     if (SN) SN[e] = S;
 }
 
+// Asked for several times per call (plans and sizes), so kept per device.
 int sm_count()
 {
+    static std::atomic<int> known[64];
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev >= 0 && dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (dev >= 0 && dev < 64) known[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
