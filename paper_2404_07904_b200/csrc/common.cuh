@@ -36,6 +36,23 @@ template <> __device__ __forceinline__ float load_f<__nv_bfloat16>(const __nv_bf
     return __bfloat162float(*p);
 }
 
+// Packed fp32 arithmetic (sm_100): one instruction per two results, each rounded exactly like the scalar op.
+__device__ __forceinline__ float2 mul_x2(float2 a, float2 b)
+{
+    float2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<unsigned long long &>(a)), "l"(reinterpret_cast<unsigned long long &>(b)));
+    return d;
+}
+__device__ __forceinline__ float2 fma_x2(float2 a, float2 b, float2 c)
+{
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<unsigned long long &>(a)), "l"(reinterpret_cast<unsigned long long &>(b)),
+          "l"(reinterpret_cast<unsigned long long &>(c)));
+    return d;
+}
+
 // four consecutive elements, aligned to their own size
 template <typename T> __device__ __forceinline__ void load4(const T *p, float (&x)[4]);
 template <> __device__ __forceinline__ void load4<float>(const float *p, float (&x)[4])

@@ -108,24 +108,6 @@ step_kernel(const T *__restrict__ o, const T *__restrict__ f, const T *__restric
     }
 }
 
-// Packed fp32 arithmetic (sm_100): one instruction per two results, each rounded exactly like the scalar op,
-// so the results below stay bit-identical to step_kernel's.
-__device__ __forceinline__ float2 mul_x2(float2 a, float2 b)
-{
-    float2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(reinterpret_cast<unsigned long long &>(d))
-        : "l"(reinterpret_cast<unsigned long long &>(a)), "l"(reinterpret_cast<unsigned long long &>(b)));
-    return d;
-}
-__device__ __forceinline__ float2 fma_x2(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(reinterpret_cast<unsigned long long &>(d))
-        : "l"(reinterpret_cast<unsigned long long &>(a)), "l"(reinterpret_cast<unsigned long long &>(b)),
-          "l"(reinterpret_cast<unsigned long long &>(c)));
-    return d;
-}
-
 // Several successive tokens in one launch (multi-token / speculative decode): a unit's state is read once, kept in
 // registers while Eq. 3 is applied Tn times, and written once, so the state traffic per token falls Tn-fold.
 // d_k = d_v = D.  Row order, arithmetic and summation order are those of step_kernel, so the results are
