@@ -119,13 +119,15 @@ static_assert(alu::bwd_smem_floats(kD, kD, kExactC) * sizeof(float) <= kSmemByte
 // walked outwards from the middle of the chunk in blocks of four rows (a short loop body: the role shares its
 // scheduler's instruction stream with four others).  Returns this half's sums of a and e.
 // do_g points at element (row 0 of the chunk, column k) of d_o in global memory.  oraw, fraw: the chunk's raw
-// o and f as plain [64][128] bf16 tiles (rows beyond the end of the sequence hold zeros, or in a packed batch
-// the next sequence's tokens: they are patched to the neutral f = 1, o = 0).  Qs and Ks are recomputed from
-// them with the transform's own roundings, so the operand stage does not have to be held until the outputs
+// o and f as plain [64][128] bf16 tiles (rows beyond the end of the sequence hold the neutral f = 1, o = 0).
+// Qs and Ks are recomputed from them with the transform's own roundings, so the operand stage does not have to be held until the outputs
 // are done.  The role is bound by its instruction count: per element one reciprocal (1/f is the ratio of two
-// consecutive products), fused packed multiply-adds, and a single running sum.
-template <bool kUp, bool kRagged, bool kEnc>
-__device__ __forceinline__ void phase_main(uint32_t tmem_lane, const __nv_bfloat16 *oraw, const __nv_bfloat16 *fraw,
+// consecutive products), fused packed multiply-adds, and a single running sum.  kPartial: a sequence's last, partial
+// chunk.  Such chunks have an instance of their own, and so have their d_f and d_i below: a test per row, or per block
+// of rows, on the stores of every chunk made the ragged backward 5 to 11 % slower than the other (160 us instead of
+// 142 for 128 units of 2047 and 2048 tokens; 146 now).
+template <bool kUp, bool kPartial, bool kEnc>
+__device__ __forceinline__ void phase_main(uint32_t tmem_lane, const unsigned short *oraw, const unsigned short *fraw,
                                            int k, __nv_bfloat16 *do_g, int n_valid, float &asum, float &esum)
 {
     float cp = 1.f, ci = 1.f;       // running product of f between the middle and the current row, and its reciprocal
@@ -143,9 +145,8 @@ __device__ __forceinline__ void phase_main(uint32_t tmem_lane, const __nv_bfloat
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int t = t0 + j;
-            fw[j] = reinterpret_cast<const unsigned short *>(fraw)[t * kD + k];
-            qw[j] = reinterpret_cast<const unsigned short *>(oraw)[t * kD + k];
-            if (kRagged && t >= n_valid) { fw[j] = kEnc ? 0x8000u : 0x3F80u; qw[j] = 0u; }
+            fw[j] = fraw[t * kD + k];
+            qw[j] = oraw[t * kD + k];
             if (kEnc) {                       // fw[j] becomes the bf16 bits of k, as the transform formed them
                 float kv;
                 gate_decode(fw[j], fv[j], kv);
@@ -190,8 +191,8 @@ __device__ __forceinline__ void phase_main(uint32_t tmem_lane, const __nv_bfloat
             const float2 w2 = fma2(KSn, Z, a2);                 // a - e
             Gp = add2(Gp, a2);
             const float2 dk2 = mul2(add2(Y, Z), make_float2(sk[j], sk[j + 1]));
-            if (!kRagged || t0 + j < n_valid) do_g[(size_t)(t0 + j) * kD] = __float2bfloat16_rn(dox.x);
-            if (!kRagged || t0 + j + 1 < n_valid) do_g[(size_t)(t0 + j + 1) * kD] = __float2bfloat16_rn(dox.y);
+            if (!kPartial || t0 + j < n_valid) do_g[(size_t)(t0 + j) * kD] = __float2bfloat16_rn(dox.x);
+            if (!kPartial || t0 + j + 1 < n_valid) do_g[(size_t)(t0 + j + 1) * kD] = __float2bfloat16_rn(dox.y);
             w[j] = w2.x; w[j + 1] = w2.y;
             dk[j] = dk2.x; dk[j + 1] = dk2.y;
         }
@@ -248,8 +249,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     uint8_t *dsbuf = smem + kOffDS;
     uint8_t *pbuf = smem + kOffP;
     uint8_t *dpbuf = smem + kOffDP;
-    const __nv_bfloat16 *oraw = reinterpret_cast<const __nv_bfloat16 *>(smem + kOffRawO);
-    const __nv_bfloat16 *fraw = reinterpret_cast<const __nv_bfloat16 *>(smem + kOffRawF);
+    unsigned short *oraw = reinterpret_cast<unsigned short *>(smem + kOffRawO);          // bf16 bits
+    unsigned short *fraw = reinterpret_cast<unsigned short *>(smem + kOffRawF);
     uint8_t *vbuf = smem + kOffV;
     float *rr = reinterpret_cast<float *>(smem + kOffR);
     float *xa = reinterpret_cast<float *>(smem + kOffX);
@@ -350,11 +351,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
             PT_STAMP(status, 1, tid == 0 && it == 16) PT_STAMP(status, 20, tid == 0 && it == 18)
             const int n_valid = kRagged ? N - c * kC : kC;
             // Pm and E of the chunk are not kept: the backward takes them from what the forward saved
-            if (n_valid >= kC) {
-                transform_stream<true, kEnc, kSS, kSlab>(qbuf + kOffQ, qbuf + kOffK, nullptr, nullptr, nullptr, nullptr, kC, tid);
-            } else {
-                transform_stream<false, kEnc, kSS, kSlab>(qbuf + kOffQ, qbuf + kOffK, nullptr, nullptr, nullptr, nullptr, n_valid, tid);
-            }
+            if (kRagged && n_valid < kC) neutral_rows<kEnc, kSS, kSlab>(qbuf + kOffQ, qbuf + kOffK, n_valid, tid);
+            transform_stream<kEnc, kSS, kSlab>(qbuf + kOffQ, qbuf + kOffK, nullptr, nullptr, nullptr, nullptr, tid);
             fence_proxy_async_smem();
             mbar_arrive(&ctl->t_done[s]);
             PT_MARK(1)
@@ -484,8 +482,21 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
             tc_fence_after_sync();
             float asum, esum;
             PT_STAMP(status, 14, tid == kWarpE3 * 32 && it == 16)
-            if (half) phase_main<true, kRagged, kEnc>(tl, oraw, fraw, krow, d_o + crow0 * kD + krow, n_valid, asum, esum);
-            else      phase_main<false, kRagged, kEnc>(tl, oraw, fraw, krow, d_o + crow0 * kD + krow, n_valid, asum, esum);
+            __nv_bfloat16 *do_g = d_o + crow0 * kD + krow;
+            if (kRagged && n_valid < kC) {
+                // rows beyond the end: see neutral_rows (this thread's column of its half)
+#pragma unroll 1
+                for (int r = max(n_valid, 32 * half); r < 32 * half + 32; ++r) {
+                    oraw[r * kD + krow] = 0u;
+                    fraw[r * kD + krow] = kEnc ? 0x8000u : 0x3F80u;
+                }
+                if (half) phase_main<true, true, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
+                else      phase_main<false, true, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
+                fence_proxy_async_smem();                        // the rows written here, before the tiles' next load
+            } else {
+                if (half) phase_main<true, false, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
+                else      phase_main<false, false, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
+            }
             mbar_arrive(&ctl->raw_read);
             if (half) xa[krow] = asum; else xe[krow] = esum;
             tmem_wait_st();
@@ -505,15 +516,29 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                 const float K = rr[(it & 1) * 128 + krow] + xa[krow] + xe[krow];
                 __nv_bfloat16 *df_g = d_f + crow0 * kD + krow;
                 // the thread's 64 parked values in two reads (the pass is on the chunk's critical chain)
-                uint32_t uu[32], rf[32];
-                tmem_ld32(tl + kColDQ + 32 * half, uu);
-                tmem_ld32(tl + kColDKi + 32 * half, rf);
-                tmem_wait_ld();
+                if (!kRagged || n_valid == kC) {
+                    uint32_t uu[32], rf[32];
+                    tmem_ld32(tl + kColDQ + 32 * half, uu);
+                    tmem_ld32(tl + kColDKi + 32 * half, rf);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (!kRagged || 32 * half + j < n_valid)
+                    for (int j = 0; j < 32; ++j)
                         df_g[(size_t)(32 * half + j) * kD] =
                             __float2bfloat16_rn(fmaf(K, __uint_as_float(rf[j]), __uint_as_float(uu[j])));
+                } else {
+#pragma unroll 1
+                    for (int t0 = 32 * half; t0 < 32 * half + 32; t0 += 4) {
+                        uint32_t uu[4], rf[4];
+                        tmem_ld4(tl + kColDQ + t0, uu);
+                        tmem_ld4(tl + kColDKi + t0, rf);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (t0 + j < n_valid)
+                                df_g[(size_t)(t0 + j) * kD] =
+                                    __float2bfloat16_rn(fmaf(K, __uint_as_float(rf[j]), __uint_as_float(uu[j])));
+                    }
+                }
             }
             tc_fence_before_sync();
             mbar_arrive(&ctl->acc_free2);
@@ -544,15 +569,26 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
             PT_STAMP(status, 16, tid == kWarpO * 32 && it == 16)
             tc_fence_after_sync();
             // d_i = dV: lane = value dimension, columns = local times
+            __nv_bfloat16 *di_g = d_i + crow0 * kD + krow;
+            if (!kRagged || n_valid == kC) {
 #pragma unroll 1
-            for (int b = 0; b < 8; ++b) {
-                uint32_t r[8];
-                tmem_ld8(tl + kColDV + 8 * b, r);
-                tmem_wait_ld();
+                for (int b = 0; b < 8; ++b) {
+                    uint32_t r[8];
+                    tmem_ld8(tl + kColDV + 8 * b, r);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (8 * b + j < n_valid)
-                        d_i[(crow0 + 8 * b + j) * kD + krow] = __float2bfloat16_rn(__uint_as_float(r[j]));
+                    for (int j = 0; j < 8; ++j) di_g[(size_t)(8 * b + j) * kD] = __float2bfloat16_rn(__uint_as_float(r[j]));
+                }
+            } else {
+#pragma unroll 1
+                for (int b = 0; b < 8; ++b) {
+                    uint32_t r[8];
+                    tmem_ld8(tl + kColDV + 8 * b, r);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (8 * b + j < n_valid) di_g[(size_t)(8 * b + j) * kD] = __float2bfloat16_rn(__uint_as_float(r[j]));
+                }
             }
             tc_fence_before_sync();
             mbar_arrive(&ctl->acc_freeV);

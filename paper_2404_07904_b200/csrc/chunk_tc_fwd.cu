@@ -187,13 +187,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
             PT_MARK(0)
             const int n_valid = kRagged ? N - c * kC : kC;
             float *tg = totals ? totals + (slot0 + c) * 2 * kD : nullptr;       // Pm, E of the chunk for the backward
-            if (n_valid >= kC) {
-                transform_stream<true, kEnc>(qbuf, qbuf + kTile, pm + (c & 3) * 128, ee + (c & 3) * 128, tg, tg ? tg + kD : nullptr,
-                                       kC, tt);
-            } else {
-                transform_stream<false, kEnc>(qbuf, qbuf + kTile, pm + (c & 3) * 128, ee + (c & 3) * 128, tg, tg ? tg + kD : nullptr,
-                                        n_valid, tt);
-            }
+            if (kRagged && n_valid < kC) neutral_rows<kEnc>(qbuf, qbuf + kTile, n_valid, tt);
+            transform_stream<kEnc>(qbuf, qbuf + kTile, pm + (c & 3) * 128, ee + (c & 3) * 128, tg, tg ? tg + kD : nullptr, tt);
             fence_proxy_async_smem();
             mbar_arrive(&ctl->t_done[s]);
             PT_MARK(1)

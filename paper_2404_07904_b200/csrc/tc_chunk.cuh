@@ -95,13 +95,11 @@ __device__ __forceinline__ uint4 pack8(const uint32_t *r)
 // current one (the tiles are rewritten in place, so the compiler would otherwise serialise every
 // load behind the previous row's stores).  Pm (product over rows 0..31) and E (product over rows
 // 32..63) of the chunk are left in pm[128] and ee[128] (shared memory) and / or pm_g[128], ee_g[128]
-// (global memory); either pair may be null.  Rows at or beyond n_valid are the neutral token
-// f = 1, o = 0.  kEnc: the gate tile holds the SMALLER of f and k = 1 - f, with the sign bit set when it is k
+// (global memory); either pair may be null.  kEnc: the gate tile holds the SMALLER of f and k = 1 - f, with the sign bit set when it is k
 // (gate_decode below).  The gated entry points hand the kernels that: bf16 then resolves the gate to 2^-9 of
 // min(f, 1 - f) at both ends of [0, 1], whereas a bf16 f close to 1 would distort every decay product.
-template <bool kFull, bool kUp, uint32_t kQSlabStride, uint32_t kFSlabStride, bool kEnc>
-__device__ __forceinline__ void transform_half(uint8_t *qbuf, uint8_t *fbuf, float *tot, float *tot_g, int n_valid,
-                                               int p)
+template <bool kUp, uint32_t kQSlabStride, uint32_t kFSlabStride, bool kEnc>
+__device__ __forceinline__ void transform_half(uint8_t *qbuf, uint8_t *fbuf, float *tot, float *tot_g, int p)
 {
     const int col = 2 * p;
     const int jch = (col & 63) >> 3;
@@ -137,7 +135,6 @@ __device__ __forceinline__ void transform_half(uint8_t *qbuf, uint8_t *fbuf, flo
         for (int j = 0; j < 8; ++j) {
             const int r = row_of(8 * b + j);
             const uint32_t off = xo[r & 7] + r * 128;
-            if (!kFull && r >= n_valid) { fw[j] = kEnc ? 0x80008000u : 0x3F803F80u; qw[j] = 0u; }
             float f0, f1, k0 = 0.f, k1 = 0.f;
             if (kEnc) {
                 gate_decode(fw[j], f0, k0);
@@ -166,12 +163,26 @@ __device__ __forceinline__ void transform_half(uint8_t *qbuf, uint8_t *fbuf, flo
 }
 
 // kQSlabStride, kFSlabStride: distance in bytes between the two 64-column slabs of the q tile and of the f tile.
-template <bool kFull, bool kEnc, uint32_t kQSlabStride = kSlab, uint32_t kFSlabStride = kSlab>
+template <bool kEnc, uint32_t kQSlabStride = kSlab, uint32_t kFSlabStride = kSlab>
 __device__ __forceinline__ void transform_stream(uint8_t *qbuf, uint8_t *fbuf, float *pm, float *ee, float *pm_g,
-                                                 float *ee_g, int n_valid, int tid)
+                                                 float *ee_g, int tid)
 {
-    if (tid >> 6) transform_half<kFull, true, kQSlabStride, kFSlabStride, kEnc>(qbuf, fbuf, ee, ee_g, n_valid, tid & 63);
-    else          transform_half<kFull, false, kQSlabStride, kFSlabStride, kEnc>(qbuf, fbuf, pm, pm_g, n_valid, tid & 63);
+    if (tid >> 6) transform_half<true, kQSlabStride, kFSlabStride, kEnc>(qbuf, fbuf, ee, ee_g, tid & 63);
+    else          transform_half<false, kQSlabStride, kFSlabStride, kEnc>(qbuf, fbuf, pm, pm_g, tid & 63);
+}
+
+// A partial chunk: the rows at or beyond n_valid (zeros, or in a packed batch the next sequence's tokens) become the
+// neutral token f = 1, o = 0, each thread in what it is about to transform.  Done in the tiles and not in the transform's
+// registers, which would cost two selects per row pair of every chunk or a second copy of its code.
+template <bool kEnc, uint32_t kQSlabStride = kSlab, uint32_t kFSlabStride = kSlab>
+__device__ __noinline__ void neutral_rows(uint8_t *qbuf, uint8_t *fbuf, int n_valid, int tid)
+{
+    const int col = 2 * (tid & 63), slab = col >> 6, lo = 32 * (tid >> 6);
+    for (int r = max(n_valid, lo); r < lo + 32; ++r) {
+        const uint32_t off = (((((col & 63) >> 3) ^ (r & 7)) << 4)) + (col & 7) * 2 + r * 128;
+        *reinterpret_cast<uint32_t *>(fbuf + slab * kFSlabStride + off) = kEnc ? 0x80008000u : 0x3F803F80u;
+        *reinterpret_cast<uint32_t *>(qbuf + slab * kQSlabStride + off) = 0u;
+    }
 }
 
 // Causal mask + bf16 of 32 columns (32 * half ...) of one 64 x 64 fp32 accumulator in the M = 64
