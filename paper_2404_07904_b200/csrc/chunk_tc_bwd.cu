@@ -258,7 +258,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     Ctl *ctl = reinterpret_cast<Ctl *>(smem + kOffCtl);
     volatile int *abort_flag = &ctl->abort_flag;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int u = blockIdx.x;
     // This CTA's sequence: rows [row0, row0 + N) of plane zu of the [planes][rows][128] tensors, NC chunks, chunk-start
     // state c in slot slot0 + c.  Packed batches (ragged instantiations only) read theirs from the offsets array.
@@ -598,71 +598,69 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         PT_DUMP(status, 11, 4, tid == kWarpO * 32)
     } else if (warp == kWarpLoad) {
         // ================= L: TMA loads =================
-        if (lane == 0) {
-            int n_stage = 0, n_v = 0, n_state = 0, n_raw = 0;       // fills asked for so far, per buffer
-            auto issue_stage = [&](int it) {
-                n_stage = it + 1;
-                const int s = it % kStages, c = NC - 1 - it;
-                uint8_t *st = smem + s * kStageBytes;
-                mbar_arrive_expect_tx(&ctl->full[s], kStageBytes);
-                for (int b = 0; b < 2; ++b) {
-                    tma_load_3d(st + kOffQ + b * kSS, &map_o, &ctl->full[s], 64 * b, row0 + c * kC, zu);
-                    tma_load_3d(st + kOffK + b * kSlab, &map_f, &ctl->full[s], 64 * b, row0 + c * kC, zu);
-                }
-                for (int b = 0; b < 2; ++b)
-                    tma_load_3d(st + kOffG + b * kSS, &map_dy, &ctl->full[s], 64 * b, row0 + c * kC, zu);
-            };
-            auto issue_v = [&](int it) {
-                n_v = it + 1;
-                const int c = NC - 1 - it;
-                mbar_arrive_expect_tx(&ctl->vfull, kTile);
-                for (int b = 0; b < 2; ++b) tma_load_3d(vbuf + b * kSlab, &map_i, &ctl->vfull, 64 * b, row0 + c * kC, zu);
-            };
-            auto issue_raw = [&](int it) {
-                n_raw = it + 1;
-                const int c = NC - 1 - it;
-                mbar_arrive_expect_tx(&ctl->rawfull, 2 * kTile);
-                tma_load_3d(smem + kOffRawO, &map_o_raw, &ctl->rawfull, 0, row0 + c * kC, zu);
-                tma_load_3d(smem + kOffRawF, &map_f_raw, &ctl->rawfull, 0, row0 + c * kC, zu);
-            };
-            auto issue_state = [&](int it) {
-                n_state = it + 1;
-                const int c = NC - 1 - it;
-                mbar_arrive_expect_tx(&ctl->sfull, kStateTile);
-                for (int b = 0; b < 2; ++b)
-                    tma_load_3d(sbuf + b * kStateSlab, &map_saved, &ctl->sfull, 64 * b, 0, (int)(slot0 + c));
-            };
-            issue_stage(0);
-            issue_v(0);
-            issue_state(0);
-            issue_raw(0);
-            if (NC > 1) issue_stage(1);
-            // Every buffer is refilled as soon as its last reader of chunk `it` is done; the waits below are in
-            // the order in which those readers finish.
-            // A barrier must never be armed twice within one phase.  Normally a buffer's previous fill has long been
-            // consumed when its readers report; on the time-out exit those waits return at once, so before every
-            // refill the previous fill is waited for explicitly (one poll that succeeds at once in normal running).
-            for (int it = 0; it + 1 < NC; ++it) {
-                mbar_wait(&ctl->barX, it & 1, abort_flag);           // dA = dY V^T ...
-                mbar_wait(&ctl->barY1, it & 1, abort_flag);          // ... and dKs_inter^T = dS'' V^T have read v
-                mbar_wait_drain(&ctl->vfull, it & 1, 20000000ull);
-                issue_v(it + 1);
-                mbar_wait(&ctl->r_ready[it & 1], (it >> 1) & 1, abort_flag);   // R has read S' ...
-                mbar_wait(&ctl->barY2, it & 1, abort_flag);          // ... and so have the chunk's products;
-                mbar_wait_drain(&ctl->sfull, it & 1, 20000000ull);
-                issue_state(it + 1);
-                if (it + 2 < NC) {                                   // o, f, dy of the stage are free as well
-                    mbar_wait_drain(&ctl->full[it % kStages], (it / kStages) & 1, 20000000ull);
-                    issue_stage(it + 2);
-                }
-                PT_STAMP(status, 0, it == 14) PT_STAMP(status, 21, it == 16) PT_STAMP(status, 22, it == 15)
-                mbar_wait(&ctl->raw_read, it & 1, abort_flag);       // the output warps are done with raw o, f
-                mbar_wait_drain(&ctl->rawfull, it & 1, 20000000ull);
-                issue_raw(it + 1);
+        int n_stage = 0, n_v = 0, n_state = 0, n_raw = 0;       // fills asked for so far, per buffer
+        auto issue_stage = [&](int it) {
+            n_stage = it + 1;
+            const int s = it % kStages, c = NC - 1 - it;
+            uint8_t *st = smem + s * kStageBytes;
+            mbar_arrive_expect_tx(&ctl->full[s], kStageBytes);
+            for (int b = 0; b < 2; ++b) {
+                tma_load_3d(st + kOffQ + b * kSS, &map_o, &ctl->full[s], 64 * b, row0 + c * kC, zu);
+                tma_load_3d(st + kOffK + b * kSlab, &map_f, &ctl->full[s], 64 * b, row0 + c * kC, zu);
             }
-            ctl->l_stage = n_stage; ctl->l_v = n_v; ctl->l_state = n_state; ctl->l_raw = n_raw;
+            for (int b = 0; b < 2; ++b)
+                tma_load_3d(st + kOffG + b * kSS, &map_dy, &ctl->full[s], 64 * b, row0 + c * kC, zu);
+        };
+        auto issue_v = [&](int it) {
+            n_v = it + 1;
+            const int c = NC - 1 - it;
+            mbar_arrive_expect_tx(&ctl->vfull, kTile);
+            for (int b = 0; b < 2; ++b) tma_load_3d(vbuf + b * kSlab, &map_i, &ctl->vfull, 64 * b, row0 + c * kC, zu);
+        };
+        auto issue_raw = [&](int it) {
+            n_raw = it + 1;
+            const int c = NC - 1 - it;
+            mbar_arrive_expect_tx(&ctl->rawfull, 2 * kTile);
+            tma_load_3d(smem + kOffRawO, &map_o_raw, &ctl->rawfull, 0, row0 + c * kC, zu);
+            tma_load_3d(smem + kOffRawF, &map_f_raw, &ctl->rawfull, 0, row0 + c * kC, zu);
+        };
+        auto issue_state = [&](int it) {
+            n_state = it + 1;
+            const int c = NC - 1 - it;
+            mbar_arrive_expect_tx(&ctl->sfull, kStateTile);
+            for (int b = 0; b < 2; ++b)
+                tma_load_3d(sbuf + b * kStateSlab, &map_saved, &ctl->sfull, 64 * b, 0, (int)(slot0 + c));
+        };
+        issue_stage(0);
+        issue_v(0);
+        issue_state(0);
+        issue_raw(0);
+        if (NC > 1) issue_stage(1);
+        // Every buffer is refilled as soon as its last reader of chunk `it` is done; the waits below are in
+        // the order in which those readers finish.
+        // A barrier must never be armed twice within one phase.  Normally a buffer's previous fill has long been
+        // consumed when its readers report; on the time-out exit those waits return at once, so before every
+        // refill the previous fill is waited for explicitly (one poll that succeeds at once in normal running).
+        for (int it = 0; it + 1 < NC; ++it) {
+            mbar_wait(&ctl->barX, it & 1, abort_flag);           // dA = dY V^T ...
+            mbar_wait(&ctl->barY1, it & 1, abort_flag);          // ... and dKs_inter^T = dS'' V^T have read v
+            mbar_wait_drain(&ctl->vfull, it & 1, 20000000ull);
+            issue_v(it + 1);
+            mbar_wait(&ctl->r_ready[it & 1], (it >> 1) & 1, abort_flag);   // R has read S' ...
+            mbar_wait(&ctl->barY2, it & 1, abort_flag);          // ... and so have the chunk's products;
+            mbar_wait_drain(&ctl->sfull, it & 1, 20000000ull);
+            issue_state(it + 1);
+            if (it + 2 < NC) {                                   // o, f, dy of the stage are free as well
+                mbar_wait_drain(&ctl->full[it % kStages], (it / kStages) & 1, 20000000ull);
+                issue_stage(it + 2);
+            }
+            PT_STAMP(status, 0, it == 14) PT_STAMP(status, 21, it == 16) PT_STAMP(status, 22, it == 15)
+            mbar_wait(&ctl->raw_read, it & 1, abort_flag);       // the output warps are done with raw o, f
+            mbar_wait_drain(&ctl->rawfull, it & 1, 20000000ull);
+            issue_raw(it + 1);
         }
-    } else if (lane == 0) {
+        ctl->l_stage = n_stage; ctl->l_v = n_v; ctl->l_state = n_state; ctl->l_raw = n_raw;
+    } else {
         // ================= MX, MY1, MY2: MMA issue =================
         constexpr uint32_t idDS = idesc_bf16(128, 128, 1, 1);     // Qs^T (MN-major) x dY (MN-major)
         constexpr uint32_t idKK = idesc_bf16(128, 64, 0, 0);      // dS'' x V^T, S' x dY^T (all K-major)

@@ -109,7 +109,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     Ctl *ctl = reinterpret_cast<Ctl *>(smem + kOffCtl);
     volatile int *abort_flag = &ctl->abort_flag;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int u = blockIdx.x;
     // This CTA's sequence: rows [row0, row0 + N) of plane zu of the [planes][rows][128] tensors, NC chunks, chunk-start
     // state c in slot slot0 + c.  Packed batches (ragged instantiations only) read theirs from the offsets array.
@@ -332,96 +332,94 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         }
     } else if (warp == kWarpLoad) {
         // ================= L: TMA loads =================
-        if (lane == 0) {
-            int n_qf = 0, n_v = 0;                                   // chunks whose tiles have been asked for
-            for (int c = 0; c < NC; ++c) {
-                const int s = c % kStages;
-                uint8_t *st = smem + s * kStageBytes;
-                // o and f have barriers of their own in both directions: the transform, which paces the kernel,
-                // needs only them, and their tiles are free as soon as Y = Qs S' of the chunk three back is done,
-                // well before its last product Y += P V has read V
-                // A barrier must never be armed twice within one phase.  Normally the stage's previous fill has long
-                // been consumed when its empty barrier completes; on the time-out exit that wait returns at once, so
-                // the previous fill is waited for explicitly (one poll that succeeds at once in normal running;
-                // stopping this lane on the wait's return value instead cost 8 %).
-                if (c >= kStages) {
-                    mbar_wait(&ctl->emptyqf[s], ((c / kStages) - 1) & 1, abort_flag);
-                    mbar_wait_drain(&ctl->fullqf[s], ((c / kStages) - 1) & 1, 20000000ull);
-                }
-                // the next chunk's o, f tiles are asked into L2 now: their load can be issued only when their stage
-                // frees, one chunk from now, and then finds them there (measured on the fwd + bwd step: -1 %; two
-                // chunks ahead, or including the v tile, gave nothing)
-                if (c + 1 < NC)
-                    for (int b = 0; b < 2; ++b) {
-                        tma_prefetch_3d(&map_o, 64 * b, row0 + (c + 1) * kC, zu);
-                        tma_prefetch_3d(&map_f, 64 * b, row0 + (c + 1) * kC, zu);
-                    }
-                mbar_arrive_expect_tx(&ctl->fullqf[s], 2 * kTile);
-                for (int b = 0; b < 2; ++b) {
-                    tma_load_3d(st + b * kSlab, &map_o, &ctl->fullqf[s], 64 * b, row0 + c * kC, zu);
-                    tma_load_3d(st + kTile + b * kSlab, &map_f, &ctl->fullqf[s], 64 * b, row0 + c * kC, zu);
-                }
-                n_qf = c + 1;
-                if (c >= kStages) {
-                    mbar_wait(&ctl->emptyv[s], ((c / kStages) - 1) & 1, abort_flag);
-                    mbar_wait_drain(&ctl->full[s], ((c / kStages) - 1) & 1, 20000000ull);
-                }
-                mbar_arrive_expect_tx(&ctl->full[s], kTile);
-                for (int b = 0; b < 2; ++b)
-                    tma_load_3d(st + 2 * kTile + b * kSlab, &map_i, &ctl->full[s], 64 * b, row0 + c * kC, zu);
-                n_v = c + 1;
+        int n_qf = 0, n_v = 0;                                   // chunks whose tiles have been asked for
+        for (int c = 0; c < NC; ++c) {
+            const int s = c % kStages;
+            uint8_t *st = smem + s * kStageBytes;
+            // o and f have barriers of their own in both directions: the transform, which paces the kernel,
+            // needs only them, and their tiles are free as soon as Y = Qs S' of the chunk three back is done,
+            // well before its last product Y += P V has read V
+            // A barrier must never be armed twice within one phase.  Normally the stage's previous fill has long
+            // been consumed when its empty barrier completes; on the time-out exit that wait returns at once, so
+            // the previous fill is waited for explicitly (one poll that succeeds at once in normal running;
+            // stopping this lane on the wait's return value instead cost 8 %).
+            if (c >= kStages) {
+                mbar_wait(&ctl->emptyqf[s], ((c / kStages) - 1) & 1, abort_flag);
+                mbar_wait_drain(&ctl->fullqf[s], ((c / kStages) - 1) & 1, 20000000ull);
             }
-            ctl->l_qf = n_qf;
-            ctl->l_v = n_v;
+            // the next chunk's o, f tiles are asked into L2 now: their load can be issued only when their stage
+            // frees, one chunk from now, and then finds them there (measured on the fwd + bwd step: -1 %; two
+            // chunks ahead, or including the v tile, gave nothing)
+            if (c + 1 < NC)
+                for (int b = 0; b < 2; ++b) {
+                    tma_prefetch_3d(&map_o, 64 * b, row0 + (c + 1) * kC, zu);
+                    tma_prefetch_3d(&map_f, 64 * b, row0 + (c + 1) * kC, zu);
+                }
+            mbar_arrive_expect_tx(&ctl->fullqf[s], 2 * kTile);
+            for (int b = 0; b < 2; ++b) {
+                tma_load_3d(st + b * kSlab, &map_o, &ctl->fullqf[s], 64 * b, row0 + c * kC, zu);
+                tma_load_3d(st + kTile + b * kSlab, &map_f, &ctl->fullqf[s], 64 * b, row0 + c * kC, zu);
+            }
+            n_qf = c + 1;
+            if (c >= kStages) {
+                mbar_wait(&ctl->emptyv[s], ((c / kStages) - 1) & 1, abort_flag);
+                mbar_wait_drain(&ctl->full[s], ((c / kStages) - 1) & 1, 20000000ull);
+            }
+            mbar_arrive_expect_tx(&ctl->full[s], kTile);
+            for (int b = 0; b < 2; ++b)
+                tma_load_3d(st + 2 * kTile + b * kSlab, &map_i, &ctl->full[s], 64 * b, row0 + c * kC, zu);
+            n_v = c + 1;
         }
+        ctl->l_qf = n_qf;
+        ctl->l_v = n_v;
     } else if (warp == kWarpMmaS) {
         // ================= MS: state update =================
-        if (lane == 0) {
-            constexpr uint32_t idescS = idesc_bf16(128, 128, 1, 1);    // Ks^T (MN-major) x V (MN-major)
-            // Descriptors are formed once; a K step or a stage change only adds to the 14-bit
-            // start-address field (addresses are in 16-byte units and stay below 2^14).
-            const uint64_t dfm0 = smem_desc_sw128(smem_u32(smem) + kTile, kSlab, 1024);      // Ks, MN-major
-            const uint64_t dvm0 = smem_desc_sw128(smem_u32(smem) + 2 * kTile, kSlab, 1024);  // V, MN-major
-            constexpr uint32_t idescA = idesc_bf16(64, 64, 0, 0);      // Qs (K-major) x Ks (K-major)
-            const uint64_t dq0 = smem_desc_sw128(smem_u32(smem), 16, 1024);                  // Qs, K-major
-            const uint64_t dfk0 = smem_desc_sw128(smem_u32(smem) + kTile, 16, 1024);         // Ks, K-major
-            auto kmaj = [](int kk) { return (uint64_t)(((kk >> 2) * kSlab + (kk & 3) * 32) >> 4); };
-            PT_DECL
-            for (int c = 0; c < NC; ++c) {
-                const int s = c % kStages;
-                const uint64_t so = (uint64_t)s * (kStageBytes >> 4);
-                mbar_wait(&ctl->full[s], (c / kStages) & 1, abort_flag);
-                mbar_wait(&ctl->t_done[s], (c / kStages) & 1, abort_flag);
-                PT_MARK(0)
-                // A = Qs Ks^T is issued here, not by the lane of the other output products: this lane has nothing
-                // to do until the state is rescaled, and every tcgen05.mma also costs the issuing lane's scheduler
-                // (shared with a transform warp) issue time, so the products are spread over two schedulers
-                if (want_y) {
-                    const int b = c & 1;
-                    if (c >= 2) {                                    // tril(A) of chunk c - 2 has left this buffer
-                        mbar_wait(&ctl->p_ready[b], ((c - 2) >> 1) & 1, abort_flag);
-                        tc_fence_after_sync();
-                    }
-#pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        mma_bf16_ss(tmem + kColA + 64 * b, dq0 + so + kmaj(kk), dfk0 + so + kmaj(kk), idescA, kk > 0);
-                    mma_commit(&ctl->barA[b]);
+        constexpr uint32_t idescS = idesc_bf16(128, 128, 1, 1);    // Ks^T (MN-major) x V (MN-major)
+        // Descriptors are formed once; a K step or a stage change only adds to the 14-bit
+        // start-address field (addresses are in 16-byte units and stay below 2^14).
+        const uint64_t dfm0 = smem_desc_sw128(smem_u32(smem) + kTile, kSlab, 1024);      // Ks, MN-major
+        const uint64_t dvm0 = smem_desc_sw128(smem_u32(smem) + 2 * kTile, kSlab, 1024);  // V, MN-major
+        constexpr uint32_t idescA = idesc_bf16(64, 64, 0, 0);      // Qs (K-major) x Ks (K-major)
+        const uint64_t dq0 = smem_desc_sw128(smem_u32(smem), 16, 1024);                  // Qs, K-major
+        const uint64_t dfk0 = smem_desc_sw128(smem_u32(smem) + kTile, 16, 1024);         // Ks, K-major
+        auto kmaj = [](int kk) { return (uint64_t)(((kk >> 2) * kSlab + (kk & 3) * 32) >> 4); };
+        PT_DECL
+        for (int c = 0; c < NC; ++c) {
+            const int s = c % kStages;
+            const uint64_t so = (uint64_t)s * (kStageBytes >> 4);
+            mbar_wait(&ctl->full[s], (c / kStages) & 1, abort_flag);
+            mbar_wait(&ctl->t_done[s], (c / kStages) & 1, abort_flag);
+            PT_MARK(0)
+            // A = Qs Ks^T is issued here, not by the lane of the other output products: this lane has nothing
+            // to do until the state is rescaled, and every tcgen05.mma also costs the issuing lane's scheduler
+            // (shared with a transform warp) issue time, so the products are spread over two schedulers
+            if (want_y) {
+                const int b = c & 1;
+                if (c >= 2) {                                    // tril(A) of chunk c - 2 has left this buffer
+                    mbar_wait(&ctl->p_ready[b], ((c - 2) >> 1) & 1, abort_flag);
+                    tc_fence_after_sync();
                 }
-                mbar_wait(&ctl->m_tmem, c & 1, abort_flag);
-                PT_MARK(1)
-                tc_fence_after_sync();
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)              // S' += Ks^T V
-                    mma_bf16_ss(tmem + kColS, dfm0 + so + (uint64_t)(kk * 128), dvm0 + so + (uint64_t)(kk * 128),
-                                idescS, 1);
-                mma_commit(&ctl->barS);
-                mma_commit(&ctl->emptyqf[s]);
-                mma_commit(&ctl->emptyv[s]);
-                PT_MARK(2)
-                // the saved chunk state, straight from the operand copy of S' (this lane is idle until the next
-                // chunk's state is ready; in the lane that issues the outputs' products the wait for the store
-                // to have read 32 KB would hold those up)
-                mbar_wait(&ctl->m_done, c & 1, abort_flag);
+                for (int kk = 0; kk < 8; ++kk)
+                    mma_bf16_ss(tmem + kColA + 64 * b, dq0 + so + kmaj(kk), dfk0 + so + kmaj(kk), idescA, kk > 0);
+                mma_commit(&ctl->barA[b]);
+            }
+            mbar_wait(&ctl->m_tmem, c & 1, abort_flag);
+            PT_MARK(1)
+            tc_fence_after_sync();
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)              // S' += Ks^T V
+                mma_bf16_ss(tmem + kColS, dfm0 + so + (uint64_t)(kk * 128), dvm0 + so + (uint64_t)(kk * 128),
+                            idescS, 1);
+            mma_commit(&ctl->barS);
+            mma_commit(&ctl->emptyqf[s]);
+            mma_commit(&ctl->emptyv[s]);
+            PT_MARK(2)
+            // the saved chunk state, straight from the operand copy of S' (this lane is idle until the next
+            // chunk's state is ready; in the lane that issues the outputs' products the wait for the store
+            // to have read 32 KB would hold those up)
+            mbar_wait(&ctl->m_done, c & 1, abort_flag);
+            if (lane == 0) {
                 if (want_saved) {
                     tma_store_3d(&map_saved, sbuf, 0, 0, (int)(slot0 + c));
                     tma_store_3d(&map_saved, sbuf + kStateSlab, 64, 0, (int)(slot0 + c));
@@ -430,58 +428,57 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                 }
                 mbar_arrive(&ctl->barS2);                   // second arrival: the tcgen05.commit of Y = Qs S'
             }
-            PT_DUMP(status, 12, 3, true)
-            if (want_saved) tma_store_wait_all();
-            mma_commit(&ctl->drain);
+            __syncwarp();
         }
+        PT_DUMP(status, 12, 3, true)
+        if (want_saved && lane == 0) tma_store_wait_all();
+        mma_commit(&ctl->drain);
     } else if (warp == kWarpMmaY) {
         // ================= MY: outputs (+ saved-state stores) =================
-        if (lane == 0) {
-            constexpr uint32_t idescY = idesc_bf16(64, 128, 0, 1);     // Qs or P (K-major) x S' or V (MN-major)
-            const uint64_t dq0 = smem_desc_sw128(smem_u32(smem), 16, 1024);                  // Qs, K-major
-            const uint64_t dvm0 = smem_desc_sw128(smem_u32(smem) + 2 * kTile, kSlab, 1024);  // V, MN-major
-            const uint64_t dsm = smem_desc_sw128(smem_u32(sbuf), kStateSlab, 1024);          // S', MN-major
-            const uint64_t dp0 = smem_desc_sw128(smem_u32(pbuf), 16, 1024);                  // tril(A), K-major
-            auto kmaj = [](int kk) { return (uint64_t)(((kk >> 2) * kSlab + (kk & 3) * 32) >> 4); };
-            PT_DECL
-            for (int c = 0; c < NC; ++c) {
-                const int s = c % kStages, b = c & 1;
-                const uint64_t so = (uint64_t)s * (kStageBytes >> 4);
-                const uint64_t dq = dq0 + so, dvm = dvm0 + so;
-                const uint64_t dp = dp0 + (uint64_t)b * (kSlab >> 4);
-                const uint32_t ty = tmem + kColY + 128 * b;
-                mbar_wait(&ctl->full[s], (c / kStages) & 1, abort_flag);
-                mbar_wait(&ctl->t_done[s], (c / kStages) & 1, abort_flag);
-                PT_MARK(0)
-                mbar_wait(&ctl->m_done, c & 1, abort_flag);
-                PT_MARK(1)
-                if (want_y) {
-                    if (c >= 2) {
-                        mbar_wait(&ctl->y_tfree[b], ((c - 2) >> 1) & 1, abort_flag);
-                        tc_fence_after_sync();
-                    }
-#pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)          // Y = Qs S'
-                        mma_bf16_ss(ty, dq + kmaj(kk), dsm + (uint64_t)(kk * 128), idescY, kk > 0);
-                }
-                PT_MARK(2)
-                mma_commit(&ctl->barS2);
-                mma_commit(&ctl->emptyqf[s]);               // A and Y = Qs S' were the last readers of Qs, Ks here
-                if (want_y) {
-                    mbar_wait(&ctl->p_ready[b], (c >> 1) & 1, abort_flag);
-                    PT_MARK(3)
+        constexpr uint32_t idescY = idesc_bf16(64, 128, 0, 1);     // Qs or P (K-major) x S' or V (MN-major)
+        const uint64_t dq0 = smem_desc_sw128(smem_u32(smem), 16, 1024);                  // Qs, K-major
+        const uint64_t dvm0 = smem_desc_sw128(smem_u32(smem) + 2 * kTile, kSlab, 1024);  // V, MN-major
+        const uint64_t dsm = smem_desc_sw128(smem_u32(sbuf), kStateSlab, 1024);          // S', MN-major
+        const uint64_t dp0 = smem_desc_sw128(smem_u32(pbuf), 16, 1024);                  // tril(A), K-major
+        auto kmaj = [](int kk) { return (uint64_t)(((kk >> 2) * kSlab + (kk & 3) * 32) >> 4); };
+        PT_DECL
+        for (int c = 0; c < NC; ++c) {
+            const int s = c % kStages, b = c & 1;
+            const uint64_t so = (uint64_t)s * (kStageBytes >> 4);
+            const uint64_t dq = dq0 + so, dvm = dvm0 + so;
+            const uint64_t dp = dp0 + (uint64_t)b * (kSlab >> 4);
+            const uint32_t ty = tmem + kColY + 128 * b;
+            mbar_wait(&ctl->full[s], (c / kStages) & 1, abort_flag);
+            mbar_wait(&ctl->t_done[s], (c / kStages) & 1, abort_flag);
+            PT_MARK(0)
+            mbar_wait(&ctl->m_done, c & 1, abort_flag);
+            PT_MARK(1)
+            if (want_y) {
+                if (c >= 2) {
+                    mbar_wait(&ctl->y_tfree[b], ((c - 2) >> 1) & 1, abort_flag);
                     tc_fence_after_sync();
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)          // Y += P V
-                        mma_bf16_ss(ty, dp + (uint64_t)(kk * 2), dvm + (uint64_t)(kk * 128), idescY, 1);
-                    mma_commit(&ctl->barY[b]);
                 }
-                mma_commit(&ctl->emptyv[s]);
-                PT_MARK(4)
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)          // Y = Qs S'
+                    mma_bf16_ss(ty, dq + kmaj(kk), dsm + (uint64_t)(kk * 128), idescY, kk > 0);
             }
-            PT_DUMP(status, 15, 5, true)
-            mma_commit(&ctl->drain);
+            PT_MARK(2)
+            mma_commit(&ctl->barS2);
+            mma_commit(&ctl->emptyqf[s]);               // A and Y = Qs S' were the last readers of Qs, Ks here
+            if (want_y) {
+                mbar_wait(&ctl->p_ready[b], (c >> 1) & 1, abort_flag);
+                PT_MARK(3)
+                tc_fence_after_sync();
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)          // Y += P V
+                    mma_bf16_ss(ty, dp + (uint64_t)(kk * 2), dvm + (uint64_t)(kk * 128), idescY, 1);
+                mma_commit(&ctl->barY[b]);
+            }
+            mma_commit(&ctl->emptyv[s]);
+            PT_MARK(4)
         }
+        PT_DUMP(status, 15, 5, true)
+        mma_commit(&ctl->drain);
     } else {
         // ================= ST: Y stores =================
         if constexpr (!kRagged) {

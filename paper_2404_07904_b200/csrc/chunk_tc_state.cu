@@ -79,7 +79,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
     Ctl *ctl = reinterpret_cast<Ctl *>(smem + G::kOffCtl);
     volatile int *abort_flag = &ctl->abort_flag;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int u = blockIdx.x;
     // this CTA's segment: rows [row0, row0 + N) of plane zu, NC chunks
     int row0 = 0, zu = u, N = N_all, NC = NC_all;
@@ -217,45 +217,41 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
         }
     } else if (warp == kWarpLoad) {
         // ================= L: TMA loads =================
-        if (lane == 0) {
-            int issued = 0;
-            for (int n = 0; n < NC; ++n) {
-                const int s = n % kStages, c = kBwd ? n : NC - 1 - n;
-                uint8_t *st = smem + s * G::kStageBytes;
-                if (n >= kStages) {
-                    mbar_wait(&ctl->empty[s], ((n / kStages) - 1) & 1, abort_flag);
-                    // never arm a barrier twice within one phase (the wait above returns at once on the time-out exit)
-                    mbar_wait_drain(&ctl->full[s], ((n / kStages) - 1) & 1, 20000000ull);
-                }
-                mbar_arrive_expect_tx(&ctl->full[s], G::kStageBytes);
-                for (int b = 0; b < 2; ++b) {
-                    if (kBwd) tma_load_3d(st + G::kOffX + b * kSlab, &map_o, &ctl->full[s], 64 * b, row0 + c * kC, zu);
-                    tma_load_3d(st + G::kOffF + b * kSlab, &map_f, &ctl->full[s], 64 * b, row0 + c * kC, zu);
-                    tma_load_3d(st + G::kOffW + b * kSlab, &map_w, &ctl->full[s], 64 * b, row0 + c * kC, zu);
-                }
-                issued = n + 1;
+        int issued = 0;
+        for (int n = 0; n < NC; ++n) {
+            const int s = n % kStages, c = kBwd ? n : NC - 1 - n;
+            uint8_t *st = smem + s * G::kStageBytes;
+            if (n >= kStages) {
+                mbar_wait(&ctl->empty[s], ((n / kStages) - 1) & 1, abort_flag);
+                // never arm a barrier twice within one phase (the wait above returns at once on the time-out exit)
+                mbar_wait_drain(&ctl->full[s], ((n / kStages) - 1) & 1, 20000000ull);
             }
-            ctl->l_issued = issued;
+            mbar_arrive_expect_tx(&ctl->full[s], G::kStageBytes);
+            for (int b = 0; b < 2; ++b) {
+                if (kBwd) tma_load_3d(st + G::kOffX + b * kSlab, &map_o, &ctl->full[s], 64 * b, row0 + c * kC, zu);
+                tma_load_3d(st + G::kOffF + b * kSlab, &map_f, &ctl->full[s], 64 * b, row0 + c * kC, zu);
+                tma_load_3d(st + G::kOffW + b * kSlab, &map_w, &ctl->full[s], 64 * b, row0 + c * kC, zu);
+            }
+            issued = n + 1;
         }
+        ctl->l_issued = issued;
     } else {
         // ================= M: accumulate X^T W =================
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(128, 128, 1, 1);           // X^T (MN-major) x W (MN-major)
-            const uint64_t dx0 = smem_desc_sw128(smem_u32(smem) + G::kOffX, kSlab, 1024);
-            const uint64_t dw0 = smem_desc_sw128(smem_u32(smem) + G::kOffW, kSlab, 1024);
-            for (int n = 0; n < NC; ++n) {
-                const int s = n % kStages;
-                const uint64_t so = (uint64_t)s * (G::kStageBytes >> 4);
-                mbar_wait(&ctl->t_done[s], (n / kStages) & 1, abort_flag);
-                tc_fence_after_sync();
+        constexpr uint32_t idesc = idesc_bf16(128, 128, 1, 1);           // X^T (MN-major) x W (MN-major)
+        const uint64_t dx0 = smem_desc_sw128(smem_u32(smem) + G::kOffX, kSlab, 1024);
+        const uint64_t dw0 = smem_desc_sw128(smem_u32(smem) + G::kOffW, kSlab, 1024);
+        for (int n = 0; n < NC; ++n) {
+            const int s = n % kStages;
+            const uint64_t so = (uint64_t)s * (G::kStageBytes >> 4);
+            mbar_wait(&ctl->t_done[s], (n / kStages) & 1, abort_flag);
+            tc_fence_after_sync();
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    mma_bf16_ss(tmem, dx0 + so + (uint64_t)(kk * 128), dw0 + so + (uint64_t)(kk * 128), idesc,
-                                (n > 0 || kk > 0) ? 1u : 0u);
-                mma_commit(&ctl->empty[s]);
-            }
-            mma_commit(&ctl->acc_done);
+            for (int kk = 0; kk < 4; ++kk)
+                mma_bf16_ss(tmem, dx0 + so + (uint64_t)(kk * 128), dw0 + so + (uint64_t)(kk * 128), idesc,
+                            (n > 0 || kk > 0) ? 1u : 0u);
+            mma_commit(&ctl->empty[s]);
         }
+        mma_commit(&ctl->acc_done);
     }
     tc_fence_before_sync();
     __syncthreads();

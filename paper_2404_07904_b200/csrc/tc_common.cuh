@@ -46,9 +46,11 @@ __device__ __forceinline__ void fence_barrier_init()
 {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
+// Whole warp, see "warp-wide issue" below; so are the copies.
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
 {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
@@ -155,6 +157,16 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity, 
     return true;
 }
 
+// ---- warp-wide issue --------------------------------------------------------------------------------
+// The roles that issue tensor-core products and bulk copies run as whole warps, and only the issuing instruction itself
+// is predicated to one lane, elected anew each time (always the same one).  A role that runs inside `if (lane == 0)` is
+// divergent code, where the compiler has to move every descriptor and address into the uniform registers these
+// instructions take, two moves per descriptor of every product; in code it knows to be convergent (`warp` comes
+// from a shuffle for that reason) they are formed there.  With 20 products on the critical chain of a chunk of the
+// backward this counts: 148 units of 2048 tokens backward 148 -> 140 us (145 with the products alone, the copies still
+// issued from one lane), 128 units 141 -> 136 us, forward 73 -> 71 us.
+// Everything below that says "whole warp" must be reached by all lanes of a warp together.
+
 // ---- proxies and fences -------------------------------------------------------------------------
 // Makes generic-proxy writes to shared memory visible to the async proxy (TMA, tcgen05.mma).
 __device__ __forceinline__ void fence_proxy_async_smem()
@@ -169,19 +181,21 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *map)
 {
     asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
-// 3-D tiled load: coordinates (x = innermost element, y, z); completion is counted in bytes on `bar`.
+// Whole warp: 3-D tiled load: coordinates (x = innermost element, y, z); completion is counted in bytes on `bar`.
 // x * element size must be a multiple of 16 bytes.
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y, int z)
 {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];\n\t}"
         ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
         : "memory");
 }
-// Asks for the tile to be brought into L2 (no shared-memory destination, no completion to wait for).
+// Whole warp: asks for the tile to be brought into L2 (no shared-memory destination, no completion to wait for).
 __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap *map, int x, int y, int z)
 {
-    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];"
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];\n\t}"
                  ::"l"(map), "r"(x), "r"(y), "r"(z)
                  : "memory");
 }
@@ -212,21 +226,25 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem], bf16 operands, fp32 accumulation; issued by ONE thread.
+// D[tmem] (+)= A[smem] * B[smem], bf16 operands, fp32 accumulation.  Called by a whole warp, issued by its elected lane
+// (see "warp-wide issue" above).
 __device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                             uint32_t accumulate)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// Arrives once on `bar` when every tcgen05 operation this thread issued before has completed.
+// Arrives once on `bar` when every tcgen05 operation this warp issued before has completed (called by the whole warp).
 __device__ __forceinline__ void mma_commit(uint64_t *bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+    asm volatile("{\n\t.reg .pred e;\n\t"
+                 "elect.sync _|e, 0xffffffff;\n\t"
+                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar))
                  : "memory");
 }
 
