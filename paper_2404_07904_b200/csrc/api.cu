@@ -472,8 +472,8 @@ hgrn2_status hgrn2_span_summary_fwd(const hgrn2_desc *desc, const void *f, const
     if (U == 0) return cudaMemsetAsync(ws, 0, sizeof(StatusBlock), stream) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
     cudaError_t e;
     if (use_tc(desc) && desc->N > 0) {
-        e = launch_tc_state_fwd(f, i, (uint64_t)U, desc->N, S_loc, lam, false, static_cast<StatusBlock *>(ws), true,
-                                (desc->flags & HGRN2_FLAG_DEBUG_EXPIRE_WAITS) ? 1 : 0, stream);
+        e = launch_tc_span(false, nullptr, f, i, (uint64_t)U, desc->N, S_loc, lam, static_cast<StatusBlock *>(ws), true,
+                           (desc->flags & HGRN2_FLAG_DEBUG_EXPIRE_WAITS) ? 1 : 0, stream);
     } else {
         if (cudaMemsetAsync(ws, 0, sizeof(StatusBlock), stream) != cudaSuccess) return HGRN2_ERR_CUDA;
         e = launch_span_summary(false, desc->io, nullptr, f, i, U, desc->N, desc->dk, desc->dv, S_loc, lam, stream);
@@ -498,8 +498,8 @@ hgrn2_status hgrn2_span_summary_bwd(const hgrn2_desc *desc, const void *o, const
     if (U == 0) return cudaMemsetAsync(ws, 0, sizeof(StatusBlock), stream) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
     cudaError_t e;
     if (use_tc(desc) && desc->N > 0) {
-        e = launch_tc_state_bwd(o, f, dy, (uint64_t)U, desc->N, G_loc, lam, false, static_cast<StatusBlock *>(ws), true,
-                                (desc->flags & HGRN2_FLAG_DEBUG_EXPIRE_WAITS) ? 1 : 0, stream);
+        e = launch_tc_span(true, o, f, dy, (uint64_t)U, desc->N, G_loc, lam, static_cast<StatusBlock *>(ws), true,
+                           (desc->flags & HGRN2_FLAG_DEBUG_EXPIRE_WAITS) ? 1 : 0, stream);
     } else {
         if (cudaMemsetAsync(ws, 0, sizeof(StatusBlock), stream) != cudaSuccess) return HGRN2_ERR_CUDA;
         e = launch_span_summary(true, desc->io, o, f, dy, U, desc->N, desc->dk, desc->dv, G_loc, lam, stream);

@@ -62,6 +62,7 @@ constexpr int kWarpE1 = kTWarps, kWarpE3 = kWarpE1 + kE1Warps, kWarpO = kWarpE3 
 constexpr int kWarpLoad = kWarpO + kOWarps, kWarpMmaX = kWarpLoad + 1, kWarpMmaY1 = kWarpLoad + 2,
               kWarpMmaY2 = kWarpLoad + 3;
 constexpr int kThreads = (kWarpMmaY2 + 1) * 32;
+constexpr int kRingWarps = kTWarps + kE1Warps + kE3Warps + kOWarps + 3;   // readers of the item ring
 
 constexpr int kStages = 2;
 constexpr uint32_t kStageBytes = 3 * kTile;                       // q, dy, f: free again when the chunk's products are done
@@ -79,7 +80,7 @@ constexpr uint32_t kOffRawF = kOffRawO + kTile;                   // the output 
 constexpr uint32_t kOffR = kOffRawF + kTile;                      // float rr[2][128]
 constexpr uint32_t kOffX = kOffR + 2 * 128 * 4;                   // float xa[128], xe[128]
 constexpr uint32_t kOffCtl = kOffX + 2 * 128 * 4;
-constexpr uint32_t kSmemBytes = kOffCtl + 256;                    // no slack: the base must be 1024-byte aligned
+constexpr uint32_t kSmemBytes = kOffCtl + 768;                    // no slack: the base must be 1024-byte aligned
 
 constexpr uint32_t kColDS = 0, kColA = 128, kColDA = 192, kColDQ = 256, kColDKi = 320, kColDKx = 384, kColDV = 448;
 
@@ -103,13 +104,14 @@ struct Ctl {
     uint64_t parked;              // E3 -> E3: every thread's parked values and the halves' sums are in place
     uint64_t acc_free2;           // E3 -> M: dQs^T and dKs_intra^T columns are free again
     uint64_t drain;               // tcgen05.commit (MX, MY1, MY2, after their loops): every product issued has completed
+    alignas(16) ItemRing ring;
     int abort_flag;               // set by the first wait that runs out: every later wait returns at once
     uint32_t tmem_base;
     int o_done;                   // E3 -> T: output walks finished so far, counted per warp (pacing only)
     int exact_flag;               // E1: a decay of this CTA's tokens left the range of the rescaled operands
     int l_stage, l_v, l_state, l_raw;   // L: fills asked for so far, per buffer, for the abort epilogue
 };
-static_assert(sizeof(Ctl) <= 256, "control block");
+static_assert(sizeof(Ctl) <= 768, "control block");
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 
 constexpr int kExactC = 32;       // chunk length of the exact fp32 routines at d = 128 (their shared-memory budget)
@@ -219,19 +221,19 @@ __device__ __forceinline__ void phase_main(uint32_t tmem_lane, const unsigned sh
     esum = asum - W;
 }
 
-// kRagged: N is not a whole number of chunks (the tail chunk is padded with neutral tokens); when false,
-// every per-row validity test below folds away.
-// kMultiCta: a unit runs as several CTAs (segments) of this launch (see the forward kernel).
+// kRagged: sequences need not be whole chunks (a partial chunk is padded with neutral tokens), and a packed batch is one.
 // kEnc: the f tensor holds the signed gate encoding (see transform_half); d_f stays the gradient with respect to f.
-template <bool kRagged, bool kMultiCta, bool kEnc>
+// kPersist: several items per CTA (tc_chunk.cuh).
+template <bool kRagged, bool kEnc, bool kPersist>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__ CUtensorMap map_f,
               const __grid_constant__ CUtensorMap map_i, const __grid_constant__ CUtensorMap map_dy,
               const __grid_constant__ CUtensorMap map_saved, const __grid_constant__ CUtensorMap map_o_raw,
               const __grid_constant__ CUtensorMap map_f_raw, const float *__restrict__ totals,
-              const float *__restrict__ dSN, __nv_bfloat16 *__restrict__ d_o, __nv_bfloat16 *__restrict__ d_f,
-              __nv_bfloat16 *__restrict__ d_i, float *__restrict__ dS0, int N_all, int NC_all, StatusBlock *status,
-              int clear_status, const ExactArgs ex, const PackedArgs pk, int start_aborted)
+              const float *__restrict__ dSN, const float *__restrict__ chain, __nv_bfloat16 *__restrict__ d_o,
+              __nv_bfloat16 *__restrict__ d_f, __nv_bfloat16 *__restrict__ d_i, float *__restrict__ dS0,
+              const __grid_constant__ WorkArgs wk, StatusBlock *status, int clear_status, const ExactArgs ex,
+              int start_aborted)
 {
     // the first kernel of a call zeroes the status word; the only early report, the alignment check below, is the
     // same in every CTA, so CTA 0 repeats it after its own clear
@@ -259,33 +261,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     volatile int *abort_flag = &ctl->abort_flag;
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    const int u = blockIdx.x;
-    // This CTA's sequence: rows [row0, row0 + N) of plane zu of the [planes][rows][128] tensors, NC chunks, chunk-start
-    // state c in slot slot0 + c.  Packed batches (ragged instantiations only) read theirs from the offsets array.
-    int row0 = 0, zu = u, N = N_all, NC = NC_all;
-    size_t slot0 = (size_t)u * NC_all;
-    if constexpr (kRagged) {
-        if (pk.cu != nullptr) {
-            const int b = u / pk.H;
-            zu = u - b * pk.H;
-            row0 = __ldg(pk.cu + b);
-            N = __ldg(pk.cu + b + 1) - row0;
-            NC = (N + kC - 1) / kC;
-            slot0 = (size_t)zu * pk.slots_per_head + row0 / kC + b;
-            if (row0 < 0 || N < 0 || row0 + N > N_all) {          // malformed offsets: report, touch nothing
-                if (tid == 0) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
-                return;
-            }
-            if (N <= 0) {                // empty sequence: the state gradient passes through
-                if (dS0 != nullptr)
-                    for (int x = tid; x < kD * kD; x += kThreads)
-                        dS0[(size_t)u * kD * kD + x] = dSN ? dSN[(size_t)u * kD * kD + x] : 0.f;
-                return;
-            }
-        }
-    }
-    const size_t grow0 = (size_t)zu * N_all + row0;                 // first row of the sequence in the [planes * rows][128] view
-
+    bool malformed = false;
+    const Item first = warp_uniform(work_item<kRagged, true>(wk, blockIdx.x, malformed));
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&ctl->full[s], 1);
@@ -312,7 +289,13 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         ctl->o_done = 0;
         ctl->exact_flag = 0;
         ctl->l_stage = ctl->l_v = ctl->l_state = ctl->l_raw = 0;
+        ring_init(ctl->ring, kRingWarps);
         fence_barrier_init();
+        if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
+        if (kPersist) {
+            ctl->ring.item[0] = first;
+            mbar_arrive(&ctl->ring.full[0]);
+        }
         tma_prefetch_desc(&map_o);
         tma_prefetch_desc(&map_f);
         tma_prefetch_desc(&map_i);
@@ -330,334 +313,389 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     const uint32_t lane_base = static_cast<uint32_t>(32 * sub) << 16;
     const int krow = 32 * sub + lane;                                // TMEM lane of this thread
 
-    // it = 0, 1, ... counts processed chunks; chunk index c = NC - 1 - it
+    // it = 0, 1, ... counts the chunks over all of the CTA's items; an item's chunks are visited from its last to its first
     if (warp < kTWarps) {
         // ================= T: transform =================
         PT_DECL
-        for (int it = 0; it < NC; ++it) {
-            const int s = it % kStages, c = NC - 1 - it;
-            uint8_t *qbuf = smem + s * kStageBytes;
-            mbar_wait(&ctl->full[s], (it / kStages) & 1, abort_flag);
-            // Pacing, not a data dependence: the transform of chunk `it` starts only when the output walk of chunk
-            // it - 2 is over (its completion pass may still run).  The tiles are there well before, but run earlier
-            // the transform shares the issue slots with that walk, the longest stretch of the per-chunk loop
-            // (event stamps: waiting for the completion pass as well made this the longest chain of the kernel;
-            // no pacing at all measured the same as this).
-            if (it >= 2) {
-                if (lane == 0) count_wait(&ctl->o_done, kE3Warps * (it - 1), abort_flag);   // one poller per warp
-                __syncwarp();
+        int it = 0;
+        Item im;
+        for (int k = 0; next_item<kPersist>(&ctl->ring, k, abort_flag, first, im); ++k) {
+            for (int c = (im.n + kC - 1) / kC - 1; c >= 0; --c, ++it) {
+                const int s = it % kStages;
+                uint8_t *qbuf = smem + s * kStageBytes;
+                mbar_wait(&ctl->full[s], (it / kStages) & 1, abort_flag);
+                // Pacing, not a data dependence: the transform of chunk `it` starts only when the output walk of chunk
+                // it - 2 is over (its completion pass may still run).  The tiles are there well before, but run earlier
+                // the transform shares the issue slots with that walk, the longest stretch of the per-chunk loop
+                // (event stamps: waiting for the completion pass as well made this the longest chain of the kernel;
+                // no pacing at all measured the same as this).
+                if (it >= 2) {
+                    if (lane == 0) count_wait(&ctl->o_done, kE3Warps * (it - 1), abort_flag);   // one poller per warp
+                    __syncwarp();
+                }
+                PT_MARK(0)
+                PT_STAMP(status, 1, tid == 0 && it == 16) PT_STAMP(status, 20, tid == 0 && it == 18)
+                // Pm and E of the chunk are not kept: the backward takes them from what the forward saved
+                if (kRagged && im.n - c * kC < kC) neutral_rows<kEnc, kSS, kSlab>(qbuf + kOffQ, qbuf + kOffK, im.n - c * kC, tid);
+                transform_stream<kEnc, kSS, kSlab>(qbuf + kOffQ, qbuf + kOffK, nullptr, nullptr, nullptr, nullptr, tid);
+                fence_proxy_async_smem();
+                mbar_arrive(&ctl->t_done[s]);
+                PT_MARK(1)
+                PT_STAMP(status, 2, tid == 0 && it == 16)
             }
-            PT_MARK(0)
-            PT_STAMP(status, 1, tid == 0 && it == 16) PT_STAMP(status, 20, tid == 0 && it == 18)
-            const int n_valid = kRagged ? N - c * kC : kC;
-            // Pm and E of the chunk are not kept: the backward takes them from what the forward saved
-            if (kRagged && n_valid < kC) neutral_rows<kEnc, kSS, kSlab>(qbuf + kOffQ, qbuf + kOffK, n_valid, tid);
-            transform_stream<kEnc, kSS, kSlab>(qbuf + kOffQ, qbuf + kOffK, nullptr, nullptr, nullptr, nullptr, tid);
-            fence_proxy_async_smem();
-            mbar_arrive(&ctl->t_done[s]);
-            PT_MARK(1)
-            PT_STAMP(status, 2, tid == 0 && it == 16)
         }
         PT_DUMP(status, 0, 2, tid == 0)
     } else if (warp < kWarpE3) {
         // ================= E1: state-gradient warps =================
         // Pm, E of every chunk come from the forward's saved totals, so this chain does not wait for T
-        float pm_prev = 1.f;
-        const float *tot_u = totals + slot0 * 2 * kD + krow;
-        float pm_c = __ldg(tot_u + (size_t)(NC - 1) * 2 * kD), ee_c = __ldg(tot_u + (size_t)(NC - 1) * 2 * kD + kD);
         PT_DECL
-        for (int it = 0; it < NC; ++it) {
-            // ---- dS'' = (Pm_prev E) dS' (the accumulator, or dSN first) -> TMEM, bf16 copy -> dsbuf
-            PT_MARK(0)
-            // a total on the floor: the decay across that half chunk is more than the rescaled operands can carry
-            if (fminf(pm_c, ee_c) <= kProdFloor) ctl->exact_flag = 1;
-            const float pm_old = pm_prev, ee_old = ee_c;
-            const float factor = pm_prev * ee_c;
-            pm_prev = pm_c;
-            if (it + 1 < NC) {
-                pm_c = __ldg(tot_u + (size_t)(NC - 2 - it) * 2 * kD);
-                ee_c = __ldg(tot_u + (size_t)(NC - 2 - it) * 2 * kD + kD);
-            }
-            if (it > 0) {
-                mbar_wait(&ctl->barX, (it - 1) & 1, abort_flag);   // dS' of the previous chunk is complete
-                mbar_wait(&ctl->barY1, (it - 1) & 1, abort_flag);    // its dS'' copy is no longer read
+        int it = 0;
+        Item im;
+        for (int k = 0; next_item<kPersist>(&ctl->ring, k, abort_flag, first, im); ++k) {
+            const int nc = (im.n + kC - 1) / kC;
+            const size_t row = ((size_t)im.unit * kD + krow) * kD;
+            float pm_prev = 1.f, pm_c = 1.f, ee_c = 1.f;
+            const float *tot_u = totals + (size_t)im.slot0 * 2 * kD + krow;
+            // the accumulator starts as the gradient that comes in, so the loop over the chunks has no first-chunk case (the
+            // previous item's last update of it is done behind barX)
+            if (nc > 0) {
+                const float *init = im.chain >= 0 ? chain + ((size_t)im.chain * kD + krow) * kD : (dSN ? dSN + row : nullptr);
+                pm_c = __ldg(tot_u + (size_t)(nc - 1) * 2 * kD);
+                ee_c = __ldg(tot_u + (size_t)(nc - 1) * 2 * kD + kD);
+                if (it > 0) mbar_wait(&ctl->barX, (it - 1) & 1, abort_flag);
                 tc_fence_after_sync();
-            }
-            PT_MARK(1)
-            PT_STAMP(status, 5, tid == kWarpE1 * 32 && it == 16)
 #pragma unroll 1
-            for (int part = 0; part < 4; ++part) {
-                uint32_t r[32];
-                if (it == 0) {
-                    if (dSN) {
-                        const float4 *src = reinterpret_cast<const float4 *>(dSN + ((size_t)u * kD + krow) * kD + 32 * part);
+                for (int part = 0; part < 4; ++part) {
+                    uint32_t r[32];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const float4 v4 = __ldg(src + j);
-                            r[4 * j + 0] = __float_as_uint(v4.x); r[4 * j + 1] = __float_as_uint(v4.y);
-                            r[4 * j + 2] = __float_as_uint(v4.z); r[4 * j + 3] = __float_as_uint(v4.w);
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) r[j] = 0u;
+                    for (int j = 0; j < 8; ++j) {
+                        const float4 v4 = init ? __ldg(reinterpret_cast<const float4 *>(init + 32 * part) + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        r[4 * j + 0] = __float_as_uint(v4.x); r[4 * j + 1] = __float_as_uint(v4.y);
+                        r[4 * j + 2] = __float_as_uint(v4.z); r[4 * j + 3] = __float_as_uint(v4.w);
                     }
-                } else {
+                    tmem_st32(tmem + lane_base + kColDS + 32 * part, r);
+                }
+                tmem_wait_st();
+            }
+            for (int c = nc - 1; c >= 0; --c, ++it) {
+                // ---- dS'' = (Pm_prev E) dS' (the accumulator) -> TMEM, bf16 copy -> dsbuf
+                PT_MARK(0)
+                // a total on the floor: the decay across that half chunk is more than the rescaled operands can carry
+                if (fminf(pm_c, ee_c) <= kProdFloor) {
+                    ctl->exact_flag = 1;
+                    if (kPersist) ctl->ring.flagged[k & 7] = im.id + 1;
+                }
+                const float pm_old = pm_prev, ee_old = ee_c;
+                const float factor = pm_prev * ee_c;
+                pm_prev = pm_c;
+                const bool safe = factor >= kFactorSafe;
+                if (c > 0) {
+                    pm_c = __ldg(tot_u + (size_t)(c - 1) * 2 * kD);
+                    ee_c = __ldg(tot_u + (size_t)(c - 1) * 2 * kD + kD);
+                }
+                if (it > 0) {
+                    mbar_wait(&ctl->barX, (it - 1) & 1, abort_flag);   // dS' of the previous chunk is complete
+                    mbar_wait(&ctl->barY1, (it - 1) & 1, abort_flag);    // its dS'' copy is no longer read
+                    tc_fence_after_sync();
+                }
+                PT_MARK(1)
+                PT_STAMP(status, 5, tid == kWarpE1 * 32 && it == 16)
+#pragma unroll 1
+                for (int part = 0; part < 4; ++part) {
+                    uint32_t r[32];
                     tmem_ld32(tmem + lane_base + kColDS + 32 * part, r);
                     tmem_wait_ld();
-                }
-                if (factor >= kFactorSafe) {
-#pragma unroll
-                    for (int j = 0; j < 32; j += 2) scale2(r[j], r[j + 1], factor);
-                } else {                         // see the forward kernel: the two decays one after the other
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) * pm_old * ee_old);
-                }
-                tmem_st32(tmem + lane_base + kColDS + 32 * part, r);
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    *reinterpret_cast<uint4 *>(dsbuf + (part >> 1) * kStateSlab + slab_chunk_off(krow, 4 * (part & 1) + j)) =
-                        pack8(r + 8 * j);
-            }
-            tmem_wait_st();
-            tc_fence_before_sync();
-            fence_proxy_async_smem();
-            mbar_arrive(&ctl->m_done);
-            PT_MARK(2)
-            PT_STAMP(status, 6, tid == kWarpE1 * 32 && it == 16)
-
-            // ---- R_k = sum_v dS''[k,v] S'[k,v] from the two bf16 copies
-            mbar_wait(&ctl->sfull, it & 1, abort_flag);
-            PT_MARK(3)
-            float2 racc2 = make_float2(0.f, 0.f);
+                    float f1 = safe ? factor : pm_old;               // see the forward kernel: or the two decays one after the other
 #pragma unroll 1
-            for (int h = 0; h < 2; ++h) {
+                    for (int more = safe ? 0 : 1; more >= 0; --more, f1 = ee_old)
+#pragma unroll
+                        for (int j = 0; j < 32; j += 2) scale2(r[j], r[j + 1], f1);
+                    tmem_st32(tmem + lane_base + kColDS + 32 * part, r);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        *reinterpret_cast<uint4 *>(dsbuf + (part >> 1) * kStateSlab + slab_chunk_off(krow, 4 * (part & 1) + j)) =
+                            pack8(r + 8 * j);
+                }
+                tmem_wait_st();
+                tc_fence_before_sync();
+                fence_proxy_async_smem();
+                mbar_arrive(&ctl->m_done);
+                PT_MARK(2)
+                PT_STAMP(status, 6, tid == kWarpE1 * 32 && it == 16)
+
+                // ---- R_k = sum_v dS''[k,v] S'[k,v] from the two bf16 copies
+                mbar_wait(&ctl->sfull, it & 1, abort_flag);
+                PT_MARK(3)
+                float2 racc2 = make_float2(0.f, 0.f);
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
 #pragma unroll 2
-                for (int j = 0; j < 8; ++j) {
-                    const uint32_t off = h * kStateSlab + slab_chunk_off(krow, j);
-                    const uint4 dw = *reinterpret_cast<const uint4 *>(dsbuf + off);
-                    const uint4 sw = *reinterpret_cast<const uint4 *>(sbuf + off);
-                    racc2 = fma2(make_float2(bf16_lo(dw.x), bf16_hi(dw.x)), make_float2(bf16_lo(sw.x), bf16_hi(sw.x)), racc2);
-                    racc2 = fma2(make_float2(bf16_lo(dw.y), bf16_hi(dw.y)), make_float2(bf16_lo(sw.y), bf16_hi(sw.y)), racc2);
-                    racc2 = fma2(make_float2(bf16_lo(dw.z), bf16_hi(dw.z)), make_float2(bf16_lo(sw.z), bf16_hi(sw.z)), racc2);
-                    racc2 = fma2(make_float2(bf16_lo(dw.w), bf16_hi(dw.w)), make_float2(bf16_lo(sw.w), bf16_hi(sw.w)), racc2);
+                    for (int j = 0; j < 8; ++j) {
+                        const uint32_t off = h * kStateSlab + slab_chunk_off(krow, j);
+                        const uint4 dw = *reinterpret_cast<const uint4 *>(dsbuf + off);
+                        const uint4 sw = *reinterpret_cast<const uint4 *>(sbuf + off);
+                        racc2 = fma2(make_float2(bf16_lo(dw.x), bf16_hi(dw.x)), make_float2(bf16_lo(sw.x), bf16_hi(sw.x)), racc2);
+                        racc2 = fma2(make_float2(bf16_lo(dw.y), bf16_hi(dw.y)), make_float2(bf16_lo(sw.y), bf16_hi(sw.y)), racc2);
+                        racc2 = fma2(make_float2(bf16_lo(dw.z), bf16_hi(dw.z)), make_float2(bf16_lo(sw.z), bf16_hi(sw.z)), racc2);
+                        racc2 = fma2(make_float2(bf16_lo(dw.w), bf16_hi(dw.w)), make_float2(bf16_lo(sw.w), bf16_hi(sw.w)), racc2);
+                    }
+                }
+                const float racc = racc2.x + racc2.y;
+                rr[(it & 1) * 128 + krow] = racc;
+                mbar_arrive(&ctl->r_ready[it & 1]);
+                PT_MARK(4)
+                PT_STAMP(status, 9, tid == kWarpE1 * 32 && it == 16)
+            }
+            // dS_0 = Diag(Pm of chunk 0) dS'; without tokens the gradient passes through
+            if (dS0 != nullptr && im.last) {
+                if (nc > 0) {
+                    mbar_wait(&ctl->barX, (it - 1) & 1, abort_flag);
+                    tc_fence_after_sync();
+                }
+#pragma unroll 1
+                for (int part = 0; part < 4; ++part) {
+                    uint32_t r[32];
+                    float4 *dst = reinterpret_cast<float4 *>(dS0 + row + 32 * part);
+                    if (nc > 0) {
+                        tmem_ld32(tmem + lane_base + kColDS + 32 * part, r);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            dst[j] = make_float4(__uint_as_float(r[4 * j + 0]) * pm_prev, __uint_as_float(r[4 * j + 1]) * pm_prev,
+                                                 __uint_as_float(r[4 * j + 2]) * pm_prev, __uint_as_float(r[4 * j + 3]) * pm_prev);
+                    } else {
+#pragma unroll 1
+                        for (int j = 0; j < 8; ++j)
+                            dst[j] = dSN ? reinterpret_cast<const float4 *>(dSN + row + 32 * part)[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
                 }
             }
-            const float racc = racc2.x + racc2.y;
-            rr[(it & 1) * 128 + krow] = racc;
-            mbar_arrive(&ctl->r_ready[it & 1]);
-            PT_MARK(4)
-            PT_STAMP(status, 9, tid == kWarpE1 * 32 && it == 16)
         }
         PT_DUMP(status, 2, 5, tid == kWarpE1 * 32)
-
-        // dS_0 = Diag(Pm of chunk 0) dS'
-        mbar_wait(&ctl->barY2, (NC - 1) & 1, abort_flag);
-        tc_fence_after_sync();
-        if (dS0) {
-#pragma unroll 1
-            for (int part = 0; part < 4; ++part) {
-                uint32_t r[32];
-                tmem_ld32(tmem + lane_base + kColDS + 32 * part, r);
-                tmem_wait_ld();
-                float4 *dst = reinterpret_cast<float4 *>(dS0 + ((size_t)u * kD + krow) * kD + 32 * part);
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    dst[j] = make_float4(__uint_as_float(r[4 * j + 0]) * pm_prev, __uint_as_float(r[4 * j + 1]) * pm_prev,
-                                         __uint_as_float(r[4 * j + 2]) * pm_prev, __uint_as_float(r[4 * j + 3]) * pm_prev);
-            }
-        }
     } else if (warp < kWarpO) {
         // ================= E3: d_o and d_f =================
         const int half = (warp - kWarpE3) >> 2;                      // half of the chunk: local times [32 * half, +32)
         const uint32_t tl = tmem + lane_base;
         PT_DECL
-        for (int it = 0; it < NC; ++it) {
-            const int c = NC - 1 - it;
-            const int n_valid = kRagged ? min(kC, N - c * kC) : kC;
-            const size_t crow0 = grow0 + (size_t)c * kC;
-            // ---- outputs
-            mbar_wait(&ctl->rawfull, it & 1, abort_flag);
-            mbar_wait(&ctl->barY2, it & 1, abort_flag);
-            PT_MARK(2)
-            tc_fence_after_sync();
-            float asum, esum;
-            PT_STAMP(status, 14, tid == kWarpE3 * 32 && it == 16)
-            __nv_bfloat16 *do_g = d_o + crow0 * kD + krow;
-            if (kRagged && n_valid < kC) {
-                // rows beyond the end: see neutral_rows (this thread's column of its half)
+        int it = 0;
+        Item im;
+        for (int k = 0; next_item<kPersist>(&ctl->ring, k, abort_flag, first, im); ++k) {
+            const size_t grow0 = (size_t)im.plane * wk.N + im.row0;     // first row of the item in the [planes * rows][128] view
+            for (int c = (im.n + kC - 1) / kC - 1; c >= 0; --c, ++it) {
+                const int n_valid = kRagged ? min(kC, im.n - c * kC) : kC;
+                const size_t crow0 = grow0 + c * kC;
+                // ---- outputs
+                mbar_wait(&ctl->rawfull, it & 1, abort_flag);
+                mbar_wait(&ctl->barY2, it & 1, abort_flag);
+                PT_MARK(2)
+                tc_fence_after_sync();
+                float asum, esum;
+                PT_STAMP(status, 14, tid == kWarpE3 * 32 && it == 16)
+                __nv_bfloat16 *do_g = d_o + crow0 * kD + krow;
+                if (kRagged && n_valid < kC) {
+                    // rows beyond the end: see neutral_rows (this thread's column of its half)
 #pragma unroll 1
-                for (int r = max(n_valid, 32 * half); r < 32 * half + 32; ++r) {
-                    oraw[r * kD + krow] = 0u;
-                    fraw[r * kD + krow] = kEnc ? 0x8000u : 0x3F80u;
-                }
-                if (half) phase_main<true, true, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
-                else      phase_main<false, true, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
-                fence_proxy_async_smem();                        // the rows written here, before the tiles' next load
-            } else {
-                if (half) phase_main<true, false, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
-                else      phase_main<false, false, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
-            }
-            mbar_arrive(&ctl->raw_read);
-            if (half) xa[krow] = asum; else xe[krow] = esum;
-            tmem_wait_st();
-            tc_fence_before_sync();
-            mbar_arrive(&ctl->acc_free1);
-            mbar_arrive(&ctl->parked);
-            __syncwarp();
-            if (lane == 0) atomicAdd(&ctl->o_done, 1);
-            PT_MARK(3)
-            PT_STAMP(status, 15, tid == kWarpE3 * 32 && it == 16)
-            // ---- d_f completed from the parked values, each thread its own 32 rows, once both halves' sums and R
-            // of the chunk are there
-            mbar_wait(&ctl->r_ready[it & 1], (it >> 1) & 1, abort_flag);
-            mbar_wait(&ctl->parked, it & 1, abort_flag);
-            tc_fence_after_sync();
-            {
-                const float K = rr[(it & 1) * 128 + krow] + xa[krow] + xe[krow];
-                __nv_bfloat16 *df_g = d_f + crow0 * kD + krow;
-                // the thread's 64 parked values in two reads (the pass is on the chunk's critical chain)
-                if (!kRagged || n_valid == kC) {
-                    uint32_t uu[32], rf[32];
-                    tmem_ld32(tl + kColDQ + 32 * half, uu);
-                    tmem_ld32(tl + kColDKi + 32 * half, rf);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        df_g[(size_t)(32 * half + j) * kD] =
-                            __float2bfloat16_rn(fmaf(K, __uint_as_float(rf[j]), __uint_as_float(uu[j])));
+                    for (int r = max(n_valid, 32 * half); r < 32 * half + 32; ++r) {
+                        oraw[r * kD + krow] = 0u;
+                        fraw[r * kD + krow] = kEnc ? 0x8000u : 0x3F80u;
+                    }
+                    if (half) phase_main<true, true, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
+                    else      phase_main<false, true, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
+                    fence_proxy_async_smem();                        // the rows written here, before the tiles' next load
                 } else {
-#pragma unroll 1
-                    for (int t0 = 32 * half; t0 < 32 * half + 32; t0 += 4) {
-                        uint32_t uu[4], rf[4];
-                        tmem_ld4(tl + kColDQ + t0, uu);
-                        tmem_ld4(tl + kColDKi + t0, rf);
+                    if (half) phase_main<true, false, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
+                    else      phase_main<false, false, kEnc>(tl, oraw, fraw, krow, do_g, n_valid, asum, esum);
+                }
+                mbar_arrive(&ctl->raw_read);
+                if (half) xa[krow] = asum; else xe[krow] = esum;
+                tmem_wait_st();
+                tc_fence_before_sync();
+                mbar_arrive(&ctl->acc_free1);
+                mbar_arrive(&ctl->parked);
+                __syncwarp();
+                if (lane == 0) atomicAdd(&ctl->o_done, 1);
+                PT_MARK(3)
+                PT_STAMP(status, 15, tid == kWarpE3 * 32 && it == 16)
+                // ---- d_f completed from the parked values, each thread its own 32 rows, once both halves' sums and R
+                // of the chunk are there
+                mbar_wait(&ctl->r_ready[it & 1], (it >> 1) & 1, abort_flag);
+                mbar_wait(&ctl->parked, it & 1, abort_flag);
+                tc_fence_after_sync();
+                {
+                    const float K = rr[(it & 1) * 128 + krow] + xa[krow] + xe[krow];
+                    __nv_bfloat16 *df_g = d_f + crow0 * kD + krow;
+                    // the thread's 64 parked values in two reads (the pass is on the chunk's critical chain)
+                    if (!kRagged || n_valid == kC) {
+                        uint32_t uu[32], rf[32];
+                        tmem_ld32(tl + kColDQ + 32 * half, uu);
+                        tmem_ld32(tl + kColDKi + 32 * half, rf);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (t0 + j < n_valid)
-                                df_g[(size_t)(t0 + j) * kD] =
-                                    __float2bfloat16_rn(fmaf(K, __uint_as_float(rf[j]), __uint_as_float(uu[j])));
+                        for (int j = 0; j < 32; ++j)
+                            df_g[(size_t)(32 * half + j) * kD] =
+                                __float2bfloat16_rn(fmaf(K, __uint_as_float(rf[j]), __uint_as_float(uu[j])));
+                    } else {
+#pragma unroll 1
+                        for (int t0 = 32 * half; t0 < 32 * half + 32; t0 += 4) {
+                            uint32_t uu[4], rf[4];
+                            tmem_ld4(tl + kColDQ + t0, uu);
+                            tmem_ld4(tl + kColDKi + t0, rf);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                if (t0 + j < n_valid)
+                                    df_g[(size_t)(t0 + j) * kD] =
+                                        __float2bfloat16_rn(fmaf(K, __uint_as_float(rf[j]), __uint_as_float(uu[j])));
+                        }
                     }
                 }
+                tc_fence_before_sync();
+                mbar_arrive(&ctl->acc_free2);
+                PT_MARK(4)
             }
-            tc_fence_before_sync();
-            mbar_arrive(&ctl->acc_free2);
-            PT_MARK(4)
         }
         PT_DUMP(status, 7, 5, tid == kWarpE3 * 32)
     } else if (warp < kWarpLoad) {
         // ================= O: causal masks, d_i =================
         const uint32_t tl = tmem + lane_base;
         PT_DECL
-        for (int it = 0; it < NC; ++it) {
-            const int c = NC - 1 - it;
-            const int n_valid = kRagged ? min(kC, N - c * kC) : kC;
-            const size_t crow0 = grow0 + (size_t)c * kC;
-            // ---- tril(A), tril(dA) -> operand slabs: rows of A sit in lanes 0..63, rows of dA in lanes 64..127, a
-            // warp converts its 32 rows.  The previous chunk's products have read the slabs: this role waited for
-            // them before that chunk's d_i.
-            mbar_wait(&ctl->barX, it & 1, abort_flag);
-            tc_fence_after_sync();
+        int it = 0;
+        Item im;
+        for (int k = 0; next_item<kPersist>(&ctl->ring, k, abort_flag, first, im); ++k) {
+            const size_t grow0 = (size_t)im.plane * wk.N + im.row0;     // first row of the item in the [planes * rows][128] view
+            for (int c = (im.n + kC - 1) / kC - 1; c >= 0; --c, ++it) {
+                const int n_valid = kRagged ? min(kC, im.n - c * kC) : kC;
+                const size_t crow0 = grow0 + c * kC;
+                // ---- tril(A), tril(dA) -> operand slabs: rows of A sit in lanes 0..63, rows of dA in lanes 64..127, a
+                // warp converts its 32 rows.  The previous chunk's products have read the slabs: this role waited for
+                // them before that chunk's d_i.
+                mbar_wait(&ctl->barX, it & 1, abort_flag);
+                tc_fence_after_sync();
 #pragma unroll 1
-            for (int hh = 0; hh < 2; ++hh)
-                tril_row_block(tl + (sub < 2 ? kColA : kColDA) + 32 * hh, sub < 2 ? pbuf : dpbuf, krow & 63, hh);
-            fence_proxy_async_smem();
-            tc_fence_before_sync();
-            mbar_arrive(&ctl->pd_ready);
-            mbar_wait(&ctl->barY2, it & 1, abort_flag);
-            PT_MARK(0)
-            PT_STAMP(status, 16, tid == kWarpO * 32 && it == 16)
-            tc_fence_after_sync();
-            // d_i = dV: lane = value dimension, columns = local times
-            __nv_bfloat16 *di_g = d_i + crow0 * kD + krow;
-            if (!kRagged || n_valid == kC) {
+                for (int hh = 0; hh < 2; ++hh)
+                    tril_row_block(tl + (sub < 2 ? kColA : kColDA) + 32 * hh, sub < 2 ? pbuf : dpbuf, krow & 63, hh);
+                fence_proxy_async_smem();
+                tc_fence_before_sync();
+                mbar_arrive(&ctl->pd_ready);
+                mbar_wait(&ctl->barY2, it & 1, abort_flag);
+                PT_MARK(0)
+                PT_STAMP(status, 16, tid == kWarpO * 32 && it == 16)
+                tc_fence_after_sync();
+                // d_i = dV: lane = value dimension, columns = local times
+                __nv_bfloat16 *di_g = d_i + crow0 * kD + krow;
+                if (!kRagged || n_valid == kC) {
 #pragma unroll 1
-                for (int b = 0; b < 8; ++b) {
-                    uint32_t r[8];
-                    tmem_ld8(tl + kColDV + 8 * b, r);
-                    tmem_wait_ld();
+                    for (int b = 0; b < 8; ++b) {
+                        uint32_t r[8];
+                        tmem_ld8(tl + kColDV + 8 * b, r);
+                        tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) di_g[(size_t)(8 * b + j) * kD] = __float2bfloat16_rn(__uint_as_float(r[j]));
-                }
-            } else {
+                        for (int j = 0; j < 8; ++j) di_g[(size_t)(8 * b + j) * kD] = __float2bfloat16_rn(__uint_as_float(r[j]));
+                    }
+                } else {
 #pragma unroll 1
-                for (int b = 0; b < 8; ++b) {
-                    uint32_t r[8];
-                    tmem_ld8(tl + kColDV + 8 * b, r);
-                    tmem_wait_ld();
+                    for (int b = 0; b < 8; ++b) {
+                        uint32_t r[8];
+                        tmem_ld8(tl + kColDV + 8 * b, r);
+                        tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        if (8 * b + j < n_valid) di_g[(size_t)(8 * b + j) * kD] = __float2bfloat16_rn(__uint_as_float(r[j]));
+                        for (int j = 0; j < 8; ++j)
+                            if (8 * b + j < n_valid) di_g[(size_t)(8 * b + j) * kD] = __float2bfloat16_rn(__uint_as_float(r[j]));
+                    }
                 }
+                tc_fence_before_sync();
+                mbar_arrive(&ctl->acc_freeV);
+                PT_MARK(1)
+                PT_STAMP(status, 17, tid == kWarpO * 32 && it == 16)
             }
-            tc_fence_before_sync();
-            mbar_arrive(&ctl->acc_freeV);
-            PT_MARK(1)
-            PT_STAMP(status, 17, tid == kWarpO * 32 && it == 16)
         }
         PT_DUMP(status, 11, 4, tid == kWarpO * 32)
     } else if (warp == kWarpLoad) {
         // ================= L: TMA loads =================
         int n_stage = 0, n_v = 0, n_state = 0, n_raw = 0;       // fills asked for so far, per buffer
-        auto issue_stage = [&](int it) {
-            n_stage = it + 1;
-            const int s = it % kStages, c = NC - 1 - it;
+        struct Pos { int plane, row, slot; bool ok; };          // a chunk
+        // The stage loads lead: they walk the items, take the next one as they get to the end of the current one, and
+        // the other buffers' loads follow a chunk behind.
+        Item im = first;
+        int k = 0, c = (im.n + kC - 1) / kC;
+        bool asked = false, ask_done = false;
+        auto advance = [&]() -> Pos {
+            while (im.id >= 0) {
+                if (kPersist && c <= 2 && !ask_done) {          // two chunks ahead: the answer takes about a microsecond
+                    asked = ring_ask(&ctl->ring, k + 1, &ctl->exact_flag, abort_flag);
+                    ask_done = true;
+                }
+                if (c > 0) {
+                    --c;
+                    return Pos{im.plane, im.row0 + c * kC, im.slot0 + c, true};
+                }
+                if (!kPersist) break;
+                im = warp_uniform(*ring_take<kRagged, true>(&ctl->ring, ++k, asked, wk, status, abort_flag));
+                c = (im.n + kC - 1) / kC;
+                asked = ask_done = false;
+            }
+            return Pos{0, 0, 0, false};
+        };
+        auto issue_stage = [&](const Pos &p) {
+            const int s = n_stage++ % kStages;
             uint8_t *st = smem + s * kStageBytes;
             mbar_arrive_expect_tx(&ctl->full[s], kStageBytes);
             for (int b = 0; b < 2; ++b) {
-                tma_load_3d(st + kOffQ + b * kSS, &map_o, &ctl->full[s], 64 * b, row0 + c * kC, zu);
-                tma_load_3d(st + kOffK + b * kSlab, &map_f, &ctl->full[s], 64 * b, row0 + c * kC, zu);
+                tma_load_3d(st + kOffQ + b * kSS, &map_o, &ctl->full[s], 64 * b, p.row, p.plane);
+                tma_load_3d(st + kOffK + b * kSlab, &map_f, &ctl->full[s], 64 * b, p.row, p.plane);
             }
             for (int b = 0; b < 2; ++b)
-                tma_load_3d(st + kOffG + b * kSS, &map_dy, &ctl->full[s], 64 * b, row0 + c * kC, zu);
+                tma_load_3d(st + kOffG + b * kSS, &map_dy, &ctl->full[s], 64 * b, p.row, p.plane);
         };
-        auto issue_v = [&](int it) {
-            n_v = it + 1;
-            const int c = NC - 1 - it;
+        auto issue_v = [&](const Pos &p) {
+            ++n_v;
             mbar_arrive_expect_tx(&ctl->vfull, kTile);
-            for (int b = 0; b < 2; ++b) tma_load_3d(vbuf + b * kSlab, &map_i, &ctl->vfull, 64 * b, row0 + c * kC, zu);
+            for (int b = 0; b < 2; ++b) tma_load_3d(vbuf + b * kSlab, &map_i, &ctl->vfull, 64 * b, p.row, p.plane);
         };
-        auto issue_raw = [&](int it) {
-            n_raw = it + 1;
-            const int c = NC - 1 - it;
+        auto issue_raw = [&](const Pos &p) {
+            ++n_raw;
             mbar_arrive_expect_tx(&ctl->rawfull, 2 * kTile);
-            tma_load_3d(smem + kOffRawO, &map_o_raw, &ctl->rawfull, 0, row0 + c * kC, zu);
-            tma_load_3d(smem + kOffRawF, &map_f_raw, &ctl->rawfull, 0, row0 + c * kC, zu);
+            tma_load_3d(smem + kOffRawO, &map_o_raw, &ctl->rawfull, 0, p.row, p.plane);
+            tma_load_3d(smem + kOffRawF, &map_f_raw, &ctl->rawfull, 0, p.row, p.plane);
         };
-        auto issue_state = [&](int it) {
-            n_state = it + 1;
-            const int c = NC - 1 - it;
+        auto issue_state = [&](const Pos &p) {
+            ++n_state;
             mbar_arrive_expect_tx(&ctl->sfull, kStateTile);
             for (int b = 0; b < 2; ++b)
-                tma_load_3d(sbuf + b * kStateSlab, &map_saved, &ctl->sfull, 64 * b, 0, (int)(slot0 + c));
+                tma_load_3d(sbuf + b * kStateSlab, &map_saved, &ctl->sfull, 64 * b, 0, p.slot);
         };
-        issue_stage(0);
-        issue_v(0);
-        issue_state(0);
-        issue_raw(0);
-        if (NC > 1) issue_stage(1);
-        // Every buffer is refilled as soon as its last reader of chunk `it` is done; the waits below are in
-        // the order in which those readers finish.
+        // Every buffer is refilled as soon as its last reader of the previous chunk is done; the waits below are in
+        // the order in which those readers finish.  Pass `it` loads v, S' and the raw tiles of chunk `it`, and the stage of
+        // chunk it + 1 (pass 0 also its own stage).
         // A barrier must never be armed twice within one phase.  Normally a buffer's previous fill has long been
         // consumed when its readers report; on the time-out exit those waits return at once, so before every
         // refill the previous fill is waited for explicitly (one poll that succeeds at once in normal running).
-        for (int it = 0; it + 1 < NC; ++it) {
-            mbar_wait(&ctl->barX, it & 1, abort_flag);           // dA = dY V^T ...
-            mbar_wait(&ctl->barY1, it & 1, abort_flag);          // ... and dKs_inter^T = dS'' V^T have read v
-            mbar_wait_drain(&ctl->vfull, it & 1, 20000000ull);
-            issue_v(it + 1);
-            mbar_wait(&ctl->r_ready[it & 1], (it >> 1) & 1, abort_flag);   // R has read S' ...
-            mbar_wait(&ctl->barY2, it & 1, abort_flag);          // ... and so have the chunk's products;
-            mbar_wait_drain(&ctl->sfull, it & 1, 20000000ull);
-            issue_state(it + 1);
-            if (it + 2 < NC) {                                   // o, f, dy of the stage are free as well
-                mbar_wait_drain(&ctl->full[it % kStages], (it / kStages) & 1, 20000000ull);
-                issue_stage(it + 2);
+        Pos next = advance();
+        if (next.ok) issue_stage(next);
+        for (int it = 0; next.ok; ++it) {
+            if (it > 0) {
+                mbar_wait(&ctl->barX, (it - 1) & 1, abort_flag);     // dA = dY V^T ...
+                mbar_wait(&ctl->barY1, (it - 1) & 1, abort_flag);    // ... and dKs_inter^T = dS'' V^T have read v
+                mbar_wait_drain(&ctl->vfull, (it - 1) & 1, 20000000ull);
             }
-            PT_STAMP(status, 0, it == 14) PT_STAMP(status, 21, it == 16) PT_STAMP(status, 22, it == 15)
-            mbar_wait(&ctl->raw_read, it & 1, abort_flag);       // the output warps are done with raw o, f
-            mbar_wait_drain(&ctl->rawfull, it & 1, 20000000ull);
-            issue_raw(it + 1);
+            issue_v(next);
+            const Pos after = advance();
+            if (it > 0) {
+                mbar_wait(&ctl->r_ready[(it - 1) & 1], ((it - 1) >> 1) & 1, abort_flag);   // R has read S' ...
+                mbar_wait(&ctl->barY2, (it - 1) & 1, abort_flag);    // ... and so have the chunk's products;
+                mbar_wait_drain(&ctl->sfull, (it - 1) & 1, 20000000ull);
+            }
+            issue_state(next);
+            if (after.ok) {                                          // o, f, dy of the stage are free as well
+                if (it > 0) mbar_wait_drain(&ctl->full[(it - 1) % kStages], ((it - 1) / kStages) & 1, 20000000ull);
+                issue_stage(after);
+            }
+            if (it > 0) {
+                mbar_wait(&ctl->raw_read, (it - 1) & 1, abort_flag); // the output warps are done with raw o, f
+                mbar_wait_drain(&ctl->rawfull, (it - 1) & 1, 20000000ull);
+            }
+            issue_raw(next);
+            next = after;
         }
         ctl->l_stage = n_stage; ctl->l_v = n_v; ctl->l_state = n_state; ctl->l_raw = n_raw;
     } else {
@@ -681,100 +719,112 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         auto kmaj_s = [](int kk) { return (uint64_t)(((kk >> 2) * kStateSlab + (kk & 3) * 32) >> 4); };   // [128][128] tile
         PT_DECL
         if (warp == kWarpMmaX) {
-            for (int it = 0; it < NC; ++it) {
-                const int s = it % kStages;
-                const uint64_t so = (uint64_t)s * (kStageBytes >> 4);
-                const uint64_t dqk = dqk0 + so, dqm = dqm0 + so, dfk = dfk0 + so, dgm = dgm0 + so;
-                mbar_wait(&ctl->full[s], (it / kStages) & 1, abort_flag);
-                mbar_wait(&ctl->t_done[s], (it / kStages) & 1, abort_flag);
-                PT_MARK(0)
-                mbar_wait(&ctl->m_done, it & 1, abort_flag);          // dS'' in TMEM
-                if (it > 0) mbar_wait(&ctl->pd_ready, (it - 1) & 1, abort_flag);   // A, dA of the previous chunk read out
-                mbar_wait(&ctl->vfull, it & 1, abort_flag);
-                PT_MARK(1)
-                PT_STAMP(status, 3, it == 16)
-                tc_fence_after_sync();
+            int it = 0;
+            Item im;
+            for (int k = 0; next_item<kPersist>(&ctl->ring, k, abort_flag, first, im); ++k) {
+                for (int left = im.n; left > 0; left -= kC, ++it) {
+                    const int s = it % kStages;
+                    const uint64_t so = (uint64_t)s * (kStageBytes >> 4);
+                    const uint64_t dqk = dqk0 + so, dqm = dqm0 + so, dfk = dfk0 + so, dgm = dgm0 + so;
+                    mbar_wait(&ctl->full[s], (it / kStages) & 1, abort_flag);
+                    mbar_wait(&ctl->t_done[s], (it / kStages) & 1, abort_flag);
+                    PT_MARK(0)
+                    mbar_wait(&ctl->m_done, it & 1, abort_flag);          // dS'' in TMEM
+                    if (it > 0) mbar_wait(&ctl->pd_ready, (it - 1) & 1, abort_flag);   // A, dA of the previous chunk read out
+                    mbar_wait(&ctl->vfull, it & 1, abort_flag);
+                    PT_MARK(1)
+                    PT_STAMP(status, 3, it == 16)
+                    tc_fence_after_sync();
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)              // dS' = dS'' + Qs^T dY
-                    mma_bf16_ss(tmem + kColDS, dqm + (uint64_t)(kk * 128), dgm + (uint64_t)(kk * 128), idDS, 1);
-                {
-                    // (Qs; dY) as one 128-row operand: (Qs; dY) Ks^T has A in lanes 0..63 and (Qs; dY) V^T has dA
-                    // in lanes 64..127 (the other halves are not used), so every lane carries a row to mask
+                    for (int kk = 0; kk < 4; ++kk)              // dS' = dS'' + Qs^T dY
+                        mma_bf16_ss(tmem + kColDS, dqm + (uint64_t)(kk * 128), dgm + (uint64_t)(kk * 128), idDS, 1);
+                    {
+                        // (Qs; dY) as one 128-row operand: (Qs; dY) Ks^T has A in lanes 0..63 and (Qs; dY) V^T has dA
+                        // in lanes 64..127 (the other halves are not used), so every lane carries a row to mask
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        mma_bf16_ss(tmem + kColA, dqk + kmaj_i(kk), dfk + kmaj(kk), idKK, kk > 0);
+                        for (int kk = 0; kk < 8; ++kk)
+                            mma_bf16_ss(tmem + kColA, dqk + kmaj_i(kk), dfk + kmaj(kk), idKK, kk > 0);
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        mma_bf16_ss(tmem + kColDA, dqk + kmaj_i(kk), dvk + kmaj(kk), idKK, kk > 0);
-                    mma_commit(&ctl->barX);
+                        for (int kk = 0; kk < 8; ++kk)
+                            mma_bf16_ss(tmem + kColDA, dqk + kmaj_i(kk), dvk + kmaj(kk), idKK, kk > 0);
+                        mma_commit(&ctl->barX);
+                    }
+                    PT_MARK(2)
+                    PT_STAMP(status, 4, it == 16)
                 }
-                PT_MARK(2)
-                PT_STAMP(status, 4, it == 16)
             }
             PT_DUMP(status, 15, 3, true)
         } else if (warp == kWarpMmaY1) {
-            for (int it = 0; it < NC; ++it) {
-                const int s = it % kStages;
-                const uint64_t so = (uint64_t)s * (kStageBytes >> 4);
-                const uint64_t dfk = dfk0 + so;
-                mbar_wait(&ctl->full[s], (it / kStages) & 1, abort_flag);
-                mbar_wait(&ctl->t_done[s], (it / kStages) & 1, abort_flag);
-                mbar_wait(&ctl->m_done, it & 1, abort_flag);          // bf16 dS'' in shared memory
-                PT_MARK(0)
-                // dV^T first: its accumulator is free as soon as d_i of the previous chunk is out, long before the
-                // output warps have finished with dKs_inter^T
-                if (it > 0) mbar_wait(&ctl->acc_freeV, (it - 1) & 1, abort_flag);
-                tc_fence_after_sync();
+            int it = 0;
+            Item im;
+            for (int k = 0; next_item<kPersist>(&ctl->ring, k, abort_flag, first, im); ++k) {
+                for (int left = im.n; left > 0; left -= kC, ++it) {
+                    const int s = it % kStages;
+                    const uint64_t so = (uint64_t)s * (kStageBytes >> 4);
+                    const uint64_t dfk = dfk0 + so;
+                    mbar_wait(&ctl->full[s], (it / kStages) & 1, abort_flag);
+                    mbar_wait(&ctl->t_done[s], (it / kStages) & 1, abort_flag);
+                    mbar_wait(&ctl->m_done, it & 1, abort_flag);          // bf16 dS'' in shared memory
+                    PT_MARK(0)
+                    // dV^T first: its accumulator is free as soon as d_i of the previous chunk is out, long before the
+                    // output warps have finished with dKs_inter^T
+                    if (it > 0) mbar_wait(&ctl->acc_freeV, (it - 1) & 1, abort_flag);
+                    tc_fence_after_sync();
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)              // dV^T = dS''^T Ks^T
-                    mma_bf16_ss(tmem + kColDV, ddsm + (uint64_t)(kk * 128), dfk + kmaj(kk), idMK, kk > 0);
-                mma_commit(&ctl->barY1a);
-                mbar_wait(&ctl->vfull, it & 1, abort_flag);
-                if (it > 0) mbar_wait(&ctl->acc_free1, (it - 1) & 1, abort_flag);
-                PT_MARK(1)
-                PT_STAMP(status, 10, it == 16)
-                tc_fence_after_sync();
+                    for (int kk = 0; kk < 8; ++kk)              // dV^T = dS''^T Ks^T
+                        mma_bf16_ss(tmem + kColDV, ddsm + (uint64_t)(kk * 128), dfk + kmaj(kk), idMK, kk > 0);
+                    mma_commit(&ctl->barY1a);
+                    mbar_wait(&ctl->vfull, it & 1, abort_flag);
+                    if (it > 0) mbar_wait(&ctl->acc_free1, (it - 1) & 1, abort_flag);
+                    PT_MARK(1)
+                    PT_STAMP(status, 10, it == 16)
+                    tc_fence_after_sync();
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)              // dKs_inter^T = dS'' V^T
-                    mma_bf16_ss(tmem + kColDKx, ddsk + kmaj_s(kk), dvk + kmaj(kk), idKK, kk > 0);
-                mma_commit(&ctl->barY1);
-                PT_MARK(2)
+                    for (int kk = 0; kk < 8; ++kk)              // dKs_inter^T = dS'' V^T
+                        mma_bf16_ss(tmem + kColDKx, ddsk + kmaj_s(kk), dvk + kmaj(kk), idKK, kk > 0);
+                    mma_commit(&ctl->barY1);
+                    PT_MARK(2)
+                }
             }
             PT_DUMP(status, 18, 3, true)
         } else {
-            for (int it = 0; it < NC; ++it) {
-                const int s = it % kStages;
-                const uint64_t so = (uint64_t)s * (kStageBytes >> 4);
-                const uint64_t dqm = dqm0 + so, dfm = dfm0 + so, dgk = dgk0 + so, dgm = dgm0 + so;
-                mbar_wait(&ctl->pd_ready, it & 1, abort_flag);   // tril(A), tril(dA); implies X and T of the chunk
-                mbar_wait(&ctl->barY1a, it & 1, abort_flag);          // dV^T += ... must follow dV^T = ...
-                PT_MARK(0)
-                PT_STAMP(status, 11, it == 16)
-                tc_fence_after_sync();
-                // dV^T first: it does not touch the columns that still hold the previous chunk's parked values
+            int it = 0;
+            Item im;
+            for (int k = 0; next_item<kPersist>(&ctl->ring, k, abort_flag, first, im); ++k) {
+                for (int left = im.n; left > 0; left -= kC, ++it) {
+                    const int s = it % kStages;
+                    const uint64_t so = (uint64_t)s * (kStageBytes >> 4);
+                    const uint64_t dqm = dqm0 + so, dfm = dfm0 + so, dgk = dgk0 + so, dgm = dgm0 + so;
+                    mbar_wait(&ctl->pd_ready, it & 1, abort_flag);   // tril(A), tril(dA); implies X and T of the chunk
+                    mbar_wait(&ctl->barY1a, it & 1, abort_flag);          // dV^T += ... must follow dV^T = ...
+                    PT_MARK(0)
+                    PT_STAMP(status, 11, it == 16)
+                    tc_fence_after_sync();
+                    // dV^T first: it does not touch the columns that still hold the previous chunk's parked values
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)              // dV^T += dY^T A
-                    mma_bf16_ss(tmem + kColDV, dgm + (uint64_t)(kk * 128), dpm + (uint64_t)(kk * 128), idMM, 1);
-                mbar_wait(&ctl->sfull, it & 1, abort_flag);
-                if (it > 0) mbar_wait(&ctl->acc_free2, (it - 1) & 1, abort_flag);
-                PT_MARK(1)
-                PT_STAMP(status, 12, it == 16)
-                tc_fence_after_sync();
+                    for (int kk = 0; kk < 4; ++kk)              // dV^T += dY^T A
+                        mma_bf16_ss(tmem + kColDV, dgm + (uint64_t)(kk * 128), dpm + (uint64_t)(kk * 128), idMM, 1);
+                    mbar_wait(&ctl->sfull, it & 1, abort_flag);
+                    if (it > 0) mbar_wait(&ctl->acc_free2, (it - 1) & 1, abort_flag);
+                    PT_MARK(1)
+                    PT_STAMP(status, 12, it == 16)
+                    tc_fence_after_sync();
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)              // dQs^T = Ks^T dA^T
-                    mma_bf16_ss(tmem + kColDQ, dfm + (uint64_t)(kk * 128), ddpk + (uint64_t)(kk * 2), idMK, kk > 0);
+                    for (int kk = 0; kk < 4; ++kk)              // dQs^T = Ks^T dA^T
+                        mma_bf16_ss(tmem + kColDQ, dfm + (uint64_t)(kk * 128), ddpk + (uint64_t)(kk * 2), idMK, kk > 0);
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)              //        + S' dY^T
-                    mma_bf16_ss(tmem + kColDQ, dsk + kmaj_s(kk), dgk + kmaj_i(kk), idKK, 1);
+                    for (int kk = 0; kk < 8; ++kk)              //        + S' dY^T
+                        mma_bf16_ss(tmem + kColDQ, dsk + kmaj_s(kk), dgk + kmaj_i(kk), idKK, 1);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)              // dKs_intra^T = Qs^T dA
-                    mma_bf16_ss(tmem + kColDKi, dqm + (uint64_t)(kk * 128), ddpm + (uint64_t)(kk * 128), idMM, kk > 0);
-                // barY2 stands for every product of the chunk: dKs_inter^T is another lane's, so wait for it first
-                // (it was issued when the output warps finished the previous chunk, well before this point)
-                mbar_wait(&ctl->barY1, it & 1, abort_flag);
-                mma_commit(&ctl->barY2);
-                PT_MARK(2)
-                PT_STAMP(status, 13, it == 16)
+                    for (int kk = 0; kk < 4; ++kk)              // dKs_intra^T = Qs^T dA
+                        mma_bf16_ss(tmem + kColDKi, dqm + (uint64_t)(kk * 128), ddpm + (uint64_t)(kk * 128), idMM, kk > 0);
+                    // barY2 stands for every product of the chunk: dKs_inter^T is another lane's, so wait for it first
+                    // (it was issued when the output warps finished the previous chunk, well before this point)
+                    mbar_wait(&ctl->barY1, it & 1, abort_flag);
+                    mma_commit(&ctl->barY2);
+                    PT_MARK(2)
+                    PT_STAMP(status, 13, it == 16)
+                }
             }
             PT_DUMP(status, 21, 3, true)
         }
@@ -788,6 +838,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         mbar_wait_drain(&ctl->drain, 0, 20000000ull);
         if (*abort_flag) {
             report_error(status, HGRN2_ERR_TIMEOUT, 2);
+            if (kPersist && ctl->ring.asked > 0) mbar_wait_drain(&ctl->ring.answered, (ctl->ring.asked - 1) & 1, 20000000ull);
             // tiles asked for but never consumed may still be on their way into this CTA's shared memory
             const int ns = ctl->l_stage, nv = ctl->l_v, nst = ctl->l_state, nr = ctl->l_raw;
             for (int s = 0; s < kStages; ++s)
@@ -800,219 +851,72 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 
-    // ---- exact path (see the forward kernel): the unit is redone from its inputs and its saved chunk states by the
-    // pairwise-safe fp32 routine; with several CTAs per unit the last one to finish does it.
-    if (ex.o == nullptr) return;
-    const int unit = kMultiCta ? u / ex.G : u;
-    if constexpr (kMultiCta) {
-        if (tid == 0) {
-            if (ctl->exact_flag) atomicOr(&ex.unit_flag[unit], 1);
-            __threadfence();
-            int go = 0;
-            if (atomicAdd(&ex.unit_count[unit], 1) == ex.G - 1) {
-                __threadfence();
-                go = atomicOr(&ex.unit_flag[unit], 0);
-            }
-            ctl->exact_flag = go;
-        }
-        __syncthreads();
+    // ---- exact path (see the forward kernel): flagged items are redone from their inputs, their saved chunk states and
+    // the gradient they started from by the pairwise-safe fp32 routine
+    if (ex.o == nullptr || !ctl->exact_flag || *abort_flag) return;
+    for (int j = 0; j < (kPersist ? 8 : 1); ++j) {
+        const int id = kPersist ? ctl->ring.flagged[j] - 1 : first.id;
+        if (id < 0) continue;
+        __syncthreads();                                             // the routine's shared memory is free
+        if (tid == 0) atomicAdd(&status->exact_units, 1);
+        const Item im = work_item<kRagged, true>(wk, id, malformed);
+        const size_t seq = ((size_t)im.plane * wk.N + im.row0) * kD, st = (size_t)im.unit * kD * kD;
+        alu::bwd_unit<__nv_bfloat16, __nv_bfloat16, kEnc ? alu::kGateEnc : alu::kGateIsF>(
+            reinterpret_cast<float *>(smem), ex.o + seq, ex.f + seq, ex.i + seq, ex.dy + seq,
+            im.chain >= 0 ? chain + (size_t)im.chain * kD * kD : (dSN ? dSN + st : nullptr),
+            ex.states + (size_t)im.slot0 * kD * kD, kC / kExactC, ex.scratch + (size_t)id * kD * kD, ex.d_o + seq,
+            ex.d_f + seq, ex.d_i + seq, dS0 != nullptr && im.last ? dS0 + st : nullptr, im.n, kD, kD, kExactC,
+            (im.n + kExactC - 1) / kExactC);
     }
-    if (!ctl->exact_flag || *abort_flag) return;
-    __syncthreads();                                               // every thread has read the flag: smem is reused now
-    if (tid == 0) atomicAdd(&status->exact_units, 1);
-    const bool packed = kRagged && pk.cu != nullptr;
-    const int n_unit = packed ? N : ex.N;                          // tokens of the whole unit
-    const size_t seq = packed ? grow0 * kD : (size_t)unit * ex.N * kD, st = (size_t)unit * kD * kD;
-    const size_t slot_u = packed ? slot0 : (size_t)unit * ((ex.N + kC - 1) / kC);
-    alu::bwd_unit<__nv_bfloat16, __nv_bfloat16, kEnc ? alu::kGateEnc : alu::kGateIsF>(
-        reinterpret_cast<float *>(smem), ex.o + seq, ex.f + seq, ex.i + seq, ex.dy + seq, ex.dSN ? ex.dSN + st : nullptr,
-        ex.states + slot_u * kD * kD, kC / kExactC, ex.scratch + st, ex.d_o + seq, ex.d_f + seq,
-        ex.d_i + seq, ex.dS0 ? ex.dS0 + st : nullptr, n_unit, kD, kD, kExactC, (n_unit + kExactC - 1) / kExactC);
 }
 
 }  // namespace
 
-// ---- sequences split into segments (see chunk_tc_fwd.cu) ----------------------------------------------
-// Chains the segments in reverse: dS_end[r] = gradient w.r.t. the state at the end of segment r.
-// seg_major: see seg_combine_kernel.
-__global__ void seg_combine_bwd_kernel(const float *__restrict__ dSN, const float *__restrict__ G_loc,
-                                       const float *__restrict__ lam, float *__restrict__ dS_end,
-                                       float *__restrict__ dS0, int G, int *__restrict__ unit_flag,
-                                       int *__restrict__ unit_count, int units, int seg_major, size_t U, int H)
-{
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;      // element of [U][128][128]
-    if (e < (size_t)units) {             // exact-path bookkeeping of the full pass that follows starts at zero
-        unit_flag[e] = 0;
-        unit_count[e] = 0;
-    }
-    const size_t u = e / (kD * kD);
-    const int k = (int)((e / kD) % kD);
-    const size_t kv = e % (kD * kD);
-    float D = dSN ? dSN[e] : 0.f;
-    for (int r = G - 1; r >= 0; --r) {
-        const size_t ur = seg_index(seg_major, u, r, G, U, H);
-        dS_end[ur * kD * kD + kv] = D;
-        D = fmaf(lam[ur * kD + k], D, G_loc[ur * kD * kD + kv]);
-    }
-    if (dS0) dS0[e] = D;
-}
+// Several items per CTA (kPersist) where they are short: 4736 units of 64 tokens 247 instead of 341 us, 2368 of 128 211 / 246,
+// 1184 of 256 182 / 189, 789 of 384 182 / 186, but 592 of 512 171 / 162 and 296 of 1024 164 / 146: that instantiation's
+// larger code takes up to a tenth more per chunk.
+constexpr uint64_t kPersistChunks = 6;
 
-
-static ExactArgs exact_args(const SeqArgs &a, int N_unit, int G, int *unit_flag, int *unit_count)
+cudaError_t launch_tc_bwd(const SeqArgs &a0)
 {
+    SeqArgs a = a0;
+    const TcWork t = tc_work(a);
+    if (t.items > 0x7fffffffull) return cudaErrorInvalidConfiguration;
+    cudaError_t err;
+    if (t.wk.G > 1) {
+        // sequences cut into segments (chunk_tc_fwd.cu), mirrored: what every segment but the first adds to the state
+        // gradient (it holds for every f), chained in reverse
+        err = launch_tc_state(true, a.o, a.f, a.dy, t, a.gate_enc, a.status, a.clear_status, a.start_aborted, a.stream);
+        if (err != cudaSuccess) return err;
+        if ((err = launch_seg_chain(true, t, a.dSN, a.stream)) != cudaSuccess) return err;
+        a.clear_status = false;
+    }
+    CUtensorMap mo, mf, mi, mg, ms, mor, mfr;
+    if (!make_map(&mo, a.o, t.planes, a.N, kC) || !make_map(&mf, a.f, t.planes, a.N, kC) || !make_map(&mi, a.i, t.planes, a.N, kC) ||
+        !make_map(&mg, a.dy, t.planes, a.N, kC) || !make_map(&ms, a.states, t.slots, kD, kD) ||
+        !make_map_plain(&mor, a.o, t.planes, a.N, kC) || !make_map_plain(&mfr, a.f, t.planes, a.N, kC))
+        return cudaErrorInvalidValue;
+    const bool ragged = a.N % kC != 0 || a.cu != nullptr, persist = t.items > (uint64_t)sm_count() && t.chunks <= kPersistChunks;
+    auto kernel = a.gate_enc ? (ragged ? (persist ? tc_bwd_kernel<true, true, true> : tc_bwd_kernel<true, true, false>)
+                                       : (persist ? tc_bwd_kernel<false, true, true> : tc_bwd_kernel<false, true, false>))
+                             : (ragged ? (persist ? tc_bwd_kernel<true, false, true> : tc_bwd_kernel<true, false, false>)
+                                       : (persist ? tc_bwd_kernel<false, false, true> : tc_bwd_kernel<false, false, false>));
+    if ((err = ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), kSmemBytes)) != cudaSuccess) return err;
     ExactArgs ex;
     ex.o = static_cast<const __nv_bfloat16 *>(a.o);
     ex.f = static_cast<const __nv_bfloat16 *>(a.f);
     ex.i = static_cast<const __nv_bfloat16 *>(a.i);
     ex.dy = static_cast<const __nv_bfloat16 *>(a.dy);
-    ex.dSN = a.dSN;
     ex.d_o = static_cast<__nv_bfloat16 *>(a.d_o);
     ex.d_f = static_cast<__nv_bfloat16 *>(a.d_f);
     ex.d_i = static_cast<__nv_bfloat16 *>(a.d_i);
-    ex.dS0 = a.dS0;
     ex.states = reinterpret_cast<__nv_bfloat16 *>(a.states);
     ex.scratch = a.exact_scratch;
-    ex.N = N_unit;
-    ex.G = G;
-    ex.unit_flag = unit_flag;
-    ex.unit_count = unit_count;
-    return ex;
-}
-
-PackedArgs tc_packed_args(const SeqArgs &a, int G);
-
-// U CTAs; ordinary layout: U planes of N rows; packed batch (pk.cu set): pk.H planes of N rows shared by the U units.
-static cudaError_t launch_bwd_once(const SeqArgs &a, uint64_t U, int N, int NC, const float *dSN, float *dS0,
-                                   bool clear, const ExactArgs &ex, const PackedArgs &pk = PackedArgs{})
-{
-    CUtensorMap mo, mf, mi, mg, ms, mor, mfr;
-    const uint64_t planes = pk.cu ? (uint64_t)pk.H : U;
-    const uint64_t slots = pk.cu ? (uint64_t)pk.H * pk.slots_per_head : U * NC;
-    if (!make_map(&mo, a.o, planes, N, kC) || !make_map(&mf, a.f, planes, N, kC) || !make_map(&mi, a.i, planes, N, kC) ||
-        !make_map(&mg, a.dy, planes, N, kC) || !make_map(&ms, a.states, slots, kD, kD) ||
-        !make_map_plain(&mor, a.o, planes, N, kC) || !make_map_plain(&mfr, a.f, planes, N, kC))
-        return cudaErrorInvalidValue;
-    const bool ragged = N % kC != 0 || pk.cu != nullptr;
-    if (ex.o != nullptr && ex.G > 1 && ragged) return cudaErrorInvalidValue;      // segments are whole chunks
-    auto kernel = a.gate_enc ? (ragged ? tc_bwd_kernel<true, false, true>
-                                   : (ex.o != nullptr && ex.G > 1 ? tc_bwd_kernel<false, true, true>
-                                                                   : tc_bwd_kernel<false, false, true>))
-                         : (ragged ? tc_bwd_kernel<true, false, false>
-                                   : (ex.o != nullptr && ex.G > 1 ? tc_bwd_kernel<false, true, false>
-                                                                   : tc_bwd_kernel<false, false, false>));
-    cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), kSmemBytes);
-    if (err != cudaSuccess) return err;
-    kernel<<<(unsigned)U, kThreads, kSmemBytes, a.stream>>>(
-        mo, mf, mi, mg, ms, mor, mfr,
-        a.totals, dSN, static_cast<__nv_bfloat16 *>(a.d_o),
-        static_cast<__nv_bfloat16 *>(a.d_f), static_cast<__nv_bfloat16 *>(a.d_i), dS0, N, NC, a.status, clear ? 1 : 0, ex, pk, a.start_aborted);
+    kernel<<<(unsigned)t.items, kThreads, kSmemBytes, a.stream>>>(
+        mo, mf, mi, mg, ms, mor, mfr, a.totals, a.dSN, t.chain, static_cast<__nv_bfloat16 *>(a.d_o),
+        static_cast<__nv_bfloat16 *>(a.d_f), static_cast<__nv_bfloat16 *>(a.d_i), a.dS0, t.wk, a.status,
+        a.clear_status ? 1 : 0, ex, a.start_aborted);
     return cudaGetLastError();
-}
-
-cudaError_t launch_tc_bwd(const SeqArgs &a0)
-{
-    const uint64_t U = (uint64_t)a0.B * a0.H;
-    SeqArgs a = a0;
-    if (a.cu) {
-        // packed batch: one CTA per (sequence, head), every CTA reads its own rows from the offsets array
-        const int G = a.seg_scratch ? tc_packed_segments(U, a.N) : 1;
-        PackedArgs pk = tc_packed_args(a, G);
-        a.totals = reinterpret_cast<float *>(reinterpret_cast<char *>(a.states) +
-                                             (size_t)pk.H * pk.slots_per_head * kSavedStateBytes);
-        if (G <= 1)
-            return launch_bwd_once(a, U, a.N, 0, a.dSN, a.dS0, a.clear_status, exact_args(a, a.N, 1, nullptr, nullptr),
-                                   pk);
-        // few units: every sequence as G segments (see launch_tc_fwd)
-        const uint64_t CT = U * G;
-        char *base = static_cast<char *>(a.seg_scratch);
-        int *cu_seg = reinterpret_cast<int *>(base);
-        float *G_loc = reinterpret_cast<float *>(base + tc_packed_offsets_bytes(a.B, G));
-        float *dS_end = G_loc + CT * kD * kD;
-        float *lam = dS_end + CT * kD * kD;
-        launch_seg_offsets_packed(a.cu, a.B, G, cu_seg, a.stream);
-        cudaError_t err = cudaGetLastError();
-        if (err != cudaSuccess) return err;
-        pk.cu = cu_seg;
-        err = launch_tc_state_bwd(a.o, a.f, a.dy, (uint64_t)a.H, a.N, G_loc, lam, a.gate_enc, a.status, a.clear_status,
-                                  a.start_aborted, a.stream, cu_seg, a.B * G);
-        if (err != cudaSuccess) return err;
-        seg_combine_bwd_kernel<<<(unsigned)(U * kD * kD / 256), 256, 0, a.stream>>>(a.dSN, G_loc, lam, dS_end, a.dS0, G,
-                                                                                   nullptr, nullptr, 0, 2, (size_t)U, a.H);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
-        SeqArgs t = a;
-        t.dSN = dS_end;
-        t.dS0 = nullptr;
-        return launch_bwd_once(t, CT, a.N, 0, dS_end, nullptr, false, exact_args(t, a.N, 1, nullptr, nullptr), pk);
-    }
-    const RSegPlan rp = a.seg_scratch ? tc_rseg_plan(U, a.N, a.NC) : RSegPlan{U, 0, 1, 0};
-    if (rp.tail_units) {
-        // ragged segments (see launch_tc_fwd): state-gradient summaries per segment, chained in reverse, then the
-        // full pass per segment through the packed-batch geometry
-        const int G = rp.G;
-        const uint64_t Ut = rp.tail_units, CT = Ut * G;
-        const size_t spp = (size_t)(a.N / kC + G + 1);
-        a.totals = reinterpret_cast<float *>(reinterpret_cast<char *>(a.states) +
-                                             ((size_t)rp.main_units * a.NC + (size_t)Ut * spp) * kSavedStateBytes);
-        cudaError_t err = cudaSuccess;
-        bool clear = a.clear_status;
-        if (rp.main_units) {
-            const SeqArgs m = tc_slice_units(a, 0, rp.main_units);
-            err = launch_bwd_once(m, rp.main_units, a.N, a.NC, m.dSN, m.dS0, clear, exact_args(m, a.N, 1, nullptr, nullptr));
-            if (err != cudaSuccess) return err;
-            clear = false;
-        }
-        SeqArgs t = tc_slice_units(a, rp.main_units, Ut);
-        char *base = static_cast<char *>(a.seg_scratch);
-        int *cu = reinterpret_cast<int *>(base);
-        float *G_loc = reinterpret_cast<float *>(base + kRSegOffsetsBytes);
-        float *dS_end = G_loc + CT * kD * kD;
-        float *lam = dS_end + CT * kD * kD;
-        launch_seg_offsets(cu, G, rp.Lc * kC, a.N, a.stream);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
-        PackedArgs pk;
-        pk.cu = cu;
-        pk.H = (int)Ut;
-        pk.slots_per_head = (int)spp;
-        err = launch_tc_state_bwd(t.o, t.f, t.dy, Ut, a.N, G_loc, lam, a.gate_enc, a.status, clear, a.start_aborted,
-                                  a.stream, cu, G);
-        if (err != cudaSuccess) return err;
-        seg_combine_bwd_kernel<<<(unsigned)(Ut * kD * kD / 256), 256, 0, a.stream>>>(t.dSN, G_loc, lam, dS_end, t.dS0, G,
-                                                                                    nullptr, nullptr, 0, 1, (size_t)Ut, 1);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
-        t.dSN = dS_end;
-        t.dS0 = nullptr;
-        return launch_bwd_once(t, CT, a.N, 0, dS_end, nullptr, false, exact_args(t, a.N, 1, nullptr, nullptr), pk);
-    }
-    a.totals = reinterpret_cast<float *>(reinterpret_cast<char *>(a.states) + U * a.NC * kSavedStateBytes);
-    const SegPlan plan = a.seg_scratch ? tc_seg_plan(U, a.N, a.NC) : SegPlan{U, 0, 1};
-    cudaError_t err = cudaSuccess;
-    bool clear = a.clear_status;                                  // for the first kernel launched only
-    if (plan.main_units) {
-        const SeqArgs m = tc_slice_units(a, 0, plan.main_units);
-        err = launch_bwd_once(m, plan.main_units, a.N, a.NC, m.dSN, m.dS0, clear,
-                              exact_args(m, a.N, 1, nullptr, nullptr));
-        if (err != cudaSuccess) return err;
-        clear = false;
-    }
-    if (plan.tail_units) {
-        const SeqArgs t = tc_slice_units(a, plan.main_units, plan.tail_units);
-        const uint64_t Ut = plan.tail_units;
-        const int G = plan.G;
-        // scratch: G_local [Ut*G][128][128], dS_end [Ut*G][128][128], Lambda [Ut*G][128]
-        float *G_loc = static_cast<float *>(a.seg_scratch);
-        float *dS_end = G_loc + Ut * G * kD * kD;
-        float *lam = dS_end + Ut * G * kD * kD;
-        int *unit_flag = reinterpret_cast<int *>(lam + Ut * G * kD), *unit_count = unit_flag + Ut;
-        // state-gradient contributions of the segments (chunk_tc_state.cu): they hold for every f
-        err = launch_tc_state_bwd(t.o, t.f, t.dy, Ut * G, a.N / G, G_loc, lam, a.gate_enc, a.status, clear, a.start_aborted, a.stream);
-        if (err != cudaSuccess) return err;
-        seg_combine_bwd_kernel<<<(unsigned)(Ut * kD * kD / 256), 256, 0, a.stream>>>(t.dSN, G_loc, lam, dS_end, t.dS0, G,
-                                                                                    unit_flag, unit_count, (int)Ut, 0, (size_t)Ut, 1);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
-        err = launch_bwd_once(t, Ut * G, a.N / G, a.NC / G, dS_end, nullptr, false,
-                              exact_args(t, a.N, G, unit_flag, unit_count));
-    }
-    return err;
 }
 
 }  // namespace hgrn2

@@ -21,9 +21,12 @@
 // at the end the T warps move the accumulator to global memory.  Every wait is bounded (tc_common.cuh).
 //
 // kRagged instantiations: the segment need not be a whole number of chunks (rows past its end act as the
-// neutral token f = 1, q = 0), and a CTA may take its rows from an offsets array: CTA u = b * planes + h then
-// covers rows [cu[b], cu[b + 1]) of plane h of the [planes][rows][128] tensors (sequences cut into segments of
-// unequal length, chunk_tc_fwd.cu).
+// neutral token f = 1, q = 0).
+//
+// One CTA per SM is paced by its four transform warps (1.7 k cycles per chunk, 4.8 TB/s over 128 CTAs); with more
+// segments than SMs two CTAs share an SM, with fewer stages each.
+#include <type_traits>
+
 #include "tc_chunk.cuh"
 
 namespace hgrn2 {
@@ -35,9 +38,8 @@ using namespace tc;
 constexpr int kTWarps = 4;
 constexpr int kWarpLoad = kTWarps, kWarpMma = kTWarps + 1;
 constexpr int kThreads = (kWarpMma + 1) * 32;
-constexpr int kStages = 4;
 
-template <bool kBwd> struct Geo {
+template <bool kBwd, int kStages> struct Geo {
     // stage layout: forward [f][v]; backward [o][f][dy].  X overwrites f (forward: X = k c) or o (backward: X = q c).
     static constexpr uint32_t kOffX = 0;
     static constexpr uint32_t kOffF = kBwd ? kTile : 0;
@@ -48,7 +50,7 @@ template <bool kBwd> struct Geo {
     static constexpr uint32_t kSmemBytes = kOffCtl + 256 + 1024;         // + alignment slack
 };
 
-struct Ctl {
+template <int kStages> struct Ctl {
     uint64_t full[kStages];      // TMA -> T
     uint64_t t_done[kStages];    // T -> M
     uint64_t empty[kStages];     // tcgen05.commit -> L: the chunk's products have read the stage
@@ -57,17 +59,31 @@ struct Ctl {
     int abort_flag;
     int l_issued;                // L: chunks asked for so far, for the abort epilogue
 };
-static_assert(sizeof(Ctl) <= 256, "control block");
+static_assert(sizeof(Ctl<4>) <= 256, "control block");
+
+// What a CTA summarises: `out` and lam take its result at index `at`.
+struct Span { int plane, row0, n; size_t at; };
+// spans == true: plane x whole.  Otherwise the cuts of w (tc_chunk.cuh): forward segments 0 .. G - 2, backward segments
+// 1 .. G - 1 of every cut unit, the result in the chain slot of the boundary behind (in front of) the segment.
+template <bool kBwd>
+__device__ __forceinline__ Span span_of(const WorkArgs &w, int x, bool spans, int cut, bool &malformed)
+{
+    if (spans) return Span{x, 0, w.N, (size_t)x};
+    const int r = x / cut + (kBwd ? 1 : 0), t = x % cut;
+    const Item it = work_item<true, kBwd>(w, w.cu ? ((t / w.H) * w.G + r) * w.H + t % w.H : w.main + r * cut + t, malformed);
+    // nothing chains behind a packed sequence's last segment
+    const int n = !kBwd && it.last ? 0 : it.n;
+    return Span{it.plane, it.row0, n, (size_t)t * (w.G - 1) + (kBwd ? r - 1 : r)};
+}
 
 // kEnc: the f tensor holds the signed gate encoding (see transform_half in tc_chunk.cuh).
-template <bool kBwd, bool kEnc, bool kRagged>
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool kBwd, bool kEnc, bool kRagged, int kStages>
+__global__ void __launch_bounds__(kThreads, kStages == 4 ? 1 : 2)
 tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__ CUtensorMap map_f,
-                const __grid_constant__ CUtensorMap map_w, float *__restrict__ out, float *__restrict__ lam, int N_all,
-                int NC_all, const int *__restrict__ cu, int planes, StatusBlock *status, int clear_status,
-                int start_aborted)
+                const __grid_constant__ CUtensorMap map_w, float *__restrict__ out, float *__restrict__ lam, const WorkArgs wk,
+                int spans, int cut, StatusBlock *status, int clear_status, int start_aborted)
 {
-    using G = Geo<kBwd>;
+    using G = Geo<kBwd, kStages>;
     if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
         status->code = 0;
         status->where = 0;
@@ -76,30 +92,19 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     float *hp = reinterpret_cast<float *>(smem + G::kOffHp);
-    Ctl *ctl = reinterpret_cast<Ctl *>(smem + G::kOffCtl);
+    Ctl<kStages> *ctl = reinterpret_cast<Ctl<kStages> *>(smem + G::kOffCtl);
     volatile int *abort_flag = &ctl->abort_flag;
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    const int u = blockIdx.x;
-    // this CTA's segment: rows [row0, row0 + N) of plane zu, NC chunks
-    int row0 = 0, zu = u, N = N_all, NC = NC_all;
-    if constexpr (kRagged) {
-        if (cu != nullptr) {
-            const int b = u / planes;
-            zu = u - b * planes;
-            row0 = __ldg(cu + b);
-            N = __ldg(cu + b + 1) - row0;
-            if (row0 < 0 || N < 0 || row0 + N > N_all) {          // malformed offsets: report, touch nothing
-                if (tid == 0) report_error(status, HGRN2_ERR_INVALID_ARG, 6);
-                return;
-            }
-        }
-        NC = (N + kC - 1) / kC;
-        if (N <= 0) {                    // an empty segment contributes nothing and does not decay
-            for (int x = tid; x < kD * kD; x += kThreads) out[(size_t)u * kD * kD + x] = 0.f;
-            if (lam != nullptr && tid < kD) lam[(size_t)u * kD + tid] = 1.f;
-            return;
-        }
+    bool malformed = false;
+    const Span sp = span_of<kBwd>(wk, blockIdx.x, spans != 0, cut, malformed);
+    const int zu = sp.plane, row0 = sp.row0, N = sp.n, NC = (N + kC - 1) / kC;
+    const size_t u = sp.at;
+    if (malformed && tid == 0) report_error(status, HGRN2_ERR_INVALID_ARG, 6);
+    if (N <= 0) {                        // an empty segment contributes nothing and does not decay
+        for (int x = tid; x < kD * kD; x += kThreads) out[u * kD * kD + x] = 0.f;
+        if (lam != nullptr && tid < kD) lam[u * kD + tid] = 1.f;
+        return;
     }
 
     if (tid == 0) {
@@ -197,7 +202,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
             mbar_arrive(&ctl->t_done[s]);
         }
         if (lam != nullptr && half == 0)
-            *reinterpret_cast<float2 *>(lam + (size_t)u * kD + col) = make_float2(P0, P1);
+            *reinterpret_cast<float2 *>(lam + u * kD + col) = make_float2(P0, P1);
 
         // the accumulator, one row per thread (TMEM lane = key dimension = 32 * (warp % 4) + lane)
         mbar_wait(&ctl->acc_done, 0, abort_flag);
@@ -209,7 +214,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
             uint32_t r[32];
             tmem_ld32(tl + 32 * part, r);
             tmem_wait_ld();
-            float4 *dst = reinterpret_cast<float4 *>(out + ((size_t)u * kD + krow) * kD + 32 * part);
+            float4 *dst = reinterpret_cast<float4 *>(out + (u * kD + krow) * kD + 32 * part);
 #pragma unroll
             for (int j = 0; j < 8; ++j)
                 dst[j] = make_float4(__uint_as_float(r[4 * j + 0]), __uint_as_float(r[4 * j + 1]),
@@ -267,56 +272,60 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
     if (warp == 0) tmem_dealloc(tmem, 128);
 }
 
-template <bool kBwd, bool kEnc, bool kRagged>
-cudaError_t launch_state_t(const void *o, const void *f, const void *w, uint64_t planes, int N, uint64_t ctas, const int *cu,
-                           float *out, float *lam, StatusBlock *status, bool clear, int start_aborted, cudaStream_t stream)
+template <bool kBwd, bool kEnc, bool kRagged, int kStages>
+cudaError_t launch_state_t(const CUtensorMap &mo, const CUtensorMap &mf, const CUtensorMap &mw, uint64_t ctas, const WorkArgs &wk,
+                           bool spans, int cut, float *out, float *lam, StatusBlock *status, bool clear, int start_aborted,
+                           cudaStream_t stream)
 {
-    using G = Geo<kBwd>;
-    CUtensorMap mo, mf, mw;
-    if (!make_map(&mo, kBwd ? o : f, planes, N, kC) || !make_map(&mf, f, planes, N, kC) || !make_map(&mw, w, planes, N, kC))
-        return cudaErrorInvalidValue;
-    auto kernel = tc_state_kernel<kBwd, kEnc, kRagged>;
+    using G = Geo<kBwd, kStages>;
+    auto kernel = tc_state_kernel<kBwd, kEnc, kRagged, kStages>;
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), G::kSmemBytes);
     if (err != cudaSuccess) return err;
-    kernel<<<(unsigned)ctas, kThreads, G::kSmemBytes, stream>>>(mo, mf, mw, out, lam, N, N / kC, cu, (int)planes, status,
-                                                             clear ? 1 : 0, start_aborted);
+    kernel<<<(unsigned)ctas, kThreads, G::kSmemBytes, stream>>>(mo, mf, mw, out, lam, wk, spans, cut, status, clear ? 1 : 0,
+                                                             start_aborted);
     return cudaGetLastError();
 }
 
-// planes x N rows; without offsets one CTA per plane, with offsets nseq CTAs per plane (see the kernel)
 template <bool kBwd>
-cudaError_t launch_state(const void *o, const void *f, const void *w, uint64_t planes, int N, const int *cu, int nseq,
-                         float *out, float *lam, bool gate_enc, StatusBlock *status, bool clear, int start_aborted,
+cudaError_t launch_state(const void *o, const void *f, const void *w, uint64_t planes, const WorkArgs &wk, bool spans,
+                         uint64_t cut, float *out, float *lam, bool gate_enc, StatusBlock *status, bool clear, int start_aborted,
                          cudaStream_t stream)
 {
-    const bool ragged = cu != nullptr || N % kC != 0;
-    const uint64_t ctas = cu ? planes * (uint64_t)nseq : planes;
-    if (ctas == 0 || N <= 0) return cudaSuccess;
+    const uint64_t ctas = spans ? planes : cut * (wk.G - 1);
+    if (ctas == 0 || wk.N <= 0) return cudaSuccess;
     if (ctas > 0x7fffffffull) return cudaErrorInvalidConfiguration;
-    if (gate_enc)
-        return ragged ? launch_state_t<kBwd, true, true>(o, f, w, planes, N, ctas, cu, out, lam, status, clear, start_aborted, stream)
-                      : launch_state_t<kBwd, true, false>(o, f, w, planes, N, ctas, cu, out, lam, status, clear, start_aborted, stream);
-    return ragged ? launch_state_t<kBwd, false, true>(o, f, w, planes, N, ctas, cu, out, lam, status, clear, start_aborted, stream)
-                  : launch_state_t<kBwd, false, false>(o, f, w, planes, N, ctas, cu, out, lam, status, clear, start_aborted, stream);
+    CUtensorMap mo, mf, mw;
+    if (!make_map(&mo, kBwd ? o : f, planes, wk.N, kC) || !make_map(&mf, f, planes, wk.N, kC) || !make_map(&mw, w, planes, wk.N, kC))
+        return cudaErrorInvalidValue;
+    const bool ragged = wk.cu != nullptr || wk.N % kC != 0;
+    const bool pair = ctas > (uint64_t)sm_count();            // more CTAs than SMs: two per SM
+    constexpr int kPair = kBwd ? 2 : 3;                       // stages that leave room for a second CTA
+    auto go = [&](auto enc, auto rag) {
+        constexpr bool kEnc = decltype(enc)::value, kRagged = decltype(rag)::value;
+        return pair ? launch_state_t<kBwd, kEnc, kRagged, kPair>(mo, mf, mw, ctas, wk, spans, (int)cut, out, lam, status, clear, start_aborted, stream)
+                    : launch_state_t<kBwd, kEnc, kRagged, 4>(mo, mf, mw, ctas, wk, spans, (int)cut, out, lam, status, clear, start_aborted, stream);
+    };
+    using T = std::true_type;
+    using F = std::false_type;
+    return gate_enc ? (ragged ? go(T{}, T{}) : go(T{}, F{})) : (ragged ? go(F{}, T{}) : go(F{}, F{}));
 }
 
 }  // namespace
 
-// Forward: S_loc [.][128][128] and Lambda [.][128] from f and i.  Without `cu`: one segment per plane, the N rows
-// of each of the U planes.  With `cu` (device, nseq + 1 offsets): segment b * U + h = rows [cu[b], cu[b + 1]) of plane h.
-cudaError_t launch_tc_state_fwd(const void *f, const void *i, uint64_t U, int N, float *S_loc, float *lam, bool gate_enc,
-                                StatusBlock *status, bool clear, int start_aborted, cudaStream_t stream, const int *cu,
-                                int nseq)
+cudaError_t launch_tc_state(bool bwd, const void *o, const void *f, const void *w, const TcWork &t, bool gate_enc,
+                            StatusBlock *status, bool clear, int start_aborted, cudaStream_t stream)
 {
-    return launch_state<false>(nullptr, f, i, U, N, cu, nseq, S_loc, lam, gate_enc, status, clear, start_aborted, stream);
+    return bwd ? launch_state<true>(o, f, w, t.planes, t.wk, false, t.cut, t.chain, t.lam, gate_enc, status, clear, start_aborted, stream)
+               : launch_state<false>(o, f, w, t.planes, t.wk, false, t.cut, t.chain, t.lam, gate_enc, status, clear, start_aborted, stream);
 }
 
-// Backward: G_loc and Lambda of the same segments from o, f and dy.
-cudaError_t launch_tc_state_bwd(const void *o, const void *f, const void *dy, uint64_t U, int N, float *G_loc,
-                                float *lam, bool gate_enc, StatusBlock *status, bool clear, int start_aborted,
-                                cudaStream_t stream, const int *cu, int nseq)
+cudaError_t launch_tc_span(bool bwd, const void *o, const void *f, const void *w, uint64_t planes, int N, float *out,
+                           float *lam, StatusBlock *status, bool clear, int start_aborted, cudaStream_t stream)
 {
-    return launch_state<true>(o, f, dy, U, N, cu, nseq, G_loc, lam, gate_enc, status, clear, start_aborted, stream);
+    WorkArgs wk;
+    wk.N = N;
+    return bwd ? launch_state<true>(o, f, w, planes, wk, true, 0, out, lam, false, status, clear, start_aborted, stream)
+               : launch_state<false>(o, f, w, planes, wk, true, 0, out, lam, false, status, clear, start_aborted, stream);
 }
 
 }  // namespace hgrn2

@@ -119,7 +119,7 @@ struct SeqArgs {
     StatusBlock *status;
     float *room = nullptr;        // fp32 path: the workspace's room for one set of boundary states
     void *seg_scratch;            // tensor-core path: scratch for sequences split into segments (nullable)
-    float *exact_scratch = nullptr;   // tensor-core backward: [B*H][dk][dv] floats for units redone on the exact path
+    float *exact_scratch = nullptr;   // tensor-core backward: [work item][dk][dv] floats for the exact path
     float *totals = nullptr;      // tensor-core path: per-chunk decay totals inside the saved data (set by its launchers)
     bool clear_status = false;    // the first kernel of the call zeroes the status word itself
     int start_aborted = 0;        // tensor-core path, debugging: every CTA starts as if its first wait had run out
@@ -137,66 +137,54 @@ struct StepArgs {
     cudaStream_t stream;
 };
 
-// Tensor-core path: what a CTA needs to redo a whole unit on the exact fp32 path (chunk_alu.cuh) after its
-// sweep has found a decay that the rescaled operands cannot represent.  Plain pointers to unit 0 of the launch
-// (the kernels proper work through tensor maps); o == nullptr switches the exact path off.
+// Tensor-core path: what a CTA needs, besides its launch's other arguments, to redo an item on the exact fp32 path
+// (chunk_alu.cuh) after its sweep has found a decay that the rescaled operands cannot represent.  Plain pointers (the
+// kernels proper work through tensor maps); o == nullptr switches the exact path off.
 struct ExactArgs {
     const __nv_bfloat16 *o = nullptr, *f = nullptr, *i = nullptr, *dy = nullptr;
-    const float *S0 = nullptr, *dSN = nullptr;
     __nv_bfloat16 *y = nullptr, *d_o = nullptr, *d_f = nullptr, *d_i = nullptr;
-    float *SN = nullptr, *dS0 = nullptr;
-    __nv_bfloat16 *states = nullptr;    // saved chunk states: [unit][chunk of 64][128][128] bf16
-    float *scratch = nullptr;           // backward: [unit][128][128] floats
-    int N = 0;                          // tokens of a whole unit (rows per head of a packed batch)
-    int G = 1;                          // CTAs (segments) per unit in this launch
-    int *unit_flag = nullptr;           // G > 1: per unit, set by any segment that left the range
-    int *unit_count = nullptr;          // G > 1: per unit, segments finished so far
+    __nv_bfloat16 *states = nullptr;    // saved chunk states: [slot][128][128] bf16
+    float *scratch = nullptr;           // backward: [item][128][128] floats
 };
 
-// Packed (variable-length) batches: the sequence tensors are [H][T][d] and sequence b occupies the token rows
-// [cu[b], cu[b + 1]) of every head; unit u = b * H + h.  cu == nullptr: the ordinary [B][H][N][d] layout.
-// Chunk-start states of a packed batch live in slots: sequence b owns slots floor(cu[b] / C) + b ... of its head
-// (never overlapping the next sequence's), slots_per_head = floor(T / C) + B + 1.
-struct PackedArgs {
-    const int *cu = nullptr;
-    int H = 0;
-    int slots_per_head = 0;
+// Tensor-core path: the work items of a launch (tc_chunk.cuh).  Packed (variable-length) batches: the sequence tensors
+// are [H][T][d] and sequence b occupies the token rows [cu[b], cu[b + 1]) of every head; state u = b * H + h.
+// Chunk-start states of a packed batch live in slots: segment b * G + r of a head starts at slot
+// (its first row) / 64 + b * G + r of the head's spp = T / 64 + B * G + 1 (never overlapping the next segment's).
+struct WorkArgs {
+    int N = 0, NC = 0;             // rows per plane; chunks of a whole sequence (ordinary batch)
+    int main = 0, tail = 0;        // units taken whole, units cut into segments (ordinary batch)
+    int G = 1, Lc = 0;             // segments per cut unit, chunks per segment
+    const int *cu = nullptr;       // packed batch: row offsets on the device
+    int H = 1, spp = 0;            // packed batch: heads, state slots per head
 };
 
-// Tensor-core path, few or left-over units: which units run whole and which are split into G segments each.
+// How an ordinary batch is cut: units [0, main) run whole, the `tail` units behind them as G segments of Lc chunks (the
+// last one shorter).  tail == 0: nothing is cut.
 struct SegPlan {
-    uint64_t main_units;   // units [0, main_units) run as one CTA each
-    uint64_t tail_units;   // units [main_units, main_units + tail_units) are split into G segments each
-    int G;
+    int main, tail, G, Lc;
+    bool gain;             // the cut is expected to pay
 };
-int         sm_count();        // SMs of the current device (0: no device)
-SegPlan     tc_seg_plan(uint64_t U, int N, int NC);
-// Sequences that are NOT whole chunks, few or left-over units (as SegPlan): those units' sequences are cut into G
-// segments of Lc chunks (the last one shorter), which run through the packed-batch geometry (per-CTA rows from an
-// offsets array).
-struct RSegPlan {
-    uint64_t main_units;   // units [0, main_units) run as one CTA each
-    uint64_t tail_units;   // units [main_units, main_units + tail_units) run as G segments each (0: nothing is split)
-    int G;
-    int Lc;
-};
-RSegPlan    tc_rseg_plan(uint64_t U, int N, int NC);
-constexpr size_t kRSegOffsetsBytes = 256;      // the offsets array of the ragged segments, in front of their scratch
-void        launch_seg_offsets(int *cu, int G, int L, int N, cudaStream_t stream);
-// Packed batch on few units: every sequence is cut into the same number G of segments (short sequences leave
-// some of theirs empty); the lengths are known on the device only, so the offsets of the B * G segments are
-// written there.  G = 1: not split.
+SegPlan     tc_plan(uint64_t U, int NC);
 int         tc_packed_segments(uint64_t U, int T);
-size_t      tc_packed_offsets_bytes(int B, int G);
-void        launch_seg_offsets_packed(const int *cu, int B, int G, int *cu_seg, cudaStream_t stream);
-SeqArgs     tc_slice_units(const SeqArgs &a, uint64_t u0, uint64_t n);
-
-cudaError_t launch_tc_state_fwd(const void *f, const void *i, uint64_t U, int N, float *S_loc, float *lam, bool gate_enc,
-                                StatusBlock *status, bool clear, int start_aborted, cudaStream_t stream,
-                                const int *cu = nullptr, int nseq = 1);
-cudaError_t launch_tc_state_bwd(const void *o, const void *f, const void *dy, uint64_t U, int N, float *G_loc,
-                                float *lam, bool gate_enc, StatusBlock *status, bool clear, int start_aborted,
-                                cudaStream_t stream, const int *cu = nullptr, int nseq = 1);
+int         sm_count();        // SMs of the current device (0: no device)
+constexpr uint32_t kFlagNoSegments = 0x40000000u;      // desc->flags, internal: no sequence is cut (needs no scratch for it)
+struct TcWork {
+    WorkArgs wk;
+    uint64_t items = 0;    // CTAs of the launch
+    uint64_t cut = 0;      // units run as G segments each
+    uint64_t planes = 0;   // planes of the sequence tensors
+    uint64_t slots = 0;    // chunk-state slots
+    uint64_t chunks = 0;   // of an item, on average
+    float *chain = nullptr, *lam = nullptr;    // boundary states [cut][G - 1][128][128] and decays [cut][G - 1][128]
+};
+TcWork      tc_work(SeqArgs &a);
+cudaError_t launch_seg_chain(bool bwd, const TcWork &t, const float *init, cudaStream_t stream);
+// State-only passes (chunk_tc_state.cu): the segments of t that a chain needs, or one span per plane.
+cudaError_t launch_tc_state(bool bwd, const void *o, const void *f, const void *w, const TcWork &t, bool gate_enc,
+                            StatusBlock *status, bool clear, int start_aborted, cudaStream_t stream);
+cudaError_t launch_tc_span(bool bwd, const void *o, const void *f, const void *w, uint64_t planes, int N, float *out,
+                           float *lam, StatusBlock *status, bool clear, int start_aborted, cudaStream_t stream);
 cudaError_t launch_step(const StepArgs &a);
 bool        step_multi_supported(int dk, int dv);
 cudaError_t launch_step_multi(const StepArgs &a);

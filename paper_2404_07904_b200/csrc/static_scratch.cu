@@ -44,12 +44,15 @@ extern "C" hgrn2_status hgrn2_bwd_static_scratch(const hgrn2_desc *desc, const v
                                (desc->io == HGRN2_F32 || desc->io == HGRN2_BF16);
         return fields_ok ? HGRN2_ERR_UNSUPPORTED : HGRN2_ERR_INVALID_ARG;
     }
-    if (need > sizeof(g_static_scratch)) return HGRN2_ERR_WORKSPACE;   // problem too large for the built-in scratch
+    // a problem that does not fit with room for cutting its sequences runs without
+    hgrn2_desc d = *desc;
+    if (need > sizeof(g_static_scratch)) d.flags |= hgrn2::kFlagNoSegments;
+    if (hgrn2_workspace_bytes(&d) > sizeof(g_static_scratch)) return HGRN2_ERR_WORKSPACE;   // too large for the built-in scratch
     if (status_out && (reinterpret_cast<uintptr_t>(status_out) & 15u)) return HGRN2_ERR_ALIGNMENT;
     void *scratch = scratch_for_current_device();
     if (!scratch) return HGRN2_ERR_CUDA;
     // saved = NULL: the states are re-created inside the scratch; the call clears the status block first.
-    hgrn2_status st = hgrn2_bwd(desc, o, f, i, S0, dy, dSN, nullptr, d_o, d_f, d_i, dS0, scratch, cuda_stream);
+    hgrn2_status st = hgrn2_bwd(&d, o, f, i, S0, dy, dSN, nullptr, d_o, d_f, d_i, dS0, scratch, cuda_stream);
     if (st != HGRN2_OK) return st;
     if (status_out &&
         cudaMemcpyAsync(status_out, scratch, 8, cudaMemcpyDeviceToDevice, static_cast<cudaStream_t>(cuda_stream)) !=

@@ -229,14 +229,171 @@ __device__ __forceinline__ void tril_row_block(uint32_t taddr, uint8_t *dstbuf, 
     }
 }
 
-// Where segment r of unit u sits among the segment summaries (chunk_tc_fwd.cu, sequences split into segments):
-// order 0: u * G + r; order 1: r * U + u (ragged segments of an ordinary batch); order 2: unit u = (sequence b,
-// head h) of a packed batch with H heads, its segment r at (b * G + r) * H + h.
-__device__ __forceinline__ size_t seg_index(int order, size_t u, int r, int G, size_t U, int H)
+// ---- work items ---------------------------------------------------------------------------------------
+// A work item is a run of chunks that one CTA takes in one go: a whole sequence, or one segment of a sequence that was
+// cut into G of them (why: chunk_tc_fwd.cu).  Item x of a launch (WorkArgs: common.cuh):
+//   ordinary batch   x < main: unit x whole; beyond that item main + r * tail + t = segment r (Lc chunks, the last one
+//                    shorter) of unit main + t;
+//   packed batch     segment r of sequence b, head h at x = (b * G + r) * H + h; a sequence's segments have
+//                    max(8, ceil(chunks / G)) chunks, those beyond its end are empty (G = 1: whole sequences).
+// Between the segments of a unit sit G - 1 boundary states (chain slots, index base + r for the boundary between
+// segments r and r + 1).
+struct Item {
+    int id;                        // -1: no more work
+    int plane, row0, n;            // rows [row0, row0 + n) of plane `plane`
+    int slot0;                     // first chunk-state slot
+    int unit;                      // index of its state in S0, SN (dSN, dS0)
+    int chain;                     // chain slot of the state it starts from (backward: of the gradient it starts from), -1: S0 (dSN)
+    int last;                      // its final state is S_N (backward: its final gradient is dS_0)
+};
+
+template <bool kPackedToo, bool kBwd>
+__device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malformed)
 {
-    if (order == 1) return (size_t)r * U + u;
-    if (order == 2) return ((u / H) * G + r) * H + u % H;
-    return u * G + r;
+    Item it;
+    it.id = x;
+    if (kPackedToo && w.cu != nullptr) {
+        const int h = x % w.H, br = x / w.H, b = br / w.G, r = br - b * w.G;
+        const int start = __ldg(w.cu + b), len = __ldg(w.cu + b + 1) - start;
+        it.plane = h;
+        it.unit = b * w.H + h;
+        if (start < 0 || len < 0 || start + len > w.N) {             // malformed offsets: touch nothing
+            malformed = true;
+            it.row0 = it.n = it.slot0 = it.last = 0;
+            it.chain = -1;
+            return it;
+        }
+        int lo = 0, hi = len;
+        if (w.G > 1) {
+            const int Lc = max(8, ((len + kC - 1) / kC + w.G - 1) / w.G);
+            lo = min(r * Lc * kC, len);
+            hi = min(lo + Lc * kC, len);
+        }
+        it.row0 = start + lo;
+        it.n = hi - lo;
+        it.slot0 = h * w.spp + it.row0 / kC + br;
+        const bool ends = hi == len && (hi > lo || r == 0);          // the sequence's last segment with tokens
+        it.last = kBwd ? r == 0 : ends;
+        it.chain = (kBwd ? ends : r == 0) ? -1 : it.unit * (w.G - 1) + (kBwd ? r : r - 1);
+        return it;
+    }
+    if (x < w.main) {
+        it.plane = it.unit = x;
+        it.row0 = 0;
+        it.n = w.N;
+        it.slot0 = x * w.NC;
+        it.chain = -1;
+        it.last = 1;
+        return it;
+    }
+    const int y = x - w.main, r = y / w.tail, t = y - r * w.tail;
+    it.plane = it.unit = w.main + t;
+    it.row0 = r * w.Lc * kC;
+    it.n = min(w.Lc * kC, w.N - it.row0);
+    it.slot0 = it.unit * w.NC + r * w.Lc;
+    it.last = kBwd ? r == 0 : r == w.G - 1;
+    it.chain = (kBwd ? r == w.G - 1 : r == 0) ? -1 : t * (w.G - 1) + (kBwd ? r : r - 1);
+    return it;
+}
+
+// kPersist instantiations: a CTA works through several items, one after the other with all pipelines running on: the
+// first is its own block index, the others are taken from CTAs of the grid that have not started (cluster launch
+// control), so a launch of many short items pays a CTA's start-up and pipeline fill once per SM and keeps the hardware's
+// dynamic balance.  The load warp takes them - as late as it can, when it asks for its current item's last tiles, so
+// that an SM with a long item does not hoard another one - and publishes them in a ring that every role's warps
+// read.  All of this is out of line: the roles run concurrently, and their combined code is about what the instruction
+// cache holds (which is also why the other instantiations know nothing of it).
+constexpr int kRing = 4;           // the load warp is at most this many items ahead of the slowest role
+struct ItemRing {
+    Item item[kRing], none;
+    uint4 answer;                  // cluster launch control response (16-byte aligned)
+    uint64_t full[kRing];          // load warp -> everyone
+    uint64_t empty[kRing];         // one lane per warp -> load warp
+    uint64_t answered;             // the hardware's response has landed
+    int flagged[8];                // items (index + 1) whose decay left the operands' range, by position mod 8
+    int asked;                     // responses asked for so far, for the abort epilogue
+};
+__device__ __forceinline__ void ring_init(ItemRing &q, int warps)
+{
+    for (int s = 0; s < kRing; ++s) {
+        mbar_init(&q.full[s], 1);
+        mbar_init(&q.empty[s], warps);
+    }
+    mbar_init(&q.answered, 1);
+    for (int j = 0; j < 8; ++j) q.flagged[j] = 0;
+    q.asked = 0;
+    q.none = Item{-1, 0, 0, 0, 0, 0, -1, 0};
+}
+// The same item in every lane, in a form that tells the compiler so: the loops over its chunks stay convergent code
+// ("warp-wide issue", tc_common.cuh).
+__device__ __forceinline__ Item warp_uniform(const Item &x)
+{
+    constexpr unsigned all = 0xffffffffu;
+    return Item{__shfl_sync(all, x.id, 0),    __shfl_sync(all, x.plane, 0), __shfl_sync(all, x.row0, 0),  __shfl_sync(all, x.n, 0),
+                __shfl_sync(all, x.slot0, 0), __shfl_sync(all, x.unit, 0),  __shfl_sync(all, x.chain, 0), __shfl_sync(all, x.last, 0)};
+}
+// Item k for a reading warp, in place: valid until the warp asks for item k + 1.  id < 0: no more work.  After an abort
+// the warp is told so as one (the slot it would have read may be in flux).
+static __device__ __noinline__ const Item *ring_next(ItemRing *q, int k, volatile int *abort_flag)
+{
+    const Item *it = &q->item[k % kRing];
+    if (k > 0) {
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(&q->empty[(k - 1) % kRing]);
+        mbar_wait(&q->full[k % kRing], (k / kRing) & 1, abort_flag);
+        if (__any_sync(0xffffffffu, *abort_flag)) it = &q->none;
+    }
+    return it;
+}
+// Item k of a CTA whose first is `first`; false: no more.  Whole warp.
+template <bool kPersist>
+__device__ __forceinline__ bool next_item(ItemRing *q, int k, volatile int *abort_flag, const Item &first, Item &it)
+{
+    if constexpr (!kPersist) {
+        it = first;
+        return k == 0;
+    } else {
+        it = warp_uniform(*ring_next(q, k, abort_flag));
+        return it.id >= 0;
+    }
+}
+// Load warp: asks for item k (not before every warp has given up item k - kRing).  No more are taken once an item has been
+// flagged for the exact path, which runs after the last one (the list of flagged items stays short), or after an abort.
+static __device__ __noinline__ bool ring_ask(ItemRing *q, int k, volatile int *exact_flag, volatile int *abort_flag)
+{
+    if (k >= kRing) mbar_wait(&q->empty[k % kRing], (k / kRing - 1) & 1, abort_flag);
+    if (__any_sync(0xffffffffu, *exact_flag || *abort_flag)) return false;
+    mbar_arrive_expect_tx(&q->answered, 16);
+    if ((threadIdx.x & 31) == 0) {
+        clc_try_cancel(&q->answer, &q->answered);
+        ++q->asked;
+    }
+    __syncwarp();
+    return true;
+}
+// Load warp: the answer to ring_ask (asked = its return value) becomes item k.
+template <bool kPackedToo, bool kBwd>
+static __device__ __noinline__ const Item *ring_take(ItemRing *q, int k, bool asked, const WorkArgs &w, StatusBlock *status,
+                                                     volatile int *abort_flag)
+{
+    int x = -1;
+    if (asked) {
+        mbar_wait(&q->answered, (q->asked - 1) & 1, abort_flag);
+        if (!__any_sync(0xffffffffu, *abort_flag)) {
+            x = clc_answer(&q->answer);
+            fence_proxy_async_smem();                                // the answer has been read before the next one lands
+        }
+    }
+    Item *it = &q->item[k % kRing];
+    if ((threadIdx.x & 31) == 0) {
+        bool malformed = false;
+        if (x >= 0) *it = work_item<kPackedToo, kBwd>(w, x, malformed);
+        else *it = q->none;
+        if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
+        mbar_arrive(&q->full[k % kRing]);
+    }
+    __syncwarp();
+    return it;
 }
 
 // ---- host side: tensor maps ---------------------------------------------------------------------

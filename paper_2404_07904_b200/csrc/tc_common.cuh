@@ -157,6 +157,36 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity, 
     return true;
 }
 
+// ---- cluster launch control ----------------------------------------------------------------------
+// Asks the hardware scheduler for a CTA of this grid that has not started yet: its index is cancelled there and comes
+// back as 16 bytes at `response` (completion counted on `bar`), for this CTA to do its work.  After an answer that says
+// "none left" it must not be asked again.
+__device__ __forceinline__ void clc_try_cancel(void *response, uint64_t *bar)
+{
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                 ::"r"(smem_u32(response)), "r"(smem_u32(bar))
+                 : "memory");
+}
+// The x index of the CTA in the response, or -1.
+__device__ __forceinline__ int clc_answer(const void *response)
+{
+    uint32_t ok = 0, x = 0;
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        ".reg .b128 r;\n\t"
+        "ld.shared.b128 r, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "mov.u32 %1, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, r;\n\t"
+        "}"
+        : "=r"(ok), "=r"(x)
+        : "r"(smem_u32(response))
+        : "memory");
+    return ok ? (int)x : -1;
+}
+
 // ---- warp-wide issue --------------------------------------------------------------------------------
 // The roles that issue tensor-core products and bulk copies run as whole warps, and only the issuing instruction itself
 // is predicated to one lane, elected anew each time (always the same one).  A role that runs inside `if (lane == 0)` is
