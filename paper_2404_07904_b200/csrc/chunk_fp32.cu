@@ -256,6 +256,7 @@ fp32_local_kernel(const Args a)
     constexpr int RP = P::RP;
     extern __shared__ __align__(16) float sm[];
     float *sX = sm, *sV = sm + kL * TK, *sprod = sV + kL * TV;
+    chain_wait();
     if (a.status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) {
         a.status->code = 0;
         a.status->where = 0;
@@ -367,6 +368,7 @@ template <typename T, int kMode, bool kBwd>
 __global__ void __launch_bounds__(kScanThreads)
 fp32_scan_kernel(const Args a)
 {
+    chain_wait();
     const Where w = a.cu == nullptr
         ? Where{(a.g0 + blockIdx.x) * a.N, a.N, a.NC, (long long)blockIdx.x * a.NC, a.g0 + blockIdx.x}
         : packed_where(a, blockIdx.x % a.B, a.g0 + blockIdx.x / a.B);
@@ -431,6 +433,7 @@ template <typename T, int kMode, bool kDV, int NV>
 __global__ void __launch_bounds__(kValueThreads, 2)
 fp32_value_kernel(const Args a)
 {
+    chain_wait();
     using P = ValueShape<NV>;
     constexpr int kTile = P::kTile;
     extern __shared__ __align__(16) float sm[];
@@ -717,6 +720,7 @@ template <typename T, int kMode>
 __global__ void __launch_bounds__(kKeyThreads, 2)
 fp32_key_kernel(const Args a)
 {
+    chain_wait();
     extern __shared__ __align__(16) float sm[];
     float *sprod = sm + 6 * kSq;                                      // [8][64]
     float *sR = sprod + 8 * kL;                                       // [2][64]
@@ -1108,8 +1112,7 @@ cudaError_t launch_local_t(const Args &a, long long chunks, cudaStream_t stream)
     auto kernel = fp32_local_kernel<T, kMode, kBwd, TK, TV, SPLIT>;
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), P::kSmem);
     if (err != cudaSuccess) return err;
-    kernel<<<(unsigned)chunks, P::NT, P::kSmem, stream>>>(a);
-    return cudaGetLastError();
+    return launch_chained(kernel, dim3((unsigned)chunks), P::NT, P::kSmem, stream, a);
 }
 
 // Boundary values of `groups` groups: every chunk's own contribution, then the chain over each sequence.
@@ -1126,8 +1129,8 @@ cudaError_t launch_state(const Args &a, long long groups, cudaStream_t stream)
                         : launch_local_t<T, kMode, kBwd, 64, 64, 2>(a, chunks, stream);
     if (err != cudaSuccess) return err;
     const unsigned blocks = (a.dk * a.dv / 4 + kScanThreads - 1) / kScanThreads;
-    fp32_scan_kernel<T, kMode, kBwd><<<dim3((unsigned)(groups * units_per_group(a)), blocks), kScanThreads, 0, stream>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fp32_scan_kernel<T, kMode, kBwd>, dim3((unsigned)(groups * units_per_group(a)), blocks), kScanThreads, 0,
+                          stream, a);
 }
 
 template <typename T, int kMode, bool kDV, int NV>
@@ -1137,8 +1140,7 @@ cudaError_t launch_value_t(const Args &a, long long chunks, cudaStream_t stream)
     auto kernel = fp32_value_kernel<T, kMode, kDV, NV>;
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), P::kSmem);
     if (err != cudaSuccess) return err;
-    kernel<<<(unsigned)chunks, kValueThreads, P::kSmem, stream>>>(a);
-    return cudaGetLastError();
+    return launch_chained(kernel, dim3((unsigned)chunks), kValueThreads, P::kSmem, stream, a);
 }
 template <typename T, int kMode, bool kDV>
 cudaError_t launch_value(const Args &a, long long chunks, cudaStream_t stream)
@@ -1151,8 +1153,7 @@ cudaError_t launch_key(const Args &a, long long chunks, cudaStream_t stream)
 {
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(fp32_key_kernel<T, kMode>), kKSmem);
     if (err != cudaSuccess) return err;
-    fp32_key_kernel<T, kMode><<<dim3((unsigned)chunks, (a.dk + kL - 1) / kL), kKeyThreads, kKSmem, stream>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fp32_key_kernel<T, kMode>, dim3((unsigned)chunks, (a.dk + kL - 1) / kL), kKeyThreads, kKSmem, stream, a);
 }
 
 // groups = independent groups a launch can be restricted to: units, or heads of a packed batch

@@ -235,15 +235,14 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
               const __grid_constant__ WorkArgs wk, StatusBlock *status, int clear_status, const ExactArgs ex,
               int start_aborted)
 {
-    // the first kernel of a call zeroes the status word; the only early report, the alignment check below, is the
-    // same in every CTA, so CTA 0 repeats it after its own clear
-    if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
-        status->code = 0;
-        status->where = 0;
-        status->exact_units = 0;
-    }
     extern __shared__ __align__(1024) uint8_t smem[];
     if (smem_u32(smem) & 1023u) {          // every byte is spoken for: the swizzled tiles need the base aligned
+        chain_wait();
+        if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
+            status->code = 0;
+            status->where = 0;
+            status->exact_units = 0;
+        }
         if (threadIdx.x == 0) report_error(status, HGRN2_ERR_CUDA, 3);
         return;
     }
@@ -261,8 +260,6 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     volatile int *abort_flag = &ctl->abort_flag;
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    bool malformed = false;
-    const Item first = warp_uniform(work_item<kRagged, true>(wk, blockIdx.x, malformed));
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&ctl->full[s], 1);
@@ -291,11 +288,6 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         ctl->l_stage = ctl->l_v = ctl->l_state = ctl->l_raw = 0;
         ring_init(ctl->ring, kRingWarps);
         fence_barrier_init();
-        if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
-        if (kPersist) {
-            ctl->ring.item[0] = first;
-            mbar_arrive(&ctl->ring.full[0]);
-        }
         tma_prefetch_desc(&map_o);
         tma_prefetch_desc(&map_f);
         tma_prefetch_desc(&map_i);
@@ -305,6 +297,22 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         tma_prefetch_desc(&map_f_raw);
     }
     if (warp == 0) tmem_alloc(&ctl->tmem_base, kTmemCols);
+    chain_wait();
+    // the first kernel of a call zeroes the status word (errors are reported seconds later, after a wait ran out)
+    if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
+        status->code = 0;
+        status->where = 0;
+        status->exact_units = 0;
+    }
+    bool malformed = false;
+    const Item first = warp_uniform(work_item<kRagged, true>(wk, blockIdx.x, malformed));
+    if (tid == 0) {
+        if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
+        if (kPersist) {
+            ctl->ring.item[0] = first;
+            mbar_arrive(&ctl->ring.full[0]);
+        }
+    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -912,11 +920,7 @@ cudaError_t launch_tc_bwd(const SeqArgs &a0)
     ex.d_i = static_cast<__nv_bfloat16 *>(a.d_i);
     ex.states = reinterpret_cast<__nv_bfloat16 *>(a.states);
     ex.scratch = a.exact_scratch;
-    kernel<<<(unsigned)t.items, kThreads, kSmemBytes, a.stream>>>(
-        mo, mf, mi, mg, ms, mor, mfr, a.totals, a.dSN, t.chain, static_cast<__nv_bfloat16 *>(a.d_o),
-        static_cast<__nv_bfloat16 *>(a.d_f), static_cast<__nv_bfloat16 *>(a.d_i), a.dS0, t.wk, a.status,
-        a.clear_status ? 1 : 0, ex, a.start_aborted);
-    return cudaGetLastError();
+    return launch_chained(kernel, dim3((unsigned)t.items), kThreads, kSmemBytes, a.stream, mo, mf, mi, mg, ms, mor, mfr, a.totals, a.dSN, t.chain, static_cast<__nv_bfloat16 *>(a.d_o), static_cast<__nv_bfloat16 *>(a.d_f), static_cast<__nv_bfloat16 *>(a.d_i), a.dS0, t.wk, a.status, a.clear_status ? 1 : 0, ex, a.start_aborted);
 }
 
 }  // namespace hgrn2

@@ -95,12 +95,6 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
               const __grid_constant__ WorkArgs wk, StatusBlock *status, int clear_status, const ExactArgs ex,
               int start_aborted)
 {
-    // the first kernel of a call zeroes the status word (errors are reported seconds later, after a wait ran out)
-    if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
-        status->code = 0;
-        status->where = 0;
-        status->exact_units = 0;
-    }
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *sbuf = smem + kOffS;
@@ -112,8 +106,6 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     volatile int *abort_flag = &ctl->abort_flag;
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    bool malformed = false;
-    const Item first = warp_uniform(work_item<kRagged, false>(wk, blockIdx.x, malformed));
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&ctl->fullqf[s], 1);
@@ -141,11 +133,6 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         ctl->l_v = 0;
         ring_init(ctl->ring, kRingWarps);
         fence_barrier_init();
-        if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
-        if (kPersist) {
-            ctl->ring.item[0] = first;
-            mbar_arrive(&ctl->ring.full[0]);
-        }
         tma_prefetch_desc(&map_o);
         tma_prefetch_desc(&map_f);
         tma_prefetch_desc(&map_i);
@@ -153,6 +140,22 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         tma_prefetch_desc(&map_saved);
     }
     if (warp == 0) tmem_alloc(&ctl->tmem_base, kTmemCols);
+    chain_wait();
+    // the first kernel of a call zeroes the status word (errors are reported seconds later, after a wait ran out)
+    if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
+        status->code = 0;
+        status->where = 0;
+        status->exact_units = 0;
+    }
+    bool malformed = false;
+    const Item first = warp_uniform(work_item<kRagged, false>(wk, blockIdx.x, malformed));
+    if (tid == 0) {
+        if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
+        if (kPersist) {
+            ctl->ring.item[0] = first;
+            mbar_arrive(&ctl->ring.full[0]);
+        }
+    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -738,8 +741,9 @@ TcWork tc_work(SeqArgs &a)
 // segment r).  A thread owns four neighbouring elements; four segments' loads are in flight.
 template <bool kBwd>
 __global__ void __launch_bounds__(128)
-seg_chain_kernel(const float *__restrict__ init, float *__restrict__ chain, const float *__restrict__ lam, int G)
+seg_chain_kernel(const float *init, float *chain, const float *lam, int G)
 {
+    chain_wait();
     const size_t t = blockIdx.y;
     const int e = (blockIdx.x * 128 + threadIdx.x) * 4, k = e / kD, n = G - 1;
     float S[4] = {0.f, 0.f, 0.f, 0.f};
@@ -770,9 +774,7 @@ cudaError_t launch_seg_chain(bool bwd, const TcWork &t, const float *init, cudaS
 {
     if (init) init += (size_t)t.wk.main * kD * kD;
     const dim3 grid(kD * kD / 512, (unsigned)t.cut);
-    if (bwd) seg_chain_kernel<true><<<grid, 128, 0, stream>>>(init, t.chain, t.lam, t.wk.G);
-    else seg_chain_kernel<false><<<grid, 128, 0, stream>>>(init, t.chain, t.lam, t.wk.G);
-    return cudaGetLastError();
+    return launch_chained(bwd ? seg_chain_kernel<true> : seg_chain_kernel<false>, grid, 128, 0, stream, init, t.chain, t.lam, t.wk.G);
 }
 
 // More items than SMs: a CTA takes several (kPersist).  Against one CTA per item on 148 SMs: 4736 units of 64 tokens 193
@@ -811,10 +813,7 @@ cudaError_t launch_tc_fwd(const SeqArgs &a0)
     ex.i = static_cast<const __nv_bfloat16 *>(a.i);
     ex.y = static_cast<__nv_bfloat16 *>(a.y);
     ex.states = reinterpret_cast<__nv_bfloat16 *>(a.states);
-    kernel<<<(unsigned)t.items, kThreads, kSmemBytes, a.stream>>>(mo, mf, mi, my, ms, a.S0, t.chain, a.SN,
-                                                               want_saved ? a.totals : nullptr, want_y, want_saved, t.wk,
-                                                               a.status, a.clear_status ? 1 : 0, ex, a.start_aborted);
-    return cudaGetLastError();
+    return launch_chained(kernel, dim3((unsigned)t.items), kThreads, kSmemBytes, a.stream, mo, mf, mi, my, ms, a.S0, t.chain, a.SN, want_saved ? a.totals : nullptr, want_y, want_saved, t.wk, a.status, a.clear_status ? 1 : 0, ex, a.start_aborted);
 }
 
 }  // namespace hgrn2

@@ -84,6 +84,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
                 int spans, int cut, StatusBlock *status, int clear_status, int start_aborted)
 {
     using G = Geo<kBwd, kStages>;
+    chain_wait();
     if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
         status->code = 0;
         status->where = 0;
@@ -281,9 +282,8 @@ cudaError_t launch_state_t(const CUtensorMap &mo, const CUtensorMap &mf, const C
     auto kernel = tc_state_kernel<kBwd, kEnc, kRagged, kStages>;
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), G::kSmemBytes);
     if (err != cudaSuccess) return err;
-    kernel<<<(unsigned)ctas, kThreads, G::kSmemBytes, stream>>>(mo, mf, mw, out, lam, wk, spans, cut, status, clear ? 1 : 0,
-                                                             start_aborted);
-    return cudaGetLastError();
+    return launch_chained(kernel, dim3((unsigned)ctas), kThreads, G::kSmemBytes, stream, mo, mf, mw, out, lam, wk, spans ? 1 : 0, cut, status,
+                          clear ? 1 : 0, start_aborted);
 }
 
 template <bool kBwd>

@@ -254,7 +254,7 @@ __device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malfor
     it.id = x;
     if (kPackedToo && w.cu != nullptr) {
         const int h = x % w.H, br = x / w.H, b = br / w.G, r = br - b * w.G;
-        const int start = __ldg(w.cu + b), len = __ldg(w.cu + b + 1) - start;
+        const int start = w.cu[b], len = w.cu[b + 1] - start;
         it.plane = h;
         it.unit = b * w.H + h;
         if (start < 0 || len < 0 || start + len > w.N) {             // malformed offsets: touch nothing
