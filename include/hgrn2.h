@@ -89,16 +89,15 @@ typedef struct hgrn2_desc {
  * start of every chunk (derived from Eq. 3 by unrolling C steps) and, on the tensor-core
  * path, the two per-chunk decay totals of every key dimension.  The layout is private to the library (the
  * fp32 kernels work in chunks of 64 whatever C is and use a part of the buffer when C is smaller) and, on the
- * tensor-core path, for few long sequences that are not a whole number of chunks (which run as
- * segments), a little larger than one state per chunk: the size then depends on the current device,
- * and forward and backward of one buffer must run on devices with the same SM count.  0 on a bad desc. */
+ * tensor-core path, where sequences that are not a whole number of chunks run as segments, a little
+ * larger than one state per chunk: the size then depends on the current device, and forward and backward of one buffer must run on devices with the same SM count.  0 on a bad desc. */
 size_t hgrn2_saved_bytes(const hgrn2_desc *desc);
 
 /* Bytes of the workspace `ws` every call takes: a 256-byte status block, room for the
  * saved data that hgrn2_bwd re-creates when it is given saved = NULL and, on the tensor-core
- * path, scratch for running each sequence as several segments when the batch has too few
- * (batch, head) units to fill the GPU (the size therefore depends on the current device) and
- * one dk x dv float matrix per unit for units redone on the exact path.  0 on a bad desc. */
+ * path, scratch for running sequences as several segments where whole ones would leave SMs
+ * idle (the size therefore depends on the current device) and
+ * one dk x dv float matrix per unit or segment for what is redone on the exact path.  0 on a bad desc. */
 size_t hgrn2_workspace_bytes(const hgrn2_desc *desc);
 
 /* Forward over a whole sequence (Eq. 3 unrolled chunk by chunk; training and prefill).
@@ -282,8 +281,8 @@ hgrn2_status hgrn2_poll(const void *ws);
 /* Number of (batch, head) unit passes that the last tensor-core call using `ws` (a device pointer) redid on
  * the exact fp32 path because the unit's decay left the range described at the top of this file (Eq. 3 holds
  * on all of [0, 1]; the rescaled-operand form of the chunkwise products does not).  A backward that re-creates
- * its states (saved = NULL) counts a unit once for each of its two passes; few long sequences whose length is
- * not a whole number of 64-token chunks run as segments, each of which is redone and counted on its own.
+ * its states (saved = NULL) counts a unit once for each of its two passes; where sequences run as segments,
+ * each segment is redone and counted on its own.
  * Blocking copy: synchronise the
  * stream first.  0 on the fp32 kernels; -1 if `ws` is NULL or the copy failed. */
 int32_t hgrn2_exact_path_units(const void *ws);

@@ -78,7 +78,7 @@ hgrn2_status check_ptrs(const void *const *req, int nreq, const void *const *opt
 
 size_t state_bytes(const hgrn2_desc *d) { return (size_t)d->B * d->H * d->dk * d->dv * sizeof(float); }
 
-// packed = a variable-length batch: d->B sequences share d->N token rows per head (state slots: see PackedArgs)
+// packed = a variable-length batch: d->B sequences share d->N token rows per head (state slots: see WorkArgs)
 size_t saved_bytes_for(const hgrn2_desc *d, int C, bool packed = false)
 {
     if (use_tc(d)) return packed ? tc_saved_bytes_packed(d) : tc_saved_bytes(d, C);

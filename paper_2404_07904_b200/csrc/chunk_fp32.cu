@@ -66,7 +66,7 @@ struct Args {
 };
 
 // A unit's rows, chunks, first boundary slot.  Plain layout: unit u owns rows [u N, u N + N), slots from
-// (u - g0) NC.  Packed (see PackedArgs): head h, sequence b; slots from (h - g0) spp + cu[b] / 64 + b.
+// (u - g0) NC.  Packed: head h, sequence b; slots from (h - g0) spp + cu[b] / 64 + b.
 struct Where { long long row; int n, nc; long long slot, unit; };
 
 __device__ __forceinline__ Where packed_where(const Args &a, int b, long long h)
