@@ -20,8 +20,7 @@
 //
 // Warp roles (hand-offs are mbarriers, every wait is bounded; loops stay rolled to keep the
 // instruction footprint of the concurrently running roles small):
-//   T   4 warps: raw o, f tiles -> Qs, Ks in place, one chunk ahead (two TMA stages); paced so that it does not
-//       run alongside the output walk two chunks back;
+//   T   4 warps: raw o, f tiles -> Qs, Ks in place, one chunk ahead (two TMA stages);
 //   E1  4 warps: rescale the dS accumulator and publish its bf16 copy dS'' (the chain between chunks), R;
 //   E3  8 warps: d_o and d_f from dQs^T, dKs_intra^T, dKs_inter^T.  A thread owns (key dim, half of the chunk)
 //       and walks its 32 steps outwards from the middle, carrying the decay product and one running sum;
@@ -108,7 +107,6 @@ struct Ctl {
     alignas(16) ItemRing ring;
     int abort_flag;               // set by the first wait that runs out: every later wait returns at once
     uint32_t tmem_base;
-    int o_done;                   // E3 -> T: output walks finished so far, counted per warp (pacing only)
     int exact_flag;               // E1: a decay of this CTA's tokens left the range of the rescaled operands
     int l_stage, l_v, l_state, l_raw;   // L: fills asked for so far, per buffer, for the abort epilogue
 };
@@ -285,7 +283,6 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         mbar_init(&ctl->acc_free2, kE3Threads);
         mbar_init(&ctl->drain, 3);
         ctl->abort_flag = start_aborted;
-        ctl->o_done = 0;
         ctl->exact_flag = 0;
         ctl->l_stage = ctl->l_v = ctl->l_state = ctl->l_raw = 0;
         ring_init(ctl->ring, kRingWarps);
@@ -334,15 +331,9 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                 const int s = it % kStages;
                 uint8_t *qbuf = smem + s * kStageBytes;
                 mbar_wait(&ctl->full[s], (it / kStages) & 1, abort_flag);
-                // Pacing, not a data dependence: the transform of chunk `it` starts only when the output walk of chunk
-                // it - 2 is over (its completion pass may still run).  The tiles are there well before, but run earlier
-                // the transform shares the issue slots with that walk, the longest stretch of the per-chunk loop
-                // (event stamps: waiting for the completion pass as well made this the longest chain of the kernel;
-                // no pacing at all measured the same as this).
-                if (it >= 2) {
-                    if (lane == 0) count_wait(&ctl->o_done, kE3Warps * (it - 1), abort_flag);   // one poller per warp
-                    __syncwarp();
-                }
+                // No pacing: the transform of chunk `it` may run alongside the output walk of chunk it - 2.  (While A and
+                // dA waited for the state gradient, holding it back until that walk was over was 2 % faster; since they
+                // do not, it is 1 % slower: 128 units of 2048 tokens forward + backward 212 against 206 us, 592 of 512 256 against 252.)
                 PT_MARK(0)
                 PT_STAMP(status, 1, tid == 0 && it == 16) PT_STAMP(status, 20, tid == 0 && it == 18)
                 // Pm and E of the chunk are not kept: the backward takes them from what the forward saved
@@ -522,8 +513,6 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                 tc_fence_before_sync();
                 mbar_arrive(&ctl->acc_free1);
                 mbar_arrive(&ctl->parked);
-                __syncwarp();
-                if (lane == 0) atomicAdd(&ctl->o_done, 1);
                 PT_MARK(3)
                 PT_STAMP(status, 15, tid == kWarpE3 * 32 && it == 16)
                 // ---- d_f completed from the parked values, each thread its own 32 rows, once both halves' sums and R
