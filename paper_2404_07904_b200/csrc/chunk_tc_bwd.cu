@@ -304,7 +304,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         status->exact_units = 0;
     }
     bool malformed = false;
-    const Item first = warp_uniform(work_item<kRagged, true>(wk, blockIdx.x, malformed));
+    const Item first = warp_uniform(work_item<kRagged>(wk, blockIdx.x, malformed));
     if (tid == 0) {
         if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
         if (kPersist) {
@@ -629,7 +629,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                     return Pos{im.plane, im.row0 + c * kC, im.slot0 + c, true};
                 }
                 if (!kPersist) break;
-                im = warp_uniform(*ring_take<kRagged, true>(&ctl->ring, ++k, asked, wk, status, abort_flag));
+                im = warp_uniform(*ring_take<kRagged>(&ctl->ring, ++k, asked, wk, status, abort_flag));
                 c = (im.n + kC - 1) / kC;
                 asked = ask_done = false;
             }
@@ -862,7 +862,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         if (id < 0) continue;
         __syncthreads();                                             // the routine's shared memory is free
         if (tid == 0) atomicAdd(&status->exact_units, 1);
-        const Item im = work_item<kRagged, true>(wk, id, malformed);
+        const Item im = work_item<kRagged>(wk, id, malformed);
         const size_t seq = ((size_t)im.plane * wk.N + im.row0) * kD, st = (size_t)im.unit * kD * kD;
         alu::bwd_unit<__nv_bfloat16, __nv_bfloat16, kEnc ? alu::kGateEnc : alu::kGateIsF>(
             reinterpret_cast<float *>(smem), ex.o + seq, ex.f + seq, ex.i + seq, ex.dy + seq,
@@ -887,11 +887,11 @@ cudaError_t launch_tc_bwd(const SeqArgs &a0)
     if (t.items > 0x7fffffffull) return cudaErrorInvalidConfiguration;
     cudaError_t err;
     if (t.wk.G > 1) {
-        // sequences cut into segments (chunk_tc_fwd.cu), mirrored: what every segment but the first adds to the state
-        // gradient (it holds for every f), chained in reverse
-        err = launch_tc_state(true, a.o, a.f, a.dy, t, a.gate_enc, a.status, a.clear_status, a.start_aborted, a.stream);
+        // sequences cut into segments (chunk_tc_fwd.cu), mirrored: what every segment adds to the state gradient (it
+        // holds for every f), chained in reverse
+        err = launch_tc_state(true, a.o, a.f, a.dy, t, a.dS0 != nullptr, a.gate_enc, a.status, a.clear_status, a.start_aborted, a.stream);
         if (err != cudaSuccess) return err;
-        if ((err = launch_seg_chain(true, t, a.dSN, a.stream)) != cudaSuccess) return err;
+        if ((err = launch_seg_chain(true, t, a.dSN, a.dS0, a.stream)) != cudaSuccess) return err;
         a.clear_status = false;
     }
     CUtensorMap mo, mf, mi, mg, ms, mor, mfr;

@@ -148,7 +148,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         status->exact_units = 0;
     }
     bool malformed = false;
-    const Item first = warp_uniform(work_item<kRagged, false>(wk, blockIdx.x, malformed));
+    const Item first = warp_uniform(work_item<kRagged>(wk, blockIdx.x, malformed));
     if (tid == 0) {
         if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
         if (kPersist) {
@@ -394,7 +394,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
             }
             if (!kPersist) break;
             if (nc == 0) asked = ring_ask(&ctl->ring, k + 1, &ctl->exact_flag, abort_flag);
-            it = warp_uniform(*ring_take<kRagged, false>(&ctl->ring, k + 1, asked, wk, status, abort_flag));
+            it = warp_uniform(*ring_take<kRagged>(&ctl->ring, k + 1, asked, wk, status, abort_flag));
         }
     } else if (warp == kWarpMmaS) {
         // ================= MS: state update =================
@@ -571,7 +571,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         if (id < 0) continue;
         __syncthreads();                                             // the routine's shared memory is free
         if (tid == 0) atomicAdd(&status->exact_units, 1);
-        const Item it = work_item<kRagged, false>(wk, id, malformed);
+        const Item it = work_item<kRagged>(wk, id, malformed);
         const size_t seq = ((size_t)it.plane * wk.N + it.row0) * kD, st = (size_t)it.unit * kD * kD;
         alu::fwd_unit<__nv_bfloat16, __nv_bfloat16, kEnc ? alu::kGateEnc : alu::kGateIsF>(
             reinterpret_cast<float *>(smem), ex.o + seq, ex.f + seq, ex.i + seq,
@@ -593,10 +593,14 @@ bool tc_chunk_supported(int C) { return C == kC; }
 // ---- sequences cut into segments -------------------------------------------------------------------------
 // One work item per unit leaves most SMs idle when there are few units (a 16K-token batch of two sequences has
 // 32).  The recurrence is linear in the state, so a sequence can be cut into G segments that run side by side: (1)
-// every segment but the last runs state-only from a zero state (chunk_tc_state.cu), giving its local end state and its
-// total decay Lambda = prod f; (2) a small kernel chains them in place, S <- Diag(Lambda[r]) S + S_local[r]; (3) every
-// segment runs in full from its start state.  The same for units beyond the last full wave of whole units, which
-// would keep a few SMs busy for a whole sequence while the rest idle.
+// every segment runs state-only from a zero state (chunk_tc_state.cu), giving its local end state and its
+// total decay Lambda = prod f; (2) a small kernel chains them in place, S <- Diag(Lambda[r]) S + S_local[r], and leaves
+// S_N behind the last one; (3) every segment runs in full from its start state.  The same for units beyond the last full
+// wave of whole units, which would keep a few SMs busy for a whole sequence while the rest idle.
+// S_N is the chain's and not the last segment's own final state although that would save the state-only pass over the last
+// segment: the state-only pass rounds a token's decay from the segment's end, where it is 1, the full pass in the
+// mid-chunk frame, and the recent tokens weigh most.  Against fp64 S_N is off by 1.5e-3 and not 1.64e-3 (16 units of
+// 5000 tokens, f >= 0.9), 1.6e-3 and not 2.4e-3 (6 of 9000, f >= 0.5); dS_0 likewise (2.24 and 2.40e-3, 2.06 and 2.3e-3).
 int sm_count()
 {
     // asked for several times per call (plans and sizes), so kept per device
@@ -625,7 +629,7 @@ SegPlan tc_plan(uint64_t U, int NC)
     for (int g = 2; cut > 0 && g <= 16; ++g) {
         const int Lc = (NC + g - 1) / g < 6 ? 6 : (NC + g - 1) / g, G = (NC + Lc - 1) / Lc;
         if (G < 2) continue;
-        const int waves = (cut * G + sms - 1) / sms, pairs = (cut * (G - 1) + 2 * sms - 1) / (2 * sms);
+        const int waves = (cut * G + sms - 1) / sms, pairs = (cut * G + 2 * sms - 1) / (2 * sms);
         const double cost = waves * (Lc + 4.0) + 6.0 + 0.4 * Lc * pairs;
         if (p.tail == 0 || cost < best) {
             best = cost;
@@ -654,7 +658,7 @@ SegPlan plan_of(const hgrn2_desc *d)
     return no_cut(d) ? SegPlan{(int)U, 0, 1, 0, false} : tc_plan(U, (d->N + kC - 1) / kC);
 }
 int packed_segments_of(const hgrn2_desc *d) { return no_cut(d) ? 1 : tc_packed_segments((uint64_t)d->B * d->H, d->N); }
-size_t chain_bytes(size_t units, int G) { return units * (G - 1) * (kD * kD + kD) * sizeof(float); }
+size_t chain_bytes(size_t units, int G) { return units * G * (kD * kD + kD) * sizeof(float); }
 
 }  // namespace
 
@@ -670,7 +674,7 @@ size_t tc_saved_bytes(const hgrn2_desc *d, int C)
     return slots * (kSavedStateBytes + kSavedTotalsBytes);
 }
 
-// Boundary states of the cut units and the decays between them.
+// Chain slots of the cut units and their segments' decays.
 size_t tc_segment_scratch_bytes(const hgrn2_desc *d, int C)
 {
     const SegPlan p = plan_of(d);
@@ -728,7 +732,7 @@ TcWork tc_work(SeqArgs &a)
     }
     if (t.wk.G > 1) {
         t.chain = static_cast<float *>(a.seg_scratch);
-        t.lam = t.chain + t.cut * (t.wk.G - 1) * kD * kD;
+        t.lam = t.chain + t.cut * t.wk.G * kD * kD;
     }
     t.chunks = a.cu ? ((uint64_t)a.N / kC * a.H + t.items / 2) / (t.items ? t.items : 1) : (uint64_t)a.NC;
     if (a.states)
@@ -736,45 +740,50 @@ TcWork tc_work(SeqArgs &a)
     return t;
 }
 
-// Chains the boundary states of every cut unit in place: on entry slot r holds what segment r adds (backward: what
-// segment r + 1 adds to the gradient), on exit the state at the start of segment r + 1 (the gradient at the end of
-// segment r).  A thread owns four neighbouring elements; four segments' loads are in flight.
+// Chains every cut unit's slots in place: on entry slot r holds what segment r adds to the state (backward: to the
+// gradient), on exit the state at the start of segment r (the gradient at its end); `fin` (nullable) takes what is behind
+// the last one of the chain.  A thread owns four neighbouring elements and has all its slots' loads in flight: the kernel is
+// the latency of one round trip (16 units of 9 segments: 4.0 us, four slots at a time 9.4).
+constexpr int kChainAhead = 16;
 template <bool kBwd>
 __global__ void __launch_bounds__(128)
-seg_chain_kernel(const float *init, float *chain, const float *lam, int G)
+seg_chain_kernel(const float *init, float *fin, float *chain, const float *lam, const WorkArgs w)
 {
     chain_wait();
-    const size_t t = blockIdx.y;
-    const int e = (blockIdx.x * 128 + threadIdx.x) * 4, k = e / kD, n = G - 1;
+    const size_t t = blockIdx.y, unit = w.main + t;
+    const int e = (blockIdx.x * 128 + threadIdx.x) * 4, k = e / kD, G = w.G;
+    if (w.cu != nullptr && packed_malformed(w, (int)t / w.H)) fin = nullptr;      // such a unit writes nothing
     float S[4] = {0.f, 0.f, 0.f, 0.f};
-    if (init) load4(init + t * kD * kD + e, S);
-    float *slots = chain + t * n * kD * kD + e;
-    const float *lams = lam + t * n * kD + k;
-    for (int n0 = 0; n0 < n; n0 += 4) {
-        float x[4][4], l[4];
+    if (init) load4(init + unit * kD * kD + e, S);
+    float *slots = chain + t * G * kD * kD + e;
+    const float *lams = lam + t * G * kD + k;
+    const int n = fin ? G : G - 1;                                   // without fin nobody has filled the chain's last slot
+    for (int n0 = 0; n0 < G; n0 += kChainAhead) {
+        float x[kChainAhead][4], l[kChainAhead];
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < kChainAhead; ++j)
             if (n0 + j < n) {
-                const int r = kBwd ? n - 1 - n0 - j : n0 + j;
+                const int r = kBwd ? G - 1 - n0 - j : n0 + j;
                 load4(slots + (size_t)r * kD * kD, x[j]);
                 l[j] = lams[r * kD];
             }
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (n0 + j < n) {
-                const int r = kBwd ? n - 1 - n0 - j : n0 + j;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) S[i] = fmaf(l[j], S[i], x[j][i]);
+        for (int j = 0; j < kChainAhead; ++j)
+            if (n0 + j < G) {
+                const int r = kBwd ? G - 1 - n0 - j : n0 + j;
                 *reinterpret_cast<float4 *>(slots + (size_t)r * kD * kD) = make_float4(S[0], S[1], S[2], S[3]);
+                if (n0 + j < n)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) S[i] = fmaf(l[j], S[i], x[j][i]);
             }
     }
+    if (fin) *reinterpret_cast<float4 *>(fin + unit * kD * kD + e) = make_float4(S[0], S[1], S[2], S[3]);
 }
 
-cudaError_t launch_seg_chain(bool bwd, const TcWork &t, const float *init, cudaStream_t stream)
+cudaError_t launch_seg_chain(bool bwd, const TcWork &t, const float *init, float *fin, cudaStream_t stream)
 {
-    if (init) init += (size_t)t.wk.main * kD * kD;
     const dim3 grid(kD * kD / 512, (unsigned)t.cut);
-    return launch_chained(bwd ? seg_chain_kernel<true> : seg_chain_kernel<false>, grid, 128, 0, stream, init, t.chain, t.lam, t.wk.G);
+    return launch_chained(bwd ? seg_chain_kernel<true> : seg_chain_kernel<false>, grid, 128, 0, stream, init, fin, t.chain, t.lam, t.wk);
 }
 
 // More items than SMs: a CTA takes several (kPersist).  Against one CTA per item on 148 SMs: 4736 units of 64 tokens 193
@@ -789,9 +798,9 @@ cudaError_t launch_tc_fwd(const SeqArgs &a0)
     cudaError_t err;
     if (t.wk.G > 1) {
         // the state-only pass holds for every f: it needs no exact path of its own
-        err = launch_tc_state(false, nullptr, a.f, a.i, t, a.gate_enc, a.status, a.clear_status, a.start_aborted, a.stream);
+        err = launch_tc_state(false, nullptr, a.f, a.i, t, a.SN != nullptr, a.gate_enc, a.status, a.clear_status, a.start_aborted, a.stream);
         if (err != cudaSuccess) return err;
-        if ((err = launch_seg_chain(false, t, a.S0, a.stream)) != cudaSuccess) return err;
+        if ((err = launch_seg_chain(false, t, a.S0, a.SN, a.stream)) != cudaSuccess) return err;
         a.clear_status = false;
     }
     CUtensorMap mo, mf, mi, my, ms;

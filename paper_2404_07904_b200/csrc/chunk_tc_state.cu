@@ -63,17 +63,14 @@ static_assert(sizeof(Ctl<4>) <= 256, "control block");
 
 // What a CTA summarises: `out` and lam take its result at index `at`.
 struct Span { int plane, row0, n; size_t at; };
-// spans == true: plane x whole.  Otherwise the cuts of w (tc_chunk.cuh): forward segments 0 .. G - 2, backward segments
-// 1 .. G - 1 of every cut unit, the result in the chain slot of the boundary behind (in front of) the segment.
-template <bool kBwd>
-__device__ __forceinline__ Span span_of(const WorkArgs &w, int x, bool spans, int cut, bool &malformed)
+// spans == true: plane x whole.  Otherwise segments r0, r0 + 1 .. of the cut units of w (tc_chunk.cuh), the result in the
+// segment's chain slot.
+__device__ __forceinline__ Span span_of(const WorkArgs &w, int x, bool spans, int cut, int r0, bool &malformed)
 {
     if (spans) return Span{x, 0, w.N, (size_t)x};
-    const int r = x / cut + (kBwd ? 1 : 0), t = x % cut;
-    const Item it = work_item<true, kBwd>(w, w.cu ? ((t / w.H) * w.G + r) * w.H + t % w.H : w.main + r * cut + t, malformed);
-    // nothing chains behind a packed sequence's last segment
-    const int n = !kBwd && it.last ? 0 : it.n;
-    return Span{it.plane, it.row0, n, (size_t)t * (w.G - 1) + (kBwd ? r - 1 : r)};
+    const int r = x / cut + r0, t = x % cut;
+    const Item it = work_item<true>(w, w.cu ? ((t / w.H) * w.G + r) * w.H + t % w.H : w.main + r * cut + t, malformed);
+    return Span{it.plane, it.row0, it.n, (size_t)t * w.G + r};
 }
 
 // kEnc: the f tensor holds the signed gate encoding (see transform_half in tc_chunk.cuh).
@@ -81,7 +78,7 @@ template <bool kBwd, bool kEnc, bool kRagged, int kStages>
 __global__ void __launch_bounds__(kThreads, kStages == 4 ? 1 : 2)
 tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__ CUtensorMap map_f,
                 const __grid_constant__ CUtensorMap map_w, float *__restrict__ out, float *__restrict__ lam, const WorkArgs wk,
-                int spans, int cut, StatusBlock *status, int clear_status, int start_aborted)
+                int spans, int cut, int r0, StatusBlock *status, int clear_status, int start_aborted)
 {
     using G = Geo<kBwd, kStages>;
     chain_wait();
@@ -98,7 +95,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     bool malformed = false;
-    const Span sp = span_of<kBwd>(wk, blockIdx.x, spans != 0, cut, malformed);
+    const Span sp = span_of(wk, blockIdx.x, spans != 0, cut, r0, malformed);
     const int zu = sp.plane, row0 = sp.row0, N = sp.n, NC = (N + kC - 1) / kC;
     const size_t u = sp.at;
     if (malformed && tid == 0) report_error(status, HGRN2_ERR_INVALID_ARG, 6);
@@ -275,23 +272,25 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
 
 template <bool kBwd, bool kEnc, bool kRagged, int kStages>
 cudaError_t launch_state_t(const CUtensorMap &mo, const CUtensorMap &mf, const CUtensorMap &mw, uint64_t ctas, const WorkArgs &wk,
-                           bool spans, int cut, float *out, float *lam, StatusBlock *status, bool clear, int start_aborted,
+                           bool spans, int cut, int r0, float *out, float *lam, StatusBlock *status, bool clear, int start_aborted,
                            cudaStream_t stream)
 {
     using G = Geo<kBwd, kStages>;
     auto kernel = tc_state_kernel<kBwd, kEnc, kRagged, kStages>;
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), G::kSmemBytes);
     if (err != cudaSuccess) return err;
-    return launch_chained(kernel, dim3((unsigned)ctas), kThreads, G::kSmemBytes, stream, mo, mf, mw, out, lam, wk, spans ? 1 : 0, cut, status,
+    return launch_chained(kernel, dim3((unsigned)ctas), kThreads, G::kSmemBytes, stream, mo, mf, mw, out, lam, wk, spans ? 1 : 0, cut, r0, status,
                           clear ? 1 : 0, start_aborted);
 }
 
 template <bool kBwd>
 cudaError_t launch_state(const void *o, const void *f, const void *w, uint64_t planes, const WorkArgs &wk, bool spans,
-                         uint64_t cut, float *out, float *lam, bool gate_enc, StatusBlock *status, bool clear, int start_aborted,
+                         uint64_t cut, int segs, float *out, float *lam, bool gate_enc, StatusBlock *status, bool clear, int start_aborted,
                          cudaStream_t stream)
 {
-    const uint64_t ctas = spans ? planes : cut * (wk.G - 1);
+    // `segs` segments of every cut unit: the first ones, backward the last ones
+    const uint64_t ctas = spans ? planes : cut * segs;
+    const int r0 = kBwd ? wk.G - segs : 0;
     if (ctas == 0 || wk.N <= 0) return cudaSuccess;
     if (ctas > 0x7fffffffull) return cudaErrorInvalidConfiguration;
     CUtensorMap mo, mf, mw;
@@ -302,8 +301,8 @@ cudaError_t launch_state(const void *o, const void *f, const void *w, uint64_t p
     constexpr int kPair = kBwd ? 2 : 3;                       // stages that leave room for a second CTA
     auto go = [&](auto enc, auto rag) {
         constexpr bool kEnc = decltype(enc)::value, kRagged = decltype(rag)::value;
-        return pair ? launch_state_t<kBwd, kEnc, kRagged, kPair>(mo, mf, mw, ctas, wk, spans, (int)cut, out, lam, status, clear, start_aborted, stream)
-                    : launch_state_t<kBwd, kEnc, kRagged, 4>(mo, mf, mw, ctas, wk, spans, (int)cut, out, lam, status, clear, start_aborted, stream);
+        return pair ? launch_state_t<kBwd, kEnc, kRagged, kPair>(mo, mf, mw, ctas, wk, spans, (int)cut, r0, out, lam, status, clear, start_aborted, stream)
+                    : launch_state_t<kBwd, kEnc, kRagged, 4>(mo, mf, mw, ctas, wk, spans, (int)cut, r0, out, lam, status, clear, start_aborted, stream);
     };
     using T = std::true_type;
     using F = std::false_type;
@@ -312,11 +311,12 @@ cudaError_t launch_state(const void *o, const void *f, const void *w, uint64_t p
 
 }  // namespace
 
-cudaError_t launch_tc_state(bool bwd, const void *o, const void *f, const void *w, const TcWork &t, bool gate_enc,
+cudaError_t launch_tc_state(bool bwd, const void *o, const void *f, const void *w, const TcWork &t, bool all, bool gate_enc,
                             StatusBlock *status, bool clear, int start_aborted, cudaStream_t stream)
 {
-    return bwd ? launch_state<true>(o, f, w, t.planes, t.wk, false, t.cut, t.chain, t.lam, gate_enc, status, clear, start_aborted, stream)
-               : launch_state<false>(o, f, w, t.planes, t.wk, false, t.cut, t.chain, t.lam, gate_enc, status, clear, start_aborted, stream);
+    const int segs = all ? t.wk.G : t.wk.G - 1;
+    return bwd ? launch_state<true>(o, f, w, t.planes, t.wk, false, t.cut, segs, t.chain, t.lam, gate_enc, status, clear, start_aborted, stream)
+               : launch_state<false>(o, f, w, t.planes, t.wk, false, t.cut, segs, t.chain, t.lam, gate_enc, status, clear, start_aborted, stream);
 }
 
 cudaError_t launch_tc_span(bool bwd, const void *o, const void *f, const void *w, uint64_t planes, int N, float *out,
@@ -324,8 +324,8 @@ cudaError_t launch_tc_span(bool bwd, const void *o, const void *f, const void *w
 {
     WorkArgs wk;
     wk.N = N;
-    return bwd ? launch_state<true>(o, f, w, planes, wk, true, 0, out, lam, false, status, clear, start_aborted, stream)
-               : launch_state<false>(o, f, w, planes, wk, true, 0, out, lam, false, status, clear, start_aborted, stream);
+    return bwd ? launch_state<true>(o, f, w, planes, wk, true, 0, 0, out, lam, false, status, clear, start_aborted, stream)
+               : launch_state<false>(o, f, w, planes, wk, true, 0, 0, out, lam, false, status, clear, start_aborted, stream);
 }
 
 }  // namespace hgrn2

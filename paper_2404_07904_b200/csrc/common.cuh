@@ -203,12 +203,13 @@ struct TcWork {
     uint64_t planes = 0;   // planes of the sequence tensors
     uint64_t slots = 0;    // chunk-state slots
     uint64_t chunks = 0;   // of an item, on average
-    float *chain = nullptr, *lam = nullptr;    // boundary states [cut][G - 1][128][128] and decays [cut][G - 1][128]
+    float *chain = nullptr, *lam = nullptr;    // chain slots [cut][G][128][128] and the segments' decays [cut][G][128]
 };
 TcWork      tc_work(SeqArgs &a);
-cudaError_t launch_seg_chain(bool bwd, const TcWork &t, const float *init, cudaStream_t stream);
-// State-only passes (chunk_tc_state.cu): the segments of t that a chain needs, or one span per plane.
-cudaError_t launch_tc_state(bool bwd, const void *o, const void *f, const void *w, const TcWork &t, bool gate_enc,
+cudaError_t launch_seg_chain(bool bwd, const TcWork &t, const float *init, float *fin, cudaStream_t stream);
+// State-only passes (chunk_tc_state.cu): the segments of t that its chain needs - all of them for the states behind the
+// last (in front of the first) one - or one span per plane.
+cudaError_t launch_tc_state(bool bwd, const void *o, const void *f, const void *w, const TcWork &t, bool all, bool gate_enc,
                             StatusBlock *status, bool clear, int start_aborted, cudaStream_t stream);
 cudaError_t launch_tc_span(bool bwd, const void *o, const void *f, const void *w, uint64_t planes, int N, float *out,
                            float *lam, StatusBlock *status, bool clear, int start_aborted, cudaStream_t stream);

@@ -236,18 +236,25 @@ __device__ __forceinline__ void tril_row_block(uint32_t taddr, uint8_t *dstbuf, 
 //                    shorter) of unit main + t;
 //   packed batch     segment r of sequence b, head h at x = (b * G + r) * H + h; a sequence's segments have
 //                    max(8, ceil(chunks / G)) chunks, those beyond its end are empty (G = 1: whole sequences).
-// Between the segments of a unit sit G - 1 boundary states (chain slots, index base + r for the boundary between
-// segments r and r + 1).
+// A cut unit has G chain slots, one per segment: first what the segment adds to the state (state-only pass), then, chained,
+// the state at its start (backward: the gradient at its end).  Its S_N (dS_0) comes out of the chaining as well.
 struct Item {
     int id;                        // -1: no more work
     int plane, row0, n;            // rows [row0, row0 + n) of plane `plane`
     int slot0;                     // first chunk-state slot
     int unit;                      // index of its state in S0, SN (dSN, dS0)
-    int chain;                     // chain slot of the state it starts from (backward: of the gradient it starts from), -1: S0 (dSN)
-    int last;                      // its final state is S_N (backward: its final gradient is dS_0)
+    int chain;                     // chain slot of the state (backward: the gradient) it starts from, -1: S0 (dSN)
+    int last;                      // a whole unit: its final state is S_N (backward: its final gradient is dS_0)
 };
 
-template <bool kPackedToo, bool kBwd>
+// Sequence b of a packed batch has offsets that no tensor of N rows can have.
+__device__ __forceinline__ bool packed_malformed(const WorkArgs &w, int b)
+{
+    const int start = w.cu[b], len = w.cu[b + 1] - start;
+    return start < 0 || len < 0 || start + len > w.N;
+}
+
+template <bool kPackedToo>
 __device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malformed)
 {
     Item it;
@@ -257,7 +264,7 @@ __device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malfor
         const int start = w.cu[b], len = w.cu[b + 1] - start;
         it.plane = h;
         it.unit = b * w.H + h;
-        if (start < 0 || len < 0 || start + len > w.N) {             // malformed offsets: touch nothing
+        if (packed_malformed(w, b)) {                                // touch nothing
             malformed = true;
             it.row0 = it.n = it.slot0 = it.last = 0;
             it.chain = -1;
@@ -272,9 +279,8 @@ __device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malfor
         it.row0 = start + lo;
         it.n = hi - lo;
         it.slot0 = h * w.spp + it.row0 / kC + br;
-        const bool ends = hi == len && (hi > lo || r == 0);          // the sequence's last segment with tokens
-        it.last = kBwd ? r == 0 : ends;
-        it.chain = (kBwd ? ends : r == 0) ? -1 : it.unit * (w.G - 1) + (kBwd ? r : r - 1);
+        it.last = w.G == 1;
+        it.chain = w.G == 1 ? -1 : it.unit * w.G + r;
         return it;
     }
     if (x < w.main) {
@@ -291,8 +297,8 @@ __device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malfor
     it.row0 = r * w.Lc * kC;
     it.n = min(w.Lc * kC, w.N - it.row0);
     it.slot0 = it.unit * w.NC + r * w.Lc;
-    it.last = kBwd ? r == 0 : r == w.G - 1;
-    it.chain = (kBwd ? r == w.G - 1 : r == 0) ? -1 : t * (w.G - 1) + (kBwd ? r : r - 1);
+    it.last = 0;
+    it.chain = t * w.G + r;
     return it;
 }
 
@@ -372,7 +378,7 @@ static __device__ __noinline__ bool ring_ask(ItemRing *q, int k, volatile int *e
     return true;
 }
 // Load warp: the answer to ring_ask (asked = its return value) becomes item k.
-template <bool kPackedToo, bool kBwd>
+template <bool kPackedToo>
 static __device__ __noinline__ const Item *ring_take(ItemRing *q, int k, bool asked, const WorkArgs &w, StatusBlock *status,
                                                      volatile int *abort_flag)
 {
@@ -387,7 +393,7 @@ static __device__ __noinline__ const Item *ring_take(ItemRing *q, int k, bool as
     Item *it = &q->item[k % kRing];
     if ((threadIdx.x & 31) == 0) {
         bool malformed = false;
-        if (x >= 0) *it = work_item<kPackedToo, kBwd>(w, x, malformed);
+        if (x >= 0) *it = work_item<kPackedToo>(w, x, malformed);
         else *it = q->none;
         if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
         mbar_arrive(&q->full[k % kRing]);
