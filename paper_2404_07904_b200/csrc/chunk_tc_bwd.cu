@@ -109,6 +109,7 @@ struct Ctl {
     uint32_t tmem_base;
     int exact_flag;               // E1: a decay of this CTA's tokens left the range of the rescaled operands
     int l_stage, l_v, l_state, l_raw;   // L: fills asked for so far, per buffer, for the abort epilogue
+    int claimed;                  // redo_claim's answer
 };
 static_assert(sizeof(Ctl) <= 768, "control block");
 static_assert(kSmemBytes <= 232448, "shared memory budget");
@@ -229,7 +230,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
               const __grid_constant__ CUtensorMap map_i, const __grid_constant__ CUtensorMap map_dy,
               const __grid_constant__ CUtensorMap map_saved, const __grid_constant__ CUtensorMap map_o_raw,
               const __grid_constant__ CUtensorMap map_f_raw, const float *__restrict__ totals,
-              const float *__restrict__ dSN, const float *__restrict__ chain, __nv_bfloat16 *__restrict__ d_o,
+              const float *__restrict__ dSN, const float *__restrict__ chain, int *__restrict__ redo, __nv_bfloat16 *__restrict__ d_o,
               __nv_bfloat16 *__restrict__ d_f, __nv_bfloat16 *__restrict__ d_i, float *__restrict__ dS0,
               const __grid_constant__ WorkArgs wk, StatusBlock *status, int clear_status, const ExactArgs ex,
               int start_aborted)
@@ -309,6 +310,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
         if (kPersist) {
             ctl->ring.item[0] = first;
+            if (first.chain >= 0) ctl->ring.cuts[ctl->ring.n_cuts++] = first.id;
             mbar_arrive(&ctl->ring.full[0]);
         }
     }
@@ -854,22 +856,34 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 
-    // ---- exact path (see the forward kernel): flagged items are redone from their inputs, their saved chunk states and
-    // the gradient they started from by the pairwise-safe fp32 routine
-    if (ex.o == nullptr || !ctl->exact_flag || *abort_flag) return;
-    for (int j = 0; j < (kPersist ? 8 : 1); ++j) {
-        const int id = kPersist ? ctl->ring.flagged[j] - 1 : first.id;
-        if (id < 0) continue;
-        __syncthreads();                                             // the routine's shared memory is free
-        if (tid == 0) atomicAdd(&status->exact_units, 1);
-        const Item im = work_item<kRagged>(wk, id, malformed);
-        const size_t seq = ((size_t)im.plane * wk.N + im.row0) * kD, st = (size_t)im.unit * kD * kD;
-        alu::bwd_unit<__nv_bfloat16, __nv_bfloat16, kEnc ? alu::kGateEnc : alu::kGateIsF>(
-            reinterpret_cast<float *>(smem), ex.o + seq, ex.f + seq, ex.i + seq, ex.dy + seq,
-            im.chain >= 0 ? chain + (size_t)im.chain * kD * kD : (dSN ? dSN + st : nullptr),
-            ex.states + (size_t)im.slot0 * kD * kD, kC / kExactC, ex.scratch + (size_t)id * kD * kD, ex.d_o + seq,
-            ex.d_f + seq, ex.d_i + seq, dS0 != nullptr && im.last ? dS0 + st : nullptr, im.n, kD, kD, kExactC,
-            (im.n + kExactC - 1) / kExactC);
+    // ---- exact path (see the forward kernel): flagged items, or their units, are redone from their inputs, their saved
+    // chunk states and the gradient they started from by the pairwise-safe fp32 routine
+    if (ex.o == nullptr || *abort_flag) return;
+    const bool units = !kRagged && redo != nullptr;                  // there are segments of whole chunks
+    const int listed = kPersist ? 8 : 1, cuts = !units ? 0 : kPersist ? ctl->ring.n_cuts : first.chain >= 0 ? 1 : 0;
+    for (int j = ctl->exact_flag ? 0 : listed; j < listed + cuts; ++j) {
+        const bool claim = j >= listed;                              // flagged items, then the claims
+        const int id = kPersist ? (claim ? ctl->ring.cuts[j - listed] : ctl->ring.flagged[j] - 1) : first.id;
+        bool go = id >= 0 && !(units && id >= wk.main);
+        if (claim) {
+            if (tid == 0)
+                ctl->claimed = redo_claim(redo + 2 * ((id - wk.main) % wk.tail),
+                                          kPersist ? ring_flagged(ctl->ring, id) : ctl->exact_flag != 0, wk.G);
+            __syncthreads();
+            go = ctl->claimed != 0;
+        }
+        if (go) {
+            if (tid == 0) atomicAdd(&status->exact_units, 1);
+            const Item im = claim ? cut_unit(wk, id, wk.G - 1) : work_item<kRagged>(wk, id, malformed);
+            const size_t seq = ((size_t)im.plane * wk.N + im.row0) * kD, st = (size_t)im.unit * kD * kD;
+            alu::bwd_unit<__nv_bfloat16, __nv_bfloat16, kEnc ? alu::kGateEnc : alu::kGateIsF>(
+                reinterpret_cast<float *>(smem), ex.o + seq, ex.f + seq, ex.i + seq, ex.dy + seq,
+                im.chain >= 0 ? chain + (size_t)im.chain * kD * kD : (dSN ? dSN + st : nullptr),
+                ex.states + (size_t)im.slot0 * kD * kD, kC / kExactC, ex.scratch + (size_t)id * kD * kD, ex.d_o + seq,
+                ex.d_f + seq, ex.d_i + seq, dS0 != nullptr && im.last ? dS0 + st : nullptr, im.n, kD, kD, kExactC,
+                (im.n + kExactC - 1) / kExactC);
+        }
+        __syncthreads();                                             // the routine's shared memory, and the answer, are free
     }
 }
 
@@ -915,7 +929,7 @@ cudaError_t launch_tc_bwd(const SeqArgs &a0)
     ex.d_i = static_cast<__nv_bfloat16 *>(a.d_i);
     ex.states = reinterpret_cast<__nv_bfloat16 *>(a.states);
     ex.scratch = a.exact_scratch;
-    return launch_chained(kernel, dim3((unsigned)t.items), kThreads, kSmemBytes, a.stream, mo, mf, mi, mg, ms, mor, mfr, a.totals, a.dSN, t.chain, static_cast<__nv_bfloat16 *>(a.d_o), static_cast<__nv_bfloat16 *>(a.d_f), static_cast<__nv_bfloat16 *>(a.d_i), a.dS0, t.wk, a.status, a.clear_status ? 1 : 0, ex, a.start_aborted);
+    return launch_chained(kernel, dim3((unsigned)t.items), kThreads, kSmemBytes, a.stream, mo, mf, mi, mg, ms, mor, mfr, a.totals, a.dSN, t.chain, t.redo, static_cast<__nv_bfloat16 *>(a.d_o), static_cast<__nv_bfloat16 *>(a.d_f), static_cast<__nv_bfloat16 *>(a.d_i), a.dS0, t.wk, a.status, a.clear_status ? 1 : 0, ex, a.start_aborted);
 }
 
 }  // namespace hgrn2

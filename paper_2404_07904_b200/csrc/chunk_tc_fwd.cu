@@ -75,6 +75,7 @@ struct Ctl {
     uint32_t tmem_base;
     int exact_flag;              // E1: a decay of this CTA's tokens left the range of the rescaled operands
     int l_qf, l_v;               // L: chunks whose o, f tiles (i tile) have been asked for, for the abort epilogue
+    int claimed;                 // redo_claim's answer
 };
 static_assert(sizeof(Ctl) <= 768, "control block");
 static_assert(kSmemBytes <= 232448, "shared memory budget");
@@ -91,7 +92,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__ CUtensorMap map_f,
               const __grid_constant__ CUtensorMap map_i, const __grid_constant__ CUtensorMap map_y,
               const __grid_constant__ CUtensorMap map_saved, const float *__restrict__ S0, const float *__restrict__ chain,
-              float *__restrict__ SN, float *__restrict__ totals, int want_y, int want_saved,
+              int *__restrict__ redo, float *__restrict__ SN, float *__restrict__ totals, int want_y, int want_saved,
               const __grid_constant__ WorkArgs wk, StatusBlock *status, int clear_status, const ExactArgs ex,
               int start_aborted)
 {
@@ -153,6 +154,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
         if (kPersist) {
             ctl->ring.item[0] = first;
+            if (first.chain >= 0) ctl->ring.cuts[ctl->ring.n_cuts++] = first.id;
             mbar_arrive(&ctl->ring.full[0]);
         }
     }
@@ -563,21 +565,34 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 
-    // ---- exact path: the sweep met a decay its operands cannot represent, so the item is redone, from its inputs and
-    // the state it started from, by the pairwise-safe fp32 routine (every output of the item is overwritten)
-    if (ex.o == nullptr || !ctl->exact_flag || *abort_flag) return;
-    for (int j = 0; j < (kPersist ? 8 : 1); ++j) {
-        const int id = kPersist ? ctl->ring.flagged[j] - 1 : first.id;
-        if (id < 0) continue;
-        __syncthreads();                                             // the routine's shared memory is free
-        if (tid == 0) atomicAdd(&status->exact_units, 1);
-        const Item it = work_item<kRagged>(wk, id, malformed);
-        const size_t seq = ((size_t)it.plane * wk.N + it.row0) * kD, st = (size_t)it.unit * kD * kD;
-        alu::fwd_unit<__nv_bfloat16, __nv_bfloat16, kEnc ? alu::kGateEnc : alu::kGateIsF>(
-            reinterpret_cast<float *>(smem), ex.o + seq, ex.f + seq, ex.i + seq,
-            it.chain >= 0 ? chain + (size_t)it.chain * kD * kD : (S0 ? S0 + st : nullptr), ex.y ? ex.y + seq : nullptr,
-            SN != nullptr && it.last ? SN + st : nullptr, ex.states ? ex.states + (size_t)it.slot0 * kD * kD : nullptr,
-            kC / kExactC, it.n, kD, kD, kExactC, (it.n + kExactC - 1) / kExactC);
+    // ---- exact path: the sweep met a decay its operands cannot represent, so the item - or, for segments of whole chunks,
+    // the unit (redo_claim) - is redone, from its inputs and the state it started from, by the pairwise-safe fp32
+    // routine (every output of it is overwritten)
+    if (ex.o == nullptr || *abort_flag) return;
+    const bool units = !kRagged && redo != nullptr;                  // there are segments of whole chunks
+    const int listed = kPersist ? 8 : 1, cuts = !units ? 0 : kPersist ? ctl->ring.n_cuts : first.chain >= 0 ? 1 : 0;
+    for (int j = ctl->exact_flag ? 0 : listed; j < listed + cuts; ++j) {
+        const bool claim = j >= listed;                              // flagged items, then the claims
+        const int id = kPersist ? (claim ? ctl->ring.cuts[j - listed] : ctl->ring.flagged[j] - 1) : first.id;
+        bool go = id >= 0 && !(units && id >= wk.main);
+        if (claim) {
+            if (tid == 0)
+                ctl->claimed = redo_claim(redo + 2 * ((id - wk.main) % wk.tail),
+                                          kPersist ? ring_flagged(ctl->ring, id) : ctl->exact_flag != 0, wk.G);
+            __syncthreads();
+            go = ctl->claimed != 0;
+        }
+        if (go) {
+            if (tid == 0) atomicAdd(&status->exact_units, 1);
+            const Item it = claim ? cut_unit(wk, id, 0) : work_item<kRagged>(wk, id, malformed);
+            const size_t seq = ((size_t)it.plane * wk.N + it.row0) * kD, st = (size_t)it.unit * kD * kD;
+            alu::fwd_unit<__nv_bfloat16, __nv_bfloat16, kEnc ? alu::kGateEnc : alu::kGateIsF>(
+                reinterpret_cast<float *>(smem), ex.o + seq, ex.f + seq, ex.i + seq,
+                it.chain >= 0 ? chain + (size_t)it.chain * kD * kD : (S0 ? S0 + st : nullptr), ex.y ? ex.y + seq : nullptr,
+                SN != nullptr && it.last ? SN + st : nullptr, ex.states ? ex.states + (size_t)it.slot0 * kD * kD : nullptr,
+                kC / kExactC, it.n, kD, kD, kExactC, (it.n + kExactC - 1) / kExactC);
+        }
+        __syncthreads();                                             // the routine's shared memory, and the answer, are free
     }
 }
 
@@ -658,7 +673,7 @@ SegPlan plan_of(const hgrn2_desc *d)
     return no_cut(d) ? SegPlan{(int)U, 0, 1, 0, false} : tc_plan(U, (d->N + kC - 1) / kC);
 }
 int packed_segments_of(const hgrn2_desc *d) { return no_cut(d) ? 1 : tc_packed_segments((uint64_t)d->B * d->H, d->N); }
-size_t chain_bytes(size_t units, int G) { return units * G * (kD * kD + kD) * sizeof(float); }
+size_t chain_bytes(size_t units, int G) { return units * G * (kD * kD + kD) * sizeof(float) + ((units * 2 * sizeof(int) + 15) & ~(size_t)15); }
 
 }  // namespace
 
@@ -674,7 +689,7 @@ size_t tc_saved_bytes(const hgrn2_desc *d, int C)
     return slots * (kSavedStateBytes + kSavedTotalsBytes);
 }
 
-// Chain slots of the cut units and their segments' decays.
+// Chain slots of the cut units, their segments' decays and what redo_claim counts.
 size_t tc_segment_scratch_bytes(const hgrn2_desc *d, int C)
 {
     const SegPlan p = plan_of(d);
@@ -733,6 +748,7 @@ TcWork tc_work(SeqArgs &a)
     if (t.wk.G > 1) {
         t.chain = static_cast<float *>(a.seg_scratch);
         t.lam = t.chain + t.cut * t.wk.G * kD * kD;
+        if (!a.cu && a.N % kC == 0) t.redo = reinterpret_cast<int *>(t.lam + t.cut * t.wk.G * kD);
     }
     t.chunks = a.cu ? ((uint64_t)a.N / kC * a.H + t.items / 2) / (t.items ? t.items : 1) : (uint64_t)a.NC;
     if (a.states)
@@ -747,11 +763,12 @@ TcWork tc_work(SeqArgs &a)
 constexpr int kChainAhead = 16;
 template <bool kBwd>
 __global__ void __launch_bounds__(128)
-seg_chain_kernel(const float *init, float *fin, float *chain, const float *lam, const WorkArgs w)
+seg_chain_kernel(const float *init, float *fin, float *chain, const float *lam, int *redo, const WorkArgs w)
 {
     chain_wait();
     const size_t t = blockIdx.y, unit = w.main + t;
     const int e = (blockIdx.x * 128 + threadIdx.x) * 4, k = e / kD, G = w.G;
+    if (redo != nullptr && blockIdx.x == 0 && threadIdx.x < 2) redo[2 * t + threadIdx.x] = 0;
     if (w.cu != nullptr && packed_malformed(w, (int)t / w.H)) fin = nullptr;      // such a unit writes nothing
     float S[4] = {0.f, 0.f, 0.f, 0.f};
     if (init) load4(init + unit * kD * kD + e, S);
@@ -783,7 +800,7 @@ seg_chain_kernel(const float *init, float *fin, float *chain, const float *lam, 
 cudaError_t launch_seg_chain(bool bwd, const TcWork &t, const float *init, float *fin, cudaStream_t stream)
 {
     const dim3 grid(kD * kD / 512, (unsigned)t.cut);
-    return launch_chained(bwd ? seg_chain_kernel<true> : seg_chain_kernel<false>, grid, 128, 0, stream, init, fin, t.chain, t.lam, t.wk);
+    return launch_chained(bwd ? seg_chain_kernel<true> : seg_chain_kernel<false>, grid, 128, 0, stream, init, fin, t.chain, t.lam, t.redo, t.wk);
 }
 
 // More items than SMs: a CTA takes several (kPersist).  Against one CTA per item on 148 SMs: 4736 units of 64 tokens 193
@@ -822,7 +839,7 @@ cudaError_t launch_tc_fwd(const SeqArgs &a0)
     ex.i = static_cast<const __nv_bfloat16 *>(a.i);
     ex.y = static_cast<__nv_bfloat16 *>(a.y);
     ex.states = reinterpret_cast<__nv_bfloat16 *>(a.states);
-    return launch_chained(kernel, dim3((unsigned)t.items), kThreads, kSmemBytes, a.stream, mo, mf, mi, my, ms, a.S0, t.chain, a.SN, want_saved ? a.totals : nullptr, want_y, want_saved, t.wk, a.status, a.clear_status ? 1 : 0, ex, a.start_aborted);
+    return launch_chained(kernel, dim3((unsigned)t.items), kThreads, kSmemBytes, a.stream, mo, mf, mi, my, ms, a.S0, t.chain, t.redo, a.SN, want_saved ? a.totals : nullptr, want_y, want_saved, t.wk, a.status, a.clear_status ? 1 : 0, ex, a.start_aborted);
 }
 
 }  // namespace hgrn2

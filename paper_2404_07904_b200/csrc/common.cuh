@@ -204,6 +204,7 @@ struct TcWork {
     uint64_t slots = 0;    // chunk-state slots
     uint64_t chunks = 0;   // of an item, on average
     float *chain = nullptr, *lam = nullptr;    // chain slots [cut][G][128][128] and the segments' decays [cut][G][128]
+    int *redo = nullptr;   // whole-chunk sequences: [cut][2], see redo_claim (tc_chunk.cuh)
 };
 TcWork      tc_work(SeqArgs &a);
 cudaError_t launch_seg_chain(bool bwd, const TcWork &t, const float *init, float *fin, cudaStream_t stream);

@@ -302,6 +302,13 @@ __device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malfor
     return it;
 }
 
+// The whole unit of which item x is a segment, starting from what its chain slot r holds.
+__device__ __forceinline__ Item cut_unit(const WorkArgs &w, int x, int r)
+{
+    const int t = (x - w.main) % w.tail, unit = w.main + t;
+    return Item{x, unit, 0, w.N, unit * w.NC, unit, t * w.G + r, 1};
+}
+
 // kPersist instantiations: a CTA works through several items, one after the other with all pipelines running on: the
 // first is its own block index, the others are taken from CTAs of the grid that have not started (cluster launch
 // control), so a launch of many short items pays a CTA's start-up and pipeline fill once per SM and keeps the hardware's
@@ -310,6 +317,7 @@ __device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malfor
 // read.  All of this is out of line: the roles run concurrently, and their combined code is about what the instruction
 // cache holds (which is also why the other instantiations know nothing of it).
 constexpr int kRing = 4;           // the load warp is at most this many items ahead of the slowest role
+constexpr int kMaxCuts = 8;        // a CTA takes no further items once it has had this many segments
 struct ItemRing {
     Item item[kRing], none;
     uint4 answer;                  // cluster launch control response (16-byte aligned)
@@ -317,6 +325,7 @@ struct ItemRing {
     uint64_t empty[kRing];         // one lane per warp -> load warp
     uint64_t answered;             // the hardware's response has landed
     int flagged[8];                // items (index + 1) whose decay left the operands' range, by position mod 8
+    int cuts[kMaxCuts], n_cuts;    // the CTA's items that are segments (redo_claim)
     int asked;                     // responses asked for so far, for the abort epilogue
 };
 __device__ __forceinline__ void ring_init(ItemRing &q, int warps)
@@ -328,6 +337,7 @@ __device__ __forceinline__ void ring_init(ItemRing &q, int warps)
     mbar_init(&q.answered, 1);
     for (int j = 0; j < 8; ++j) q.flagged[j] = 0;
     q.asked = 0;
+    q.n_cuts = 0;
     q.none = Item{-1, 0, 0, 0, 0, 0, -1, 0};
 }
 // The same item in every lane, in a form that tells the compiler so: the loops over its chunks stay convergent code
@@ -368,7 +378,7 @@ __device__ __forceinline__ bool next_item(ItemRing *q, int k, volatile int *abor
 static __device__ __noinline__ bool ring_ask(ItemRing *q, int k, volatile int *exact_flag, volatile int *abort_flag)
 {
     if (k >= kRing) mbar_wait(&q->empty[k % kRing], (k / kRing - 1) & 1, abort_flag);
-    if (__any_sync(0xffffffffu, *exact_flag || *abort_flag)) return false;
+    if (__any_sync(0xffffffffu, *exact_flag || *abort_flag || q->n_cuts >= kMaxCuts)) return false;
     mbar_arrive_expect_tx(&q->answered, 16);
     if ((threadIdx.x & 31) == 0) {
         clc_try_cancel(&q->answer, &q->answered);
@@ -395,11 +405,31 @@ static __device__ __noinline__ const Item *ring_take(ItemRing *q, int k, bool as
         bool malformed = false;
         if (x >= 0) *it = work_item<kPackedToo>(w, x, malformed);
         else *it = q->none;
+        if (it->chain >= 0) q->cuts[q->n_cuts++] = x;
         if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
         mbar_arrive(&q->full[k % kRing]);
     }
     __syncwarp();
     return it;
+}
+
+// The exact path of a unit that runs as segments of whole chunks: the last of its G CTAs to finish redoes the whole unit,
+// from its S_0 (dS_N), if any of them met a decay out of range, so S_N, dS_0 and every output are what they are for a unit
+// that is not cut (redone segment by segment they would carry the state-only pass's bf16 operands).  redo = the
+// unit's {flag, count}, zeroed by the chaining.  Called by one thread behind a barrier, its CTA's outputs complete.
+__device__ __forceinline__ int redo_claim(int *redo, bool flagged, int G)
+{
+    if (flagged) atomicOr(redo, 1);
+    __threadfence();
+    if (atomicAdd(redo + 1, 1) != G - 1) return 0;
+    __threadfence();
+    return atomicOr(redo, 0);
+}
+__device__ __forceinline__ bool ring_flagged(const ItemRing &q, int id)
+{
+    bool hit = false;
+    for (int j = 0; j < 8; ++j) hit |= q.flagged[j] == id + 1;
+    return hit;
 }
 
 // ---- host side: tensor maps ---------------------------------------------------------------------
