@@ -296,16 +296,19 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         // ================= E2: output warps =================
         const int t = 16 * sub + lane;                               // accumulator row of lanes 0..15
         PT_DECL
-        // step g: tril(A(g)) -> operand slab | Y(g-1) -> staging tile; what is left behind the last chunk follows then
+        // A step: tril(A(g)) -> operand slab | Y(g-1) -> staging tile.  Y(g-1) is not held back over an item without tokens:
+        // the store warp cannot give its item up before it has the tile, and no item kRing further on is published before
+        // it has, so this role would wait for an item that waits for this role.
         int left = 0;
-        for (int g = 0, k = 0;; ++g, --left) {
-            bool more = true;
-            while (left == 0 && more) {
+        bool more = true, held = false;                              // held: Y(g-1) is still to be staged
+        for (int g = 0, k = 0; more;) {
+            if (left == 0) {
                 Item it;
                 more = next_item<kPersist>(&ctl->ring, k++, abort_flag, first, it);
                 left = more && want_y ? (it.n + kC - 1) / kC : 0;
             }
-            if (more) {
+            const bool chunk = left > 0;
+            if (chunk) {
                 const int b = g & 1;
                 mbar_wait(&ctl->barA[b], (g >> 1) & 1, abort_flag);
                 PT_MARK(0)
@@ -318,7 +321,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                 mbar_arrive(&ctl->p_ready[b]);
                 PT_MARK(1)
             }
-            if (g >= 1) {
+            if (held) {
                 const int b = (g - 1) & 1;
                 mbar_wait(&ctl->barY[b], ((g - 1) >> 1) & 1, abort_flag);
                 PT_MARK(2)
@@ -344,7 +347,11 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                 mbar_arrive(&ctl->y_staged);
                 PT_MARK(4)
             }
-            if (!more) break;
+            held = chunk;
+            if (chunk) {
+                ++g;
+                --left;
+            }
         }
         PT_DUMP(status, 7, 5, tid == kWarpE2 * 32)
     } else if (warp == kWarpLoad) {

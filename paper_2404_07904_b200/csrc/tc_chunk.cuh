@@ -314,7 +314,10 @@ __device__ __forceinline__ Item cut_unit(const WorkArgs &w, int x, int r)
 // control), so a launch of many short items pays a CTA's start-up and pipeline fill once per SM and keeps the hardware's
 // dynamic balance.  The load warp takes them - as late as it can, when it asks for its current item's last tiles, so
 // that an SM with a long item does not hoard another one - and publishes them in a ring that every role's warps
-// read.  All of this is out of line: the roles run concurrently, and their combined code is about what the instruction
+// read.  Item k + kRing is not published before every warp has given up item k, and any number of items in a row may be
+// without tokens: so a role may hold back work that another one needs to finish an item (its last output, its last loads)
+// only while it asks for the item right behind it.
+// All of this is out of line: the roles run concurrently, and their combined code is about what the instruction
 // cache holds (which is also why the other instantiations know nothing of it).
 constexpr int kRing = 4;           // the load warp is at most this many items ahead of the slowest role
 constexpr int kMaxCuts = 8;        // a CTA takes no further items once it has had this many segments
