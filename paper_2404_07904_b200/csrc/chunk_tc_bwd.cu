@@ -620,8 +620,9 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         Item im = first;
         int k = 0, c = (im.n + kC - 1) / kC;
         bool asked = false, ask_done = false;
+        // The next chunk, of this item or the one behind it; not ok: that one is empty, or (im.id < 0) there is none.
         auto advance = [&]() -> Pos {
-            while (im.id >= 0) {
+            for (int step = 0; step < 2 && im.id >= 0; ++step) {
                 if (kPersist && c <= 2 && !ask_done) {          // two chunks ahead: the answer takes about a microsecond
                     asked = ring_ask(&ctl->ring, k + 1, &ctl->exact_flag, abort_flag);
                     ask_done = true;
@@ -630,12 +631,18 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                     --c;
                     return Pos{im.plane, im.row0 + c * kC, im.slot0 + c, true};
                 }
-                if (!kPersist) break;
+                if (!kPersist || step > 0) break;
                 im = warp_uniform(*ring_take<kRagged>(&ctl->ring, ++k, asked, wk, status, abort_flag));
                 c = (im.n + kC - 1) / kC;
                 asked = ask_done = false;
             }
             return Pos{0, 0, 0, false};
+        };
+        // Any further: only with nothing of a chunk left to be asked for.  The roles cannot finish that chunk's item without
+        // it, and an item kRing further on cannot be asked for before they have (tc_chunk.cuh).
+        auto over_empty = [&](Pos p) -> Pos {
+            while (kPersist && !p.ok && im.id >= 0) p = advance();
+            return p;
         };
         auto issue_stage = [&](const Pos &p) {
             const int s = n_stage++ % kStages;
@@ -671,7 +678,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         // A barrier must never be armed twice within one phase.  Normally a buffer's previous fill has long been
         // consumed when its readers report; on the time-out exit those waits return at once, so before every
         // refill the previous fill is waited for explicitly (one poll that succeeds at once in normal running).
-        Pos next = advance();
+        Pos next = over_empty(advance());
         if (next.ok) issue_stage(next);
         for (int it = 0; next.ok; ++it) {
             if (it > 0) {
@@ -680,7 +687,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                 mbar_wait_drain(&ctl->vfull, (it - 1) & 1, 20000000ull);
             }
             issue_v(next);
-            const Pos after = advance();
+            Pos after = advance();
             if (it > 0) {
                 mbar_wait(&ctl->r_ready[(it - 1) & 1], ((it - 1) >> 1) & 1, abort_flag);   // R has read S' ...
                 mbar_wait(&ctl->barY2, (it - 1) & 1, abort_flag);    // ... and so have the chunk's products;
@@ -696,6 +703,13 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                 mbar_wait_drain(&ctl->rawfull, (it - 1) & 1, 20000000ull);
             }
             issue_raw(next);
+            if (kPersist && !after.ok) {
+                after = over_empty(after);
+                if (after.ok) {
+                    if (it > 0) mbar_wait_drain(&ctl->full[(it - 1) % kStages], ((it - 1) / kStages) & 1, 20000000ull);
+                    issue_stage(after);
+                }
+            }
             next = after;
         }
         ctl->l_stage = n_stage; ctl->l_v = n_v; ctl->l_state = n_state; ctl->l_raw = n_raw;

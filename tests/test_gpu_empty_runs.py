@@ -40,3 +40,13 @@ def test_forward_over_runs_of_empty_sequences(name):
     G.assert_close({"y": y.float().cpu().numpy(), "SN": SN.cpu().numpy()}, {k: want[k] for k in ("y", "SN")}, TOL, name)
     empty = [b for b, n in enumerate(RUNS[name]) if n == 0]
     np.testing.assert_array_equal(SN.cpu().numpy()[empty], inp["S0"][empty])
+
+
+@pytest.mark.parametrize("use_saved", [True, False])
+@pytest.mark.parametrize("name", RUNS)
+def test_backward_over_runs_of_empty_sequences(name, use_saved):
+    inp = _inputs(RUNS[name])
+    got, _ = TV._run_gpu(inp, "bf16", use_saved=use_saved)
+    G.assert_close(got, TV._oracle(inp), TOL, name)
+    empty = [b for b, n in enumerate(RUNS[name]) if n == 0]
+    np.testing.assert_array_equal(got["dS0"][empty], inp["dSN"][empty])
