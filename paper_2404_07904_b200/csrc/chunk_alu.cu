@@ -21,9 +21,8 @@ __device__ inline Geom unit_geom(long long u, int N, int C, int NC, const int *c
     if (cu == nullptr) return Geom{u * N, N, NC, u * NC};
     const int B = gridDim.x / H;
     const int b = (int)(u / H), h = (int)(u - (long long)b * H);
-    const int start = cu[b];
-    int n = cu[b + 1] - start;
-    if (start < 0 || n < 0 || start + n > N) n = 0;          // malformed offsets: touch nothing
+    const int start = cu[b], end = cu[b + 1];
+    const int n = rows_malformed(start, end, N) ? 0 : end - start;       // malformed offsets: touch nothing
     return Geom{(long long)h * N + start, n, (n + C - 1) / C, (long long)h * (N / C + B + 1) + start / C + b};
 }
 

@@ -71,9 +71,8 @@ struct Where { long long row; int n, nc; long long slot, unit; };
 
 __device__ __forceinline__ Where packed_where(const Args &a, int b, long long h)
 {
-    const int start = a.cu[b];
-    int n = a.cu[b + 1] - start;
-    if (start < 0 || n < 0 || start + n > a.N) n = 0;          // malformed offsets: touch nothing
+    const int start = a.cu[b], end = a.cu[b + 1];
+    const int n = rows_malformed(start, end, a.N) ? 0 : end - start;     // malformed offsets: touch nothing
     return Where{h * a.N + start, n, (n + kL - 1) / kL, (h - a.g0) * a.spp + start / kL + b, b * (long long)a.H + h};
 }
 

@@ -129,6 +129,9 @@ inline cudaError_t ensure_dynamic_smem(const void *kernel, size_t bytes)
     return err;
 }
 
+// Rows [start, end) of a packed sequence cannot be rows of a tensor of N.  (end - start may leave int's range.)
+__device__ __forceinline__ bool rows_malformed(int start, int end, int N) { return start < 0 || end < start || end > N; }
+
 // ---- internal launchers (defined in the .cu files, called from api.cu) ----------------------
 
 struct SeqArgs {

@@ -250,8 +250,7 @@ struct Item {
 // Sequence b of a packed batch has offsets that no tensor of N rows can have.
 __device__ __forceinline__ bool packed_malformed(const WorkArgs &w, int b)
 {
-    const int start = w.cu[b], len = w.cu[b + 1] - start;
-    return start < 0 || len < 0 || start + len > w.N;
+    return rows_malformed(w.cu[b], w.cu[b + 1], w.N);
 }
 
 template <bool kPackedToo>
@@ -261,7 +260,6 @@ __device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malfor
     it.id = x;
     if (kPackedToo && w.cu != nullptr) {
         const int h = x % w.H, br = x / w.H, b = br / w.G, r = br - b * w.G;
-        const int start = w.cu[b], len = w.cu[b + 1] - start;
         it.plane = h;
         it.unit = b * w.H + h;
         if (packed_malformed(w, b)) {                                // touch nothing
@@ -270,6 +268,7 @@ __device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malfor
             it.chain = -1;
             return it;
         }
+        const int start = w.cu[b], len = w.cu[b + 1] - start;
         int lo = 0, hi = len;
         if (w.G > 1) {
             const int Lc = max(8, ((len + kC - 1) / kC + w.G - 1) / w.G);
