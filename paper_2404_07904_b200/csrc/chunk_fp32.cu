@@ -256,11 +256,7 @@ fp32_local_kernel(const Args a)
     extern __shared__ __align__(16) float sm[];
     float *sX = sm, *sV = sm + kL * TK, *sprod = sV + kL * TV;
     chain_wait();
-    if (a.status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) {
-        a.status->code = 0;
-        a.status->where = 0;
-        a.status->exact_units = 0;
-    }
+    if (a.status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) clear_block(a.status);
     Where w;
     int c;
     if (!chunk_of(a, w, c)) return;

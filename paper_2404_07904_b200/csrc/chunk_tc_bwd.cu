@@ -238,12 +238,10 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     extern __shared__ __align__(1024) uint8_t smem[];
     if (smem_u32(smem) & 1023u) {          // every byte is spoken for: the swizzled tiles need the base aligned
         chain_wait();
-        if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
-            status->code = 0;
-            status->where = 0;
-            status->exact_units = 0;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            if (clear_status) clear_block(status);
+            report_error(status, HGRN2_ERR_CUDA, 3);
         }
-        if (threadIdx.x == 0) report_error(status, HGRN2_ERR_CUDA, 3);
         return;
     }
     uint8_t *sbuf = smem + kOffS;
@@ -298,21 +296,12 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     }
     if (warp == 0) tmem_alloc(&ctl->tmem_base, kTmemCols);
     chain_wait();
-    // the first kernel of a call zeroes the status word (errors are reported seconds later, after a wait ran out)
-    if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
-        status->code = 0;
-        status->where = 0;
-        status->exact_units = 0;
-    }
-    bool malformed = false;
-    const Item first = warp_uniform(work_item<kRagged>(wk, blockIdx.x, malformed));
-    if (tid == 0) {
-        if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
-        if (kPersist) {
-            ctl->ring.item[0] = first;
-            if (first.chain >= 0) ctl->ring.cuts[ctl->ring.n_cuts++] = first.id;
-            mbar_arrive(&ctl->ring.full[0]);
-        }
+    if (clear_status && blockIdx.x == 0) begin_call(status, kRagged ? wk.cu : nullptr, wk.B, wk.N);
+    const Item first = warp_uniform(work_item<kRagged>(wk, blockIdx.x));
+    if (kPersist && tid == 0) {
+        ctl->ring.item[0] = first;
+        if (first.chain >= 0) ctl->ring.cuts[ctl->ring.n_cuts++] = first.id;
+        mbar_arrive(&ctl->ring.full[0]);
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -632,7 +621,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                     return Pos{im.plane, im.row0 + c * kC, im.slot0 + c, true};
                 }
                 if (!kPersist || step > 0) break;
-                im = warp_uniform(*ring_take<kRagged>(&ctl->ring, ++k, asked, wk, status, abort_flag));
+                im = warp_uniform(*ring_take<kRagged>(&ctl->ring, ++k, asked, wk, abort_flag));
                 c = (im.n + kC - 1) / kC;
                 asked = ask_done = false;
             }
@@ -888,7 +877,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         }
         if (go) {
             if (tid == 0) atomicAdd(&status->exact_units, 1);
-            const Item im = claim ? cut_unit(wk, id, wk.G - 1) : work_item<kRagged>(wk, id, malformed);
+            const Item im = claim ? cut_unit(wk, id, wk.G - 1) : work_item<kRagged>(wk, id);
             const size_t seq = ((size_t)im.plane * wk.N + im.row0) * kD, st = (size_t)im.unit * kD * kD;
             alu::bwd_unit<__nv_bfloat16, __nv_bfloat16, kEnc ? alu::kGateEnc : alu::kGateIsF>(
                 reinterpret_cast<float *>(smem), ex.o + seq, ex.f + seq, ex.i + seq, ex.dy + seq,

@@ -142,21 +142,12 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
     }
     if (warp == 0) tmem_alloc(&ctl->tmem_base, kTmemCols);
     chain_wait();
-    // the first kernel of a call zeroes the status word (errors are reported seconds later, after a wait ran out)
-    if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
-        status->code = 0;
-        status->where = 0;
-        status->exact_units = 0;
-    }
-    bool malformed = false;
-    const Item first = warp_uniform(work_item<kRagged>(wk, blockIdx.x, malformed));
-    if (tid == 0) {
-        if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
-        if (kPersist) {
-            ctl->ring.item[0] = first;
-            if (first.chain >= 0) ctl->ring.cuts[ctl->ring.n_cuts++] = first.id;
-            mbar_arrive(&ctl->ring.full[0]);
-        }
+    if (clear_status && blockIdx.x == 0) begin_call(status, kRagged ? wk.cu : nullptr, wk.B, wk.N);
+    const Item first = warp_uniform(work_item<kRagged>(wk, blockIdx.x));
+    if (kPersist && tid == 0) {
+        ctl->ring.item[0] = first;
+        if (first.chain >= 0) ctl->ring.cuts[ctl->ring.n_cuts++] = first.id;
+        mbar_arrive(&ctl->ring.full[0]);
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -403,7 +394,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
             }
             if (!kPersist) break;
             if (nc == 0) asked = ring_ask(&ctl->ring, k + 1, &ctl->exact_flag, abort_flag);
-            it = warp_uniform(*ring_take<kRagged>(&ctl->ring, k + 1, asked, wk, status, abort_flag));
+            it = warp_uniform(*ring_take<kRagged>(&ctl->ring, k + 1, asked, wk, abort_flag));
         }
     } else if (warp == kWarpMmaS) {
         // ================= MS: state update =================
@@ -591,7 +582,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
         }
         if (go) {
             if (tid == 0) atomicAdd(&status->exact_units, 1);
-            const Item it = claim ? cut_unit(wk, id, 0) : work_item<kRagged>(wk, id, malformed);
+            const Item it = claim ? cut_unit(wk, id, 0) : work_item<kRagged>(wk, id);
             const size_t seq = ((size_t)it.plane * wk.N + it.row0) * kD, st = (size_t)it.unit * kD * kD;
             alu::fwd_unit<__nv_bfloat16, __nv_bfloat16, kEnc ? alu::kGateEnc : alu::kGateIsF>(
                 reinterpret_cast<float *>(smem), ex.o + seq, ex.f + seq, ex.i + seq,
@@ -732,6 +723,7 @@ TcWork tc_work(SeqArgs &a)
     t.wk.NC = a.NC;
     if (a.cu) {
         t.wk.cu = a.cu;
+        t.wk.B = a.B;
         t.wk.H = a.H;
         t.wk.G = a.seg_scratch ? tc_packed_segments(U, a.N) : 1;
         t.wk.spp = a.N / kC + a.B * t.wk.G + 1;

@@ -65,11 +65,11 @@ static_assert(sizeof(Ctl<4>) <= 256, "control block");
 struct Span { int plane, row0, n; size_t at; };
 // spans == true: plane x whole.  Otherwise segments r0, r0 + 1 .. of the cut units of w (tc_chunk.cuh), the result in the
 // segment's chain slot.
-__device__ __forceinline__ Span span_of(const WorkArgs &w, int x, bool spans, int cut, int r0, bool &malformed)
+__device__ __forceinline__ Span span_of(const WorkArgs &w, int x, bool spans, int cut, int r0)
 {
     if (spans) return Span{x, 0, w.N, (size_t)x};
     const int r = x / cut + r0, t = x % cut;
-    const Item it = work_item<true>(w, w.cu ? ((t / w.H) * w.G + r) * w.H + t % w.H : w.main + r * cut + t, malformed);
+    const Item it = work_item<true>(w, w.cu ? ((t / w.H) * w.G + r) * w.H + t % w.H : w.main + r * cut + t);
     return Span{it.plane, it.row0, it.n, (size_t)t * w.G + r};
 }
 
@@ -82,11 +82,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
 {
     using G = Geo<kBwd, kStages>;
     chain_wait();
-    if (clear_status && blockIdx.x == 0 && threadIdx.x == 0) {
-        status->code = 0;
-        status->where = 0;
-        status->exact_units = 0;
-    }
+    if (clear_status && blockIdx.x == 0) begin_call(status, wk.cu, wk.B, wk.N);
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     float *hp = reinterpret_cast<float *>(smem + G::kOffHp);
@@ -94,11 +90,9 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
     volatile int *abort_flag = &ctl->abort_flag;
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    bool malformed = false;
-    const Span sp = span_of(wk, blockIdx.x, spans != 0, cut, r0, malformed);
+    const Span sp = span_of(wk, blockIdx.x, spans != 0, cut, r0);
     const int zu = sp.plane, row0 = sp.row0, N = sp.n, NC = (N + kC - 1) / kC;
     const size_t u = sp.at;
-    if (malformed && tid == 0) report_error(status, HGRN2_ERR_INVALID_ARG, 6);
     if (N <= 0) {                        // an empty segment contributes nothing and does not decay
         for (int x = tid; x < kD * kD; x += kThreads) out[u * kD * kD + x] = 0.f;
         if (lam != nullptr && tid < kD) lam[u * kD + tid] = 1.f;

@@ -101,6 +101,12 @@ template <> __device__ __forceinline__ void store_f<__nv_bfloat16>(__nv_bfloat16
     *p = __float2bfloat16_rn(x);
 }
 
+__device__ __forceinline__ void clear_block(StatusBlock *sb)
+{
+    sb->code = 0;
+    sb->where = 0;
+    sb->exact_units = 0;
+}
 __device__ __forceinline__ void report_error(StatusBlock *sb, int code, int where)
 {
     if (sb != nullptr && atomicCAS(&sb->code, 0, code) == 0) sb->where = where;
@@ -186,7 +192,7 @@ struct WorkArgs {
     int main = 0, tail = 0;        // units taken whole, units cut into segments (ordinary batch)
     int G = 1, Lc = 0;             // segments per cut unit, chunks per segment
     const int *cu = nullptr;       // packed batch: row offsets on the device
-    int H = 1, spp = 0;            // packed batch: heads, state slots per head
+    int B = 0, H = 1, spp = 0;     // packed batch: sequences, heads, state slots per head
 };
 
 // How an ordinary batch is cut: units [0, main) run whole, the `tail` units behind them as G segments of Lc chunks (the

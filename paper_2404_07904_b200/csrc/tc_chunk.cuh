@@ -253,8 +253,21 @@ __device__ __forceinline__ bool packed_malformed(const WorkArgs &w, int b)
     return rows_malformed(w.cu[b], w.cu[b + 1], w.N);
 }
 
+// First CTA of a call's first kernel (all threads): the status block starts at zero, and malformed offsets are reported, of
+// whatever sequence.  By this CTA because a CTA with nothing but a malformed sequence is through in a microsecond,
+// and nothing orders its report behind the clearing (on a cold start it came first and was lost); what else is reported has
+// the sweep of a chunk, or a wait that ran out, in front of it.
+static __device__ __noinline__ void begin_call(StatusBlock *status, const int *cu, int B, int N)
+{
+    if (threadIdx.x == 0) clear_block(status);
+    if (cu == nullptr) return;
+    bool bad = false;
+    for (int b = threadIdx.x; b < B; b += blockDim.x) bad |= rows_malformed(cu[b], cu[b + 1], N);
+    if (__syncthreads_or(bad) && threadIdx.x == 0) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
+}
+
 template <bool kPackedToo>
-__device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malformed)
+__device__ __forceinline__ Item work_item(const WorkArgs &w, int x)
 {
     Item it;
     it.id = x;
@@ -263,7 +276,6 @@ __device__ __forceinline__ Item work_item(const WorkArgs &w, int x, bool &malfor
         it.plane = h;
         it.unit = b * w.H + h;
         if (packed_malformed(w, b)) {                                // touch nothing
-            malformed = true;
             it.row0 = it.n = it.slot0 = it.last = 0;
             it.chain = -1;
             return it;
@@ -391,8 +403,7 @@ static __device__ __noinline__ bool ring_ask(ItemRing *q, int k, volatile int *e
 }
 // Load warp: the answer to ring_ask (asked = its return value) becomes item k.
 template <bool kPackedToo>
-static __device__ __noinline__ const Item *ring_take(ItemRing *q, int k, bool asked, const WorkArgs &w, StatusBlock *status,
-                                                     volatile int *abort_flag)
+static __device__ __noinline__ const Item *ring_take(ItemRing *q, int k, bool asked, const WorkArgs &w, volatile int *abort_flag)
 {
     int x = -1;
     if (asked) {
@@ -404,11 +415,9 @@ static __device__ __noinline__ const Item *ring_take(ItemRing *q, int k, bool as
     }
     Item *it = &q->item[k % kRing];
     if ((threadIdx.x & 31) == 0) {
-        bool malformed = false;
-        if (x >= 0) *it = work_item<kPackedToo>(w, x, malformed);
+        if (x >= 0) *it = work_item<kPackedToo>(w, x);
         else *it = q->none;
         if (it->chain >= 0) q->cuts[q->n_cuts++] = x;
-        if (malformed) report_error(status, HGRN2_ERR_INVALID_ARG, 4);
         mbar_arrive(&q->full[k % kRing]);
     }
     __syncwarp();

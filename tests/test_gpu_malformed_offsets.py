@@ -40,3 +40,21 @@ PATHS = [("bf16", 128, 0, 1)]
 def test_lengths_beyond_the_integer_range(T, io, d, flags, status):
     # INT_MIN - 60 wraps to a length of 2^31 - 60, and start + length to a negative row
     _check([0, 60, INT_MIN, 100, 300], [0, 3], T, 2, io, d, flags, status)
+
+
+@pytest.mark.parametrize("B,T", [(2, 400), (20, 900), (700, 900)])       # whole, in segments, several per CTA
+def test_the_report_is_not_lost(B, T):
+    # the malformed sequence is the last one: its CTA has nothing to do and must not race the clearing of the status word
+    H, cu = 2, [0] * B + [T + 1]
+    x = torch.randn(H, T, 128, device="cuda").bfloat16().sigmoid()
+    cu = torch.tensor(cu, dtype=torch.int32, device="cuda")
+    junk = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
+    for turn in range(20):
+        _, _, saved, ws, _ = binding.hgrn2_fwd_varlen(x, x, x, cu)
+        torch.cuda.synchronize()
+        assert binding.hgrn2_poll(ws) == 1, turn
+        junk.fill_(turn)
+        for s in (saved, None):
+            binding.hgrn2_bwd_varlen(x, x, x, cu, None, x, None, s, ws=ws)
+            torch.cuda.synchronize()
+            assert binding.hgrn2_poll(ws) == 1, turn
