@@ -10,6 +10,9 @@
 //           start (the gradient at its end);
 //   value, key   outputs of one chunk: chunks are independent once the boundary values are there.
 //
+// Packed batches have instances of their own: the search for a chunk's sequence in the others' code cost 2 % of
+// 2 x 16 x 2048 float32.
+//
 // Formulas (q = o, k = 1 - f, v = i, b_t = sum_{r<=t} log f_r inside the chunk, m = after row 31,
 // Pm = exp(b_m), E = exp(b_C - b_m); S_in, D_out = state at the chunk's start, state gradient at its end):
 //
@@ -203,10 +206,17 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int n> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(n) : "memory"); }
 
-// Which chunk blockIdx.x stands for: false = none (a slot of a packed batch that no chunk uses).
-__device__ __forceinline__ bool chunk_of(const Args &a, Where &w, int &c)
+// Whether a slot of a packed batch holds a chunk of sequence b.
+__device__ __forceinline__ bool owns_slot(const int *cu, int b, int N, int slot)
 {
-    if (a.cu == nullptr) {
+    const int start = cu[b], end = cu[b + 1], c = slot - (start / kL + b);
+    return !rows_malformed(start, end, N) && c >= 0 && c < (end - start + kL - 1) / kL;
+}
+
+// Which chunk blockIdx.x stands for: false = none (a slot of a packed batch that no chunk uses).  Whole warps.
+template <bool kPacked> __device__ __forceinline__ bool chunk_of(const Args &a, Where &w, int &c)
+{
+    if constexpr (!kPacked) {
         const long long u = blockIdx.x / a.NC;
         c = blockIdx.x - (int)(u * a.NC);
         w = Where{(a.g0 + u) * a.N, a.N, a.NC, u * a.NC, a.g0 + u};
@@ -218,9 +228,20 @@ __device__ __forceinline__ bool chunk_of(const Args &a, Where &w, int &c)
         const int mid = (lo + hi + 1) / 2;
         if (a.cu[mid] / kL + mid <= slot) lo = mid; else hi = mid - 1;
     }
+    if (!owns_slot(a.cu, lo, a.N, slot)) {
+        // Nobody's slot - or a malformed offset has misled the search, and the well-formed sequences must come out all the
+        // same: every warp looks at all of them.
+        unsigned hits = 0;
+        for (lo = 0; lo < a.B; lo += 32) {
+            const int b = lo + (threadIdx.x & 31);
+            if ((hits = __ballot_sync(0xFFFFFFFFu, b < a.B && owns_slot(a.cu, b, a.N, slot))) != 0) break;
+        }
+        if (hits == 0) return false;
+        lo += __ffs(hits) - 1;
+    }
     w = packed_where(a, lo, a.g0 + h);
     c = slot - (a.cu[lo] / kL + lo);
-    return c >= 0 && c < w.nc;
+    return true;
 }
 
 // Where a chunk's decay totals [dk] wait for the scan: in the chunk's rows of an output that is written later (y in the
@@ -247,7 +268,7 @@ template <int TK, int TV, int SPLIT> struct LocalShape {
     static constexpr int CG = TK / 32, SEG = NW / CG, RP = kL / SEG;  // column groups, row segments, rows per segment
     static constexpr size_t kSmem = (size_t)(kL * (TK + TV) + SEG * TK) * sizeof(float);
 };
-template <typename T, int kMode, bool kBwd, int TK, int TV, int SPLIT>
+template <typename T, int kMode, bool kPacked, bool kBwd, int TK, int TV, int SPLIT>
 __global__ void __launch_bounds__(LocalShape<TK, TV, SPLIT>::NT)
 fp32_local_kernel(const Args a)
 {
@@ -259,7 +280,7 @@ fp32_local_kernel(const Args a)
     if (a.status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) clear_block(a.status);
     Where w;
     int c;
-    if (!chunk_of(a, w, c)) return;
+    if (!chunk_of<kPacked>(a, w, c)) return;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int rows = min(kL, w.n - c * kL);
     const long long row0 = w.row + (long long)c * kL;
@@ -424,7 +445,7 @@ constexpr int kValueThreads = 256;
 // the first four warps only
 __device__ __forceinline__ void sync_first_half() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
-template <typename T, int kMode, bool kDV, int NV>
+template <typename T, int kMode, bool kPacked, bool kDV, int NV>
 __global__ void __launch_bounds__(kValueThreads, 2)
 fp32_value_kernel(const Args a)
 {
@@ -438,7 +459,7 @@ fp32_value_kernel(const Args a)
     auto stage = [&](int j) { return sm + (j & 1) * (P::kStage + kTile); };
     Where w;
     int c;
-    if (!chunk_of(a, w, c)) return;
+    if (!chunk_of<kPacked>(a, w, c)) return;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int rows = min(kL, w.n - c * kL);
     const long long row0 = w.row + (long long)c * kL;
@@ -711,7 +732,7 @@ constexpr int kKTile = kW * kL;                                       // [64][32
 constexpr int kSq = kL * kL;                                          // [64][64]
 constexpr size_t kKSmem = (6 * kSq + 8 * kL + 2 * kL + 8 * kL) * sizeof(float);
 
-template <typename T, int kMode>
+template <typename T, int kMode, bool kPacked>
 __global__ void __launch_bounds__(kKeyThreads, 2)
 fp32_key_kernel(const Args a)
 {
@@ -722,7 +743,7 @@ fp32_key_kernel(const Args a)
     float *ssum = sR + 2 * kL;                                        // [2][4][64] segment sums of a and e
     Where w;
     int c;
-    if (!chunk_of(a, w, c)) return;
+    if (!chunk_of<kPacked>(a, w, c)) return;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int k0 = blockIdx.y * kL;
     const int rows = min(kL, w.n - c * kL);
@@ -1100,55 +1121,55 @@ fp32_key_kernel(const Args a)
 long long slots_per_group(const Args &a) { return a.cu ? a.spp : a.NC; }
 long long units_per_group(const Args &a) { return a.cu ? a.B : 1; }
 
-template <typename T, int kMode, bool kBwd, int TK, int TV, int SPLIT>
+template <typename T, int kMode, bool kPacked, bool kBwd, int TK, int TV, int SPLIT>
 cudaError_t launch_local_t(const Args &a, long long chunks, cudaStream_t stream)
 {
     using P = LocalShape<TK, TV, SPLIT>;
-    auto kernel = fp32_local_kernel<T, kMode, kBwd, TK, TV, SPLIT>;
+    auto kernel = fp32_local_kernel<T, kMode, kPacked, kBwd, TK, TV, SPLIT>;
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), P::kSmem);
     if (err != cudaSuccess) return err;
     return launch_chained(kernel, dim3((unsigned)chunks), P::NT, P::kSmem, stream, a);
 }
 
 // Boundary values of `groups` groups: every chunk's own contribution, then the chain over each sequence.
-template <typename T, int kMode, bool kBwd>
+template <typename T, int kMode, bool kPacked, bool kBwd>
 cudaError_t launch_state(const Args &a, long long groups, cudaStream_t stream)
 {
     const long long chunks = groups * slots_per_group(a);
     cudaError_t err;
     if (a.dk > 64)
-        err = a.dv > 64 ? launch_local_t<T, kMode, kBwd, 128, 128, 1>(a, chunks, stream)
-                        : launch_local_t<T, kMode, kBwd, 128, 64, 2>(a, chunks, stream);
+        err = a.dv > 64 ? launch_local_t<T, kMode, kPacked, kBwd, 128, 128, 1>(a, chunks, stream)
+                        : launch_local_t<T, kMode, kPacked, kBwd, 128, 64, 2>(a, chunks, stream);
     else
-        err = a.dv > 64 ? launch_local_t<T, kMode, kBwd, 64, 128, 2>(a, chunks, stream)
-                        : launch_local_t<T, kMode, kBwd, 64, 64, 2>(a, chunks, stream);
+        err = a.dv > 64 ? launch_local_t<T, kMode, kPacked, kBwd, 64, 128, 2>(a, chunks, stream)
+                        : launch_local_t<T, kMode, kPacked, kBwd, 64, 64, 2>(a, chunks, stream);
     if (err != cudaSuccess) return err;
     const unsigned blocks = (a.dk * a.dv / 4 + kScanThreads - 1) / kScanThreads;
     return launch_chained(fp32_scan_kernel<T, kMode, kBwd>, dim3((unsigned)(groups * units_per_group(a)), blocks), kScanThreads, 0,
                           stream, a);
 }
 
-template <typename T, int kMode, bool kDV, int NV>
+template <typename T, int kMode, bool kPacked, bool kDV, int NV>
 cudaError_t launch_value_t(const Args &a, long long chunks, cudaStream_t stream)
 {
     using P = ValueShape<NV>;
-    auto kernel = fp32_value_kernel<T, kMode, kDV, NV>;
+    auto kernel = fp32_value_kernel<T, kMode, kPacked, kDV, NV>;
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), P::kSmem);
     if (err != cudaSuccess) return err;
     return launch_chained(kernel, dim3((unsigned)chunks), kValueThreads, P::kSmem, stream, a);
 }
-template <typename T, int kMode, bool kDV>
+template <typename T, int kMode, bool kPacked, bool kDV>
 cudaError_t launch_value(const Args &a, long long chunks, cudaStream_t stream)
 {
-    return a.dv > 64 ? launch_value_t<T, kMode, kDV, 128>(a, chunks, stream) : launch_value_t<T, kMode, kDV, 64>(a, chunks, stream);
+    return a.dv > 64 ? launch_value_t<T, kMode, kPacked, kDV, 128>(a, chunks, stream) : launch_value_t<T, kMode, kPacked, kDV, 64>(a, chunks, stream);
 }
 
-template <typename T, int kMode>
+template <typename T, int kMode, bool kPacked>
 cudaError_t launch_key(const Args &a, long long chunks, cudaStream_t stream)
 {
-    cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(fp32_key_kernel<T, kMode>), kKSmem);
+    cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void *>(fp32_key_kernel<T, kMode, kPacked>), kKSmem);
     if (err != cudaSuccess) return err;
-    return launch_chained(fp32_key_kernel<T, kMode>, dim3((unsigned)chunks, (a.dk + kL - 1) / kL), kKeyThreads, kKSmem, stream, a);
+    return launch_chained(fp32_key_kernel<T, kMode, kPacked>, dim3((unsigned)chunks, (a.dk + kL - 1) / kL), kKeyThreads, kKSmem, stream, a);
 }
 
 // groups = independent groups a launch can be restricted to: units, or heads of a packed batch
@@ -1180,20 +1201,20 @@ long long groups_per_round(const SeqArgs &s)
     return fit < group_count(s) ? fit : group_count(s);
 }
 
-template <typename T, int kMode>
+template <typename T, int kMode, bool kPacked>
 cudaError_t fwd_t(const SeqArgs &s, const float *beta)
 {
     Args a = make_args(s, beta);
     const long long g = group_count(s);
     a.states = s.states ? s.states : s.room;
     a.status = s.clear_status ? s.status : nullptr;
-    cudaError_t err = launch_state<T, kMode, false>(a, g, s.stream);
+    cudaError_t err = launch_state<T, kMode, kPacked, false>(a, g, s.stream);
     a.status = nullptr;
     if (err != cudaSuccess || s.y == nullptr) return err;
-    return launch_value<T, kMode, false>(a, g * slots_per_group(a), s.stream);
+    return launch_value<T, kMode, kPacked, false>(a, g * slots_per_group(a), s.stream);
 }
 
-template <typename T, int kMode>
+template <typename T, int kMode, bool kPacked>
 cudaError_t bwd_t(const SeqArgs &s, const float *beta, float *dbeta)
 {
     Args a = make_args(s, beta);
@@ -1215,13 +1236,13 @@ cudaError_t bwd_t(const SeqArgs &s, const float *beta, float *dbeta)
             a.dstates = s.room + (size_t)n * spg * ss;
             Args r = a;
             r.SN = nullptr;
-            if ((err = launch_state<T, kMode, false>(r, n, s.stream)) != cudaSuccess) return err;
+            if ((err = launch_state<T, kMode, kPacked, false>(r, n, s.stream)) != cudaSuccess) return err;
             a.status = nullptr;
         }
-        if ((err = launch_state<T, kMode, true>(a, n, s.stream)) != cudaSuccess) return err;
+        if ((err = launch_state<T, kMode, kPacked, true>(a, n, s.stream)) != cudaSuccess) return err;
         a.status = nullptr;
-        if ((err = launch_value<T, kMode, true>(a, n * spg, s.stream)) != cudaSuccess) return err;
-        if ((err = launch_key<T, kMode>(a, n * spg, s.stream)) != cudaSuccess) return err;
+        if ((err = launch_value<T, kMode, kPacked, true>(a, n * spg, s.stream)) != cudaSuccess) return err;
+        if ((err = launch_key<T, kMode, kPacked>(a, n * spg, s.stream)) != cudaSuccess) return err;
         if (dbeta) a.dbeta += (size_t)n * spg * s.dk;
     }
     return cudaSuccess;
@@ -1236,19 +1257,25 @@ int fp32_dbeta_rows(int N) { return (N + kL - 1) / kL; }
 
 cudaError_t launch_fp32_fwd(const SeqArgs &s)
 {
-    return s.io == HGRN2_BF16 ? fwd_t<__nv_bfloat16, alu::kGateIsF>(s, nullptr) : fwd_t<float, alu::kGateIsF>(s, nullptr);
+    if (s.io == HGRN2_BF16)
+        return s.cu ? fwd_t<__nv_bfloat16, alu::kGateIsF, true>(s, nullptr) : fwd_t<__nv_bfloat16, alu::kGateIsF, false>(s, nullptr);
+    return s.cu ? fwd_t<float, alu::kGateIsF, true>(s, nullptr) : fwd_t<float, alu::kGateIsF, false>(s, nullptr);
 }
 cudaError_t launch_fp32_bwd(const SeqArgs &s)
 {
-    return s.io == HGRN2_BF16 ? bwd_t<__nv_bfloat16, alu::kGateIsF>(s, nullptr, nullptr) : bwd_t<float, alu::kGateIsF>(s, nullptr, nullptr);
+    if (s.io == HGRN2_BF16)
+        return s.cu ? bwd_t<__nv_bfloat16, alu::kGateIsF, true>(s, nullptr, nullptr)
+                    : bwd_t<__nv_bfloat16, alu::kGateIsF, false>(s, nullptr, nullptr);
+    return s.cu ? bwd_t<float, alu::kGateIsF, true>(s, nullptr, nullptr) : bwd_t<float, alu::kGateIsF, false>(s, nullptr, nullptr);
 }
 cudaError_t launch_fp32_fwd_gated(const SeqArgs &s, const float *beta)
 {
-    return s.io == HGRN2_BF16 ? fwd_t<__nv_bfloat16, alu::kGatePre>(s, beta) : fwd_t<float, alu::kGatePre>(s, beta);
+    return s.io == HGRN2_BF16 ? fwd_t<__nv_bfloat16, alu::kGatePre, false>(s, beta) : fwd_t<float, alu::kGatePre, false>(s, beta);
 }
 cudaError_t launch_fp32_bwd_gated(const SeqArgs &s, const float *beta, float *dbeta)
 {
-    return s.io == HGRN2_BF16 ? bwd_t<__nv_bfloat16, alu::kGatePre>(s, beta, dbeta) : bwd_t<float, alu::kGatePre>(s, beta, dbeta);
+    return s.io == HGRN2_BF16 ? bwd_t<__nv_bfloat16, alu::kGatePre, false>(s, beta, dbeta)
+                              : bwd_t<float, alu::kGatePre, false>(s, beta, dbeta);
 }
 
 }  // namespace hgrn2

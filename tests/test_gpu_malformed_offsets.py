@@ -32,7 +32,7 @@ def _check(cu, good, T, H, io, d, flags, status):
     assert (y[:, untouched] == np.float32(torch.tensor(12345.0).to(tdt).float())).all()
 
 
-PATHS = [("bf16", 128, 0, 1)]
+PATHS = [("bf16", 128, 0, 1), ("bf16", 128, binding.FLAG_FORCE_ALU, 0), ("f32", 64, 0, 0)]
 
 
 @pytest.mark.parametrize("io,d,flags,status", PATHS)
@@ -58,3 +58,13 @@ def test_the_report_is_not_lost(B, T):
             binding.hgrn2_bwd_varlen(x, x, x, cu, None, x, None, s, ws=ws)
             torch.cuda.synchronize()
             assert binding.hgrn2_poll(ws) == 1, turn
+
+
+@pytest.mark.parametrize("io,d,flags,status", PATHS)
+@pytest.mark.parametrize("cu,good", [
+    ([0, 130, -5, 130, 330], [0, 3]),                # an offset that a search by value takes for an early one
+    ([0, 64, 500, 64, 200, 330], [0, 3, 4]),         # ... for a late one
+    ([-1, 70, 100, 200, 401], [1, 2]),               # the first and the last sequence
+])
+def test_other_sequences_are_unaffected(cu, good, io, d, flags, status):
+    _check(cu, good, 400, 2, io, d, flags, status)
