@@ -180,6 +180,42 @@ __device__ __forceinline__ void mul_rows(float (&acc)[8][8], const float *A, int
         }
     }
 }
+// The products of mul (MH = NH = 2, or MH = 1) with m <= x (kLower) or m >= x only, every other one left out: a zero of a
+// masked A does not hide an Inf or NaN in B, and no token may see one in a token that it does not depend on.
+template <bool kLower, int MH, int WA, int WB>
+__device__ __forceinline__ void mul_masked(float (&acc)[8][8], const float *A, int mp, const float *B, int np, int x0, int x1)
+{
+#pragma unroll 1
+    for (int x = x0; x < x1; ++x) {
+        float av[8], bv[8];
+        load4(A + piece<WA>(x, mp), reinterpret_cast<float(&)[4]>(av));
+        if (MH == 2) load4(A + piece<WA>(x, mp + 4), reinterpret_cast<float(&)[4]>(av[4]));
+        load4(B + piece<WB>(x, np), reinterpret_cast<float(&)[4]>(bv));
+        load4(B + piece<WB>(x, np + 8), reinterpret_cast<float(&)[4]>(bv[4]));
+#pragma unroll
+        for (int i = 0; i < 4 * MH; ++i) {
+            const int m = 4 * mp + 4 * (i & 4) + (i & 3);
+            if (kLower ? m <= x : m >= x)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+        }
+    }
+}
+// Whether rows [r0, r0 + rows) of B hold an Inf or NaN in this warp's columns (pieces 16 h .. 16 h + 15, np = 16 h + lane % 8).
+template <int rows, int WB> __device__ __forceinline__ bool not_finite(const float *B, int r0, int np, int lane)
+{
+    float z = 0.f;
+#pragma unroll
+    for (int r = 0; r < rows; r += 4)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float v[4];
+            load4(B + piece<WB>(r0 + r + (lane >> 3), np + 8 * h), v);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) z = fmaf(v[j], 0.f, z);
+        }
+    return __any_sync(0xFFFFFFFFu, z != 0.f);
+}
 __device__ __forceinline__ void zero(float (&acc)[8][8])
 {
 #pragma unroll
@@ -498,7 +534,9 @@ fp32_value_kernel(const Args a)
         }
         // only the tokens on the causal side of this warp's rows contribute
         const int m_low = P::MHY == 2 ? 32 * (wy & 1) : 16 * wy;
-        mul<P::MHY, 2, kL, NV>(acc, sA, mp, sW, np, kDV ? m_low : 0, kDV ? kL : m_low + 16 * P::MHY);
+        const int x0 = kDV ? m_low : 0, x1 = kDV ? kL : m_low + 16 * P::MHY;
+        if (not_finite<16 * P::MHY, NV>(sW, m_low, np, lane)) mul_masked<kDV, P::MHY, kL, NV>(acc, sA, mp, sW, np, x0, x1);
+        else mul<P::MHY, 2, kL, NV>(acc, sA, mp, sW, np, x0, x1);
         T *yg = static_cast<T *>(kDV ? a.d_i : a.y) + row0 * a.dv;
 #pragma unroll
         for (int i = 0; i < 4 * P::MHY; ++i) {
@@ -913,6 +951,7 @@ fp32_key_kernel(const Args a)
         below |= fminf(q[0] * q[kL] * q[2 * kL] * q[3 * kL], q[4 * kL] * q[5 * kL] * q[6 * kL] * q[7 * kL]) < kHalfFloor;
     }
     const bool out_of_range = __any_sync(0xFFFFFFFFu, below);         // the same in every warp
+    float odd = 0.f;                                                  // not 0: Inf or NaN among this thread's Qs, Ks
 #pragma unroll 1
     for (int x = 0; x < 2; ++x) {
         const int kx = lane + 32 * x;
@@ -952,8 +991,10 @@ fp32_key_kernel(const Args a)
             for (int r = 0; r < 8; ++r) {
                 run *= fv[r];
                 const int at = elem<kL>(wid * 8 + r, kx);
-                sQ[at] = qv[r] * run;
-                sK[at] = kv[r] * recip(run);
+                const float Q = qv[r] * run, K = kv[r] * recip(run);
+                odd = fmaf(Q, 0.f, fmaf(K, 0.f, odd));
+                sQ[at] = Q;
+                sK[at] = K;
                 sC[at] = run;
             }
         } else {
@@ -963,14 +1004,16 @@ fp32_key_kernel(const Args a)
             for (int r = 7; r >= 0; --r) {
                 const int at = elem<kL>(wid * 8 + r, kx);
                 const float inv = recip(run);
-                sQ[at] = qv[r] * inv;
-                sK[at] = kv[r] * run;
+                const float Q = qv[r] * inv, K = kv[r] * run;
+                odd = fmaf(Q, 0.f, fmaf(K, 0.f, odd));
+                sQ[at] = Q;
+                sK[at] = K;
                 sC[at] = inv;
                 run *= fv[r];
             }
         }
     }
-    __syncthreads();
+    const bool masked = __syncthreads_or(odd != 0.f) != 0;
     if (role == 2) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -989,9 +1032,11 @@ fp32_key_kernel(const Args a)
 #pragma unroll
                 for (int i = 0; i < 8; ++i) acc[i][j] *= pm;
             }
-            mul<2, 2, kL, kL>(acc, sAT, mp, sK, np, 0, 32 * (wm + 1));
+            if (masked) mul_masked<false, 2, kL, kL>(acc, sAT, mp, sK, np, 0, 32 * (wm + 1));
+            else mul<2, 2, kL, kL>(acc, sAT, mp, sK, np, 0, 32 * (wm + 1));
         } else if (role == 2) {
-            mul<2, 2, kL, kL>(acc, sA, mp, sQ, np, 32 * wm, kL);
+            if (masked) mul_masked<true, 2, kL, kL>(acc, sA, mp, sQ, np, 32 * wm, kL);
+            else mul<2, 2, kL, kL>(acc, sA, mp, sQ, np, 32 * wm, kL);
         }
         __syncthreads();
     }
