@@ -35,6 +35,10 @@
  *     that ran out) are written to the status word at the start of `ws` and reported
  *     by hgrn2_poll after the caller has synchronised the stream.  Nothing aborts,
  *     traps or throws.
+ *   - An output should not overlap an input (other than S of the decode calls).  The tensor-core kernels do not
+ *     look: a unit that is redone (see above) is redone from its inputs.  The fp32 kernels and the decode calls
+ *     accept an output that is an input of its shape; a sequence call like that runs on serial kernels, tens of times
+ *     slower.
  *   - When B * H * N = 0 the sequence tensors have no elements and their pointers may be
  *     NULL; with N = 0 the calls copy S0 to SN (and dSN to dS0).
  *   - Supported shapes: dk, dv in {16, 32, 64, 128}; any B, H, N >= 1 (N = 0 is

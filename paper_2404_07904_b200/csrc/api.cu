@@ -3,6 +3,8 @@
 #include <stddef.h>
 #include <string.h>
 
+#include <initializer_list>
+
 #include "common.cuh"
 
 using namespace hgrn2;
@@ -74,6 +76,26 @@ hgrn2_status check_ptrs(const void *const *req, int nreq, const void *const *opt
     for (int j = 0; j < nopt; ++j)
         if (opt[j] && !aligned16(opt[j])) return HGRN2_ERR_ALIGNMENT;
     return HGRN2_OK;
+}
+
+// Whether an output of a call overlaps one of its inputs.  Each (pointer, row width).
+struct Seq { const void *p; int width; };
+bool overlap(const hgrn2_desc *d, bool packed, std::initializer_list<Seq> outs, std::initializer_list<Seq> ins)
+{
+    const size_t column = (packed ? 1 : (size_t)d->B) * d->H * d->N * (d->io == HGRN2_F32 ? 4 : 2);
+    for (const Seq &a : outs)
+        for (const Seq &b : ins) {
+            const uintptr_t x = reinterpret_cast<uintptr_t>(a.p), y = reinterpret_cast<uintptr_t>(b.p);
+            if (x < y + column * b.width && y < x + column * a.width) return true;
+        }
+    return false;
+}
+// The serial fp32 forward, leaving its states as the chunk-parallel kernels do: one per 64 tokens, whatever C is.
+SeqArgs serial_fwd(SeqArgs a)
+{
+    a.C = 64;
+    a.NC = (a.N + 63) / 64;
+    return a;
 }
 
 size_t state_bytes(const hgrn2_desc *d) { return (size_t)d->B * d->H * d->dk * d->dv * sizeof(float); }
@@ -198,7 +220,10 @@ hgrn2_status fwd_impl(const hgrn2_desc *desc, const void *o, const void *f, cons
     // The status word starts every call at zero.  The first kernel of the call does that itself (a separate clear
     // between two kernels of a stream costs a microsecond of idle GPU each time); when no kernel will run, and in
     // front of the serial fp32 kernels, it is a small asynchronous memset.
-    a.clear_status = !empty;
+    const bool tc = use_tc(desc);
+    const int dk = desc->dk, dv = desc->dv;
+    const bool serial = !tc && !empty && overlap(desc, cu != nullptr, {{y, dv}}, {{o, dk}, {f, dk}, {i, dv}});
+    a.clear_status = !empty && !serial;
     if (!a.clear_status && cudaMemsetAsync(ws, 0, sizeof(StatusBlock), a.stream) != cudaSuccess) return HGRN2_ERR_CUDA;
     if ((size_t)desc->B * desc->H == 0) return HGRN2_OK;
     if (desc->N == 0) {
@@ -209,7 +234,7 @@ hgrn2_status fwd_impl(const hgrn2_desc *desc, const void *o, const void *f, cons
         }
         return HGRN2_OK;
     }
-    cudaError_t e = use_tc(desc) ? launch_tc_fwd(a) : launch_fp32_fwd(a);
+    cudaError_t e = tc ? launch_tc_fwd(a) : serial ? launch_alu_fwd(serial_fwd(a)) : launch_fp32_fwd(a);
     return e == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
 }
 
@@ -234,7 +259,9 @@ hgrn2_status bwd_impl(const hgrn2_desc *desc, const void *o, const void *f, cons
     a.status = static_cast<StatusBlock *>(ws);
     const bool tc = use_tc(desc);
     a.states = const_cast<float *>(static_cast<const float *>(saved));
-    const bool serial = !tc && !empty && !fp32_bwd_supported(a);
+    const int dk = desc->dk, dv = desc->dv;
+    const bool serial = !tc && !empty && (!fp32_bwd_supported(a) || overlap(desc, cu != nullptr, {{d_o, dk}, {d_f, dk}, {d_i, dv}},
+                                                                            {{o, dk}, {f, dk}, {i, dv}, {dy, dv}}));
     a.clear_status = !empty && !serial;                          // see hgrn2_fwd
     if (!a.clear_status && cudaMemsetAsync(ws, 0, sizeof(StatusBlock), a.stream) != cudaSuccess) return HGRN2_ERR_CUDA;
     if ((size_t)desc->B * desc->H == 0) return HGRN2_OK;
@@ -247,8 +274,9 @@ hgrn2_status bwd_impl(const hgrn2_desc *desc, const void *o, const void *f, cons
         return HGRN2_OK;
     }
     if (!tc && !serial) return launch_fp32_bwd(a) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
-    if (!saved) {
-        // re-create the chunk-start states inside the workspace with a states-only forward
+    if (!saved || serial) {
+        // re-create the chunk-start states inside the workspace with a states-only forward (the serial kernels' chunks are
+        // not those of the saved states)
         SeqArgs r = a;
         r.y = nullptr; r.SN = nullptr;
         r.states = a.room;
@@ -357,7 +385,9 @@ hgrn2_status hgrn2_fwd_gated(const hgrn2_desc *desc, const void *zo, const void 
     a.o = zo; a.f = zf; a.i = zi; a.S0 = S0; a.y = y; a.SN = SN;
     a.status = static_cast<StatusBlock *>(ws);
     const bool tc = use_tc(desc);
-    a.clear_status = !empty;
+    const int dk = desc->dk, dv = desc->dv;
+    const bool serial = !tc && !empty && overlap(desc, false, {{y, dv}}, {{zo, dk}, {zf, dk}, {zi, dv}});
+    a.clear_status = !empty && !serial;
     if (!a.clear_status && cudaMemsetAsync(ws, 0, sizeof(StatusBlock), a.stream) != cudaSuccess) return HGRN2_ERR_CUDA;
     if ((size_t)desc->B * desc->H == 0) return HGRN2_OK;
     if (desc->N == 0) {
@@ -370,7 +400,8 @@ hgrn2_status hgrn2_fwd_gated(const hgrn2_desc *desc, const void *zo, const void 
     }
     if (!tc) {
         a.states = static_cast<float *>(saved);
-        return launch_fp32_fwd_gated(a, beta) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
+        const cudaError_t e = serial ? launch_alu_fwd_gated(serial_fwd(a), beta) : launch_fp32_fwd_gated(a, beta);
+        return e == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
     }
     // the gates go to the head of `saved` (kept for the backward) or, for inference, of the workspace's room for it
     char *gates = saved ? static_cast<char *>(saved) : static_cast<char *>(ws) + sizeof(StatusBlock);
@@ -405,7 +436,9 @@ hgrn2_status hgrn2_bwd_gated(const hgrn2_desc *desc, const void *zo, const void 
     a.status = static_cast<StatusBlock *>(ws);
     const bool tc = use_tc(desc);
     if (!tc) a.states = const_cast<float *>(static_cast<const float *>(saved));
-    const bool serial = !tc && !empty && !fp32_bwd_supported(a);
+    const int dk = desc->dk, dv = desc->dv;
+    const bool serial = !tc && !empty && (!fp32_bwd_supported(a) || overlap(desc, false, {{d_zo, dk}, {d_zf, dk}, {d_zi, dv}},
+                                                                            {{zo, dk}, {zf, dk}, {zi, dv}, {dy, dv}}));
     a.clear_status = !empty && !serial;
     if (!a.clear_status && cudaMemsetAsync(ws, 0, sizeof(StatusBlock), a.stream) != cudaSuccess) return HGRN2_ERR_CUDA;
     const size_t beta_bytes = (size_t)desc->H * desc->dk * sizeof(float);
@@ -419,7 +452,7 @@ hgrn2_status hgrn2_bwd_gated(const hgrn2_desc *desc, const void *zo, const void 
         return HGRN2_OK;
     }
     if (!tc) {
-        if (serial) {                            // one unit, states re-created: see fp32_bwd_supported
+        if (serial) {                            // states re-created
             SeqArgs r = a;
             r.y = nullptr; r.SN = nullptr;
             r.states = a.room;

@@ -1,9 +1,11 @@
 // Serial fp32 kernels: one CTA per (batch, head) unit walks the chunks in order (forward) or in reverse (backward)
 // with the running state S (forward) or state gradient dS (backward) resident in shared memory.
 //
-// Left for one case only, the backward of a single unit without saved states: its workspace holds one set of
-// boundary states, and the chunk-parallel kernels (chunk_fp32.cu) need two.  The per-unit bodies (chunk_alu.cuh)
-// are also the exact path of the tensor-core kernels.
+// Left for two kinds of calls: the backward of a single unit without saved states, whose workspace holds one set of
+// boundary states where the chunk-parallel kernels (chunk_fp32.cu) need two; and calls with an output in the place of an
+// input, which those kernels would use for scratch or overwrite before its last reader, and which here is read, a chunk at a
+// time, before that chunk of the output is written.  The per-unit bodies (chunk_alu.cuh) are also the exact path of the
+// tensor-core kernels.
 #include "chunk_alu.cuh"
 
 namespace hgrn2 {
