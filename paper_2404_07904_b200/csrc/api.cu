@@ -588,6 +588,9 @@ hgrn2_status hgrn2_step(const hgrn2_desc *desc, const void *o, const void *f, co
     a.B = desc->B; a.H = desc->H; a.dk = desc->dk; a.dv = desc->dv; a.io = desc->io;
     a.o = o; a.f = f; a.i = i; a.S = S; a.y = y;
     a.stream = static_cast<cudaStream_t>(cuda_stream);
+    hgrn2_desc one = *desc;
+    one.N = 1;
+    a.whole = overlap(&one, false, {{y, desc->dv}}, {{o, desc->dk}, {f, desc->dk}});
     return launch_step(a) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
 }
 
@@ -605,6 +608,7 @@ hgrn2_status hgrn2_step_multi(const hgrn2_desc *desc, const void *o, const void 
     a.B = desc->B; a.H = desc->H; a.dk = desc->dk; a.dv = desc->dv; a.io = desc->io; a.T = desc->N;
     a.o = o; a.f = f; a.i = i; a.S = S; a.y = y;
     a.stream = static_cast<cudaStream_t>(cuda_stream);
+    a.whole = overlap(desc, false, {{y, desc->dv}}, {{o, desc->dk}, {f, desc->dk}});
     return launch_step_multi(a) == cudaSuccess ? HGRN2_OK : HGRN2_ERR_CUDA;
 }
 

@@ -167,6 +167,7 @@ struct SeqArgs {
 struct StepArgs {
     int B, H, dk, dv, io;
     int T = 1;             // tokens per launch (launch_step_multi)
+    bool whole = false;    // y overlaps o or f: one CTA per unit, which reads all of a unit's gates before it writes its y
     const void *o, *f, *i;
     float *S;
     void *y;

@@ -120,7 +120,7 @@ step_kernel(const T *__restrict__ o, const T *__restrict__ f, const T *__restric
 // or not, so gates staged as ready-made pairs (24 bytes per row for four columns) cost as much as the arithmetic
 // twice over.  One 8-byte (f, o) per row serves eight columns here.  4096 units, bf16: 8 tokens 139 -> 104 us (83 is
 // the state traffic alone), 16 tokens 250 -> 169 us; quarter units per CTA 141 us, one token per loop body 115 us.
-template <typename T, int D, int kSplit>
+template <typename T, int D, int kSplit, int TB>
 __global__ void __launch_bounds__(Cols<D>::kThreads / kSplit)
 step_multi_kernel(const T *__restrict__ o, const T *__restrict__ f, const T *__restrict__ i,
                   float *__restrict__ S, T *__restrict__ y, int Tn, long long units)
@@ -128,7 +128,6 @@ step_multi_kernel(const T *__restrict__ o, const T *__restrict__ f, const T *__r
     constexpr int VEC = Cols<D>::kVec, NT = Cols<D>::kThreads / kSplit;
     constexpr int CW = D / kSplit, CG = CW / (4 * VEC), C4 = D / 4;
     constexpr int R = D / kRG;                 // rows per thread
-    constexpr int TB = 8;                      // tokens staged, and reduced, together
     __shared__ float2 s_fo[TB][D];
     __shared__ __align__(16) float s_i[TB][CW];
     __shared__ __align__(16) float s_red[TB][kRG][CW];
@@ -210,12 +209,13 @@ step_multi_kernel(const T *__restrict__ o, const T *__restrict__ f, const T *__r
 
 unsigned step_grid(long long ctas) { return (unsigned)(ctas < (1ll << 30) ? ctas : (1ll << 30)); }
 
-template <typename T, int D, int kSplit>
+// TB = tokens staged, and reduced, together
+template <typename T, int D, int kSplit, int TB = 8>
 cudaError_t launch_step_multi_t(const StepArgs &a)
 {
     const long long units = (long long)a.B * a.H;
     if (units == 0 || a.T == 0) return cudaSuccess;
-    step_multi_kernel<T, D, kSplit><<<step_grid(units * kSplit), Cols<D>::kThreads / kSplit, 0, a.stream>>>(
+    step_multi_kernel<T, D, kSplit, TB><<<step_grid(units * kSplit), Cols<D>::kThreads / kSplit, 0, a.stream>>>(
         static_cast<const T *>(a.o), static_cast<const T *>(a.f), static_cast<const T *>(a.i), a.S,
         static_cast<T *>(a.y), a.T, units);
     return cudaGetLastError();
@@ -235,7 +235,7 @@ cudaError_t launch_step_t(const StepArgs &a)
 template <typename T>
 cudaError_t launch_step_dv(const StepArgs &a)
 {
-    const bool few = (long long)a.B * a.H <= kFewUnits;
+    const bool few = !a.whole && (long long)a.B * a.H <= kFewUnits;
     switch (a.dv) {
         case 16:  return launch_step_t<T, 16, 1, 8>(a);
         case 32:  return launch_step_t<T, 32, 1, 8>(a);
@@ -258,8 +258,10 @@ cudaError_t launch_step_multi(const StepArgs &a)
 {
     if (!step_multi_supported(a.dk, a.dv)) return cudaErrorInvalidValue;
     if (a.io == HGRN2_BF16)
-        return a.dk == 128 ? launch_step_multi_t<__nv_bfloat16, 128, 2>(a) : launch_step_multi_t<__nv_bfloat16, 64, 1>(a);
-    return a.dk == 128 ? launch_step_multi_t<float, 128, 2>(a) : launch_step_multi_t<float, 64, 1>(a);
+        return a.dk == 64 ? launch_step_multi_t<__nv_bfloat16, 64, 1>(a)
+               : a.whole  ? launch_step_multi_t<__nv_bfloat16, 128, 1, 4>(a) : launch_step_multi_t<__nv_bfloat16, 128, 2>(a);
+    return a.dk == 64 ? launch_step_multi_t<float, 64, 1>(a)
+           : a.whole  ? launch_step_multi_t<float, 128, 1, 4>(a) : launch_step_multi_t<float, 128, 2>(a);
 }
 
 }  // namespace hgrn2

@@ -50,3 +50,23 @@ def test_gated_calls():
     t = {k: torch.from_numpy(v).cuda() for k, v in inp.items()}
     y, SN, _, _, _ = binding.hgrn2_fwd_gated(t["zo"], t["zf"], t["zi"], t["beta"], t["S0"], y=t["zi"])
     G.assert_close(_host({"y": y, "SN": SN}), {k: want[k] for k in ("y", "SN")}, 1e-4, "y in the place of zi")
+
+
+@pytest.mark.parametrize("T", [1, 3, 21])
+@pytest.mark.parametrize("io,d,H", [("bf16", 128, 8), ("f32", 128, 400), ("bf16", 64, 8), ("f32", 64, 8)])
+def test_decode_calls(io, d, H, T):
+    # few units (one token: several CTAs per unit) and many; bit for bit what goes into a buffer of its own
+    inp = W.make_inputs(W.scaled(W.CONFIGS["tiny_f32"], B=1, H=H, N=T, dk=d, dv=d, io=io, has_S0=True, seed=63, gamma=0.5))
+
+    def call(place):
+        t = G.to_dev(inp, io)
+        if T == 1:
+            t.update({k: t[k][:, :, 0].contiguous() for k in ("o", "f", "i")})
+        y = t[place] if place else None
+        y = (binding.hgrn2_step if T == 1 else binding.hgrn2_step_multi)(t["o"], t["f"], t["i"], t["S0"], y=y)
+        return y, t["S0"]
+
+    want = call(None)
+    for place in ("o", "f", "i"):
+        for got, w in zip(call(place), want):
+            assert torch.equal(got, w), place
