@@ -128,7 +128,7 @@ step_multi_kernel(const T *__restrict__ o, const T *__restrict__ f, const T *__r
     constexpr int VEC = Cols<D>::kVec, NT = Cols<D>::kThreads / kSplit;
     constexpr int CW = D / kSplit, CG = CW / (4 * VEC), C4 = D / 4;
     constexpr int R = D / kRG;                 // rows per thread
-    __shared__ float2 s_fo[TB][D];
+    __shared__ __align__(16) float2 s_fo[TB][D];              // filled 16 bytes at a time
     __shared__ __align__(16) float s_i[TB][CW];
     __shared__ __align__(16) float s_red[TB][kRG][CW];
 
