@@ -229,8 +229,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__ CUtensorMap map_f,
               const __grid_constant__ CUtensorMap map_i, const __grid_constant__ CUtensorMap map_dy,
               const __grid_constant__ CUtensorMap map_saved, const __grid_constant__ CUtensorMap map_o_raw,
-              const __grid_constant__ CUtensorMap map_f_raw, const float *__restrict__ totals,
-              const float *__restrict__ dSN, const float *__restrict__ chain, int *__restrict__ redo, __nv_bfloat16 *__restrict__ d_o,
+              const __grid_constant__ CUtensorMap map_f_raw, const float *totals,
+              const float *dSN, const float *chain, int *__restrict__ redo, __nv_bfloat16 *__restrict__ d_o,
               __nv_bfloat16 *__restrict__ d_f, __nv_bfloat16 *__restrict__ d_i, float *__restrict__ dS0,
               const __grid_constant__ WorkArgs wk, StatusBlock *status, int clear_status, const ExactArgs ex,
               int start_aborted)
@@ -352,8 +352,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
             // previous item's last update of it is done behind barX)
             if (nc > 0) {
                 const float *init = im.chain >= 0 ? chain + ((size_t)im.chain * kD + krow) * kD : (dSN ? dSN + row : nullptr);
-                pm_c = __ldg(tot_u + (size_t)(nc - 1) * 2 * kD);
-                ee_c = __ldg(tot_u + (size_t)(nc - 1) * 2 * kD + kD);
+                pm_c = tot_u[(size_t)(nc - 1) * 2 * kD];
+                ee_c = tot_u[(size_t)(nc - 1) * 2 * kD + kD];
                 if (it > 0) mbar_wait(&ctl->barX, (it - 1) & 1, abort_flag);
                 tc_fence_after_sync();
 #pragma unroll 1
@@ -361,7 +361,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                     uint32_t r[32];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        const float4 v4 = init ? __ldg(reinterpret_cast<const float4 *>(init + 32 * part) + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float4 v4 = init ? reinterpret_cast<const float4 *>(init + 32 * part)[j] : make_float4(0.f, 0.f, 0.f, 0.f);
                         r[4 * j + 0] = __float_as_uint(v4.x); r[4 * j + 1] = __float_as_uint(v4.y);
                         r[4 * j + 2] = __float_as_uint(v4.z); r[4 * j + 3] = __float_as_uint(v4.w);
                     }
@@ -382,8 +382,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                 pm_prev = pm_c;
                 const bool safe = factor >= kFactorSafe;
                 if (c > 0) {
-                    pm_c = __ldg(tot_u + (size_t)(c - 1) * 2 * kD);
-                    ee_c = __ldg(tot_u + (size_t)(c - 1) * 2 * kD + kD);
+                    pm_c = tot_u[(size_t)(c - 1) * 2 * kD];
+                    ee_c = tot_u[(size_t)(c - 1) * 2 * kD + kD];
                 }
                 if (it > 0) {
                     mbar_wait(&ctl->barX, (it - 1) & 1, abort_flag);   // dS' of the previous chunk is complete

@@ -91,7 +91,7 @@ template <bool kRagged, bool kEnc, bool kPersist>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__ CUtensorMap map_f,
               const __grid_constant__ CUtensorMap map_i, const __grid_constant__ CUtensorMap map_y,
-              const __grid_constant__ CUtensorMap map_saved, const float *__restrict__ S0, const float *__restrict__ chain,
+              const __grid_constant__ CUtensorMap map_saved, const float *S0, const float *chain,
               int *__restrict__ redo, float *__restrict__ SN, float *__restrict__ totals, int want_y, int want_saved,
               const __grid_constant__ WorkArgs wk, StatusBlock *status, int clear_status, const ExactArgs ex,
               int start_aborted)
@@ -198,7 +198,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant__
                     uint32_t r[32];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        const float4 x = init ? __ldg(reinterpret_cast<const float4 *>(init + 32 * part) + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float4 x = init ? reinterpret_cast<const float4 *>(init + 32 * part)[j] : make_float4(0.f, 0.f, 0.f, 0.f);
                         r[4 * j + 0] = __float_as_uint(x.x); r[4 * j + 1] = __float_as_uint(x.y);
                         r[4 * j + 2] = __float_as_uint(x.z); r[4 * j + 3] = __float_as_uint(x.w);
                     }

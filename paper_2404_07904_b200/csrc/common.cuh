@@ -32,9 +32,11 @@ static_assert(sizeof(StatusBlock) == 256, "status block is 256 bytes");
 // A kernel launched with launch_chained may start while its predecessor in the stream still runs its last CTAs
 // (programmatic dependent launch): the launch itself, and what the kernel does before chain_wait(), then cost nothing.
 // Every thread of it calls chain_wait() before it touches global memory or leaves: behind it everything the stream
-// did before is complete and visible, and the next kernel may be brought in.  A call of few tokens is a handful of
-// kernels of a few microseconds each, so the starts count: prefill of 5000 tokens (three kernels) 48.2 -> 45.2 us, 2 units
-// of 256 tokens on the fp32 path forward and backward (seven) 61.5 -> 55.4 us; nothing measurable at full size.
+// did before is complete and visible, and the next kernel may be brought in.  What a predecessor may have written is
+// read with plain loads (not __ldg, nor through const __restrict__): it has changed during this kernel's lifetime.
+// A call of few tokens is a handful of kernels of a few microseconds each, so the starts count: prefill of 5000 tokens
+// (three kernels) 48.2 -> 45.2 us, 2 units of 256 tokens on the fp32 path forward and backward (seven) 61.5 -> 55.4 us;
+// nothing measurable at full size.
 __device__ __forceinline__ void chain_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
