@@ -1163,6 +1163,12 @@ fp32_key_kernel(const Args a)
     }
 }
 
+// Every launch's x dimension is a number of slots or units.
+bool grid_ok(const SeqArgs &s)
+{
+    const long long g = s.cu ? s.H : (long long)s.B * s.H, per = s.cu ? (long long)s.N / kL + s.B + 1 : (s.N + kL - 1ll) / kL;
+    return per <= 0x7fffffff && g <= 0x7fffffff / per;
+}
 long long slots_per_group(const Args &a) { return a.cu ? a.spp : a.NC; }
 long long units_per_group(const Args &a) { return a.cu ? a.B : 1; }
 
@@ -1237,18 +1243,19 @@ Args make_args(const SeqArgs &s, const float *beta)
 // Slots the caller's buffers have room for: they are sized for the call's own chunk length C <= 64.
 long long slots_at_hand(const SeqArgs &s)
 {
-    return group_count(s) * (s.cu ? s.N / s.C + s.B + 1 : (s.N + s.C - 1) / s.C);
+    return group_count(s) * (s.cu ? s.N / s.C + s.B + 1ll : (s.N + s.C - 1) / s.C);
 }
 // Backward without saved states: groups whose two sets of boundary values fit the workspace's room together.
 long long groups_per_round(const SeqArgs &s)
 {
-    const long long spg = s.cu ? s.N / kL + s.B + 1 : (s.N + kL - 1) / kL, fit = slots_at_hand(s) / (2 * spg);
+    const long long spg = s.cu ? s.N / kL + s.B + 1ll : (s.N + kL - 1) / kL, fit = slots_at_hand(s) / (2 * spg);
     return fit < group_count(s) ? fit : group_count(s);
 }
 
 template <typename T, int kMode, bool kPacked>
 cudaError_t fwd_t(const SeqArgs &s, const float *beta)
 {
+    if (!grid_ok(s)) return cudaErrorInvalidConfiguration;
     Args a = make_args(s, beta);
     const long long g = group_count(s);
     a.states = s.states ? s.states : s.room;
@@ -1262,6 +1269,7 @@ cudaError_t fwd_t(const SeqArgs &s, const float *beta)
 template <typename T, int kMode, bool kPacked>
 cudaError_t bwd_t(const SeqArgs &s, const float *beta, float *dbeta)
 {
+    if (!grid_ok(s)) return cudaErrorInvalidConfiguration;
     Args a = make_args(s, beta);
     const long long g = group_count(s), spg = slots_per_group(a);
     const size_t ss = (size_t)s.dk * s.dv;

@@ -55,7 +55,9 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, si
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    if (err != cudaSuccess) cudaGetLastError();       // it is this call's error: the next one's launches ask for theirs
+    return err;
 }
 
 template <typename T> __device__ __forceinline__ float load_f(const T *p);
