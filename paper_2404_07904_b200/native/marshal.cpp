@@ -60,18 +60,17 @@ int32_t io_code(const at::Tensor &t)
     throw PyError{};
 }
 
-long integer(PyObject *x)
-{
-    const long v = PyLong_AsLong(x);
-    if (v == -1 && PyErr_Occurred()) throw PyError{};
-    return v;
-}
+// Whatever int() takes, cut to 32 bits, as a ctypes field does.
 uint32_t bits(PyObject *x)
 {
-    const unsigned long v = PyLong_AsUnsignedLongMask(x);
+    PyObject *n = PyNumber_Long(x);
+    if (!n) throw PyError{};
+    const unsigned long v = PyLong_AsUnsignedLongMask(n);
+    Py_DECREF(n);
     if (v == (unsigned long)-1 && PyErr_Occurred()) throw PyError{};
     return (uint32_t)v;
 }
+long integer(PyObject *x) { return (int32_t)bits(x); }
 bool truth(PyObject *x)
 {
     const int v = PyObject_IsTrue(x);
@@ -256,17 +255,20 @@ PyObject *bwd(PyObject *, PyObject *const *a, Py_ssize_t n)
     if (!arity(n, 20)) return nullptr;
     return guarded([&]() -> PyObject * {
         const long kind = integer(a[0]);
-        const at::Tensor &o = tensor(a[1]), &f = tensor(a[2]), &i = tensor(a[3]);
+        const at::Tensor &o = tensor(a[1]), &i = tensor(a[3]);
         Shape s = sequence_shape(kind, o, i, a[4], a[17], a[18]);
         const hgrn2_desc &d = s.d;
         Buffer d_o(a[9]), d_f(a[10]), d_i(a[11]), d_beta(a[12]), dS0(a[13]), ws(a[14]);
         if (d_o.missing()) d_o.make(o.sizes(), o.scalar_type(), o);
-        if (d_f.missing()) d_f.make(f.sizes(), f.scalar_type(), f);
+        if (d_f.missing()) {
+            const at::Tensor &f = tensor(a[2]);
+            d_f.make(f.sizes(), f.scalar_type(), f);
+        }
         if (d_i.missing()) d_i.make(i.sizes(), i.scalar_type(), i);
         if (kind == kGated && d_beta.missing() && truth(a[16])) d_beta.make({d.H, d.dk}, at::kFloat, o);
         if (dS0.missing() && truth(a[15])) dS0.make({d.B, d.H, d.dk, d.dv}, at::kFloat, o);
         if (ws.missing()) make_workspace(ws, kind, &d, o);
-        void *po = ptr(o), *pf = ptr(f), *pi = ptr(i), *px = ptr(a[4]), *pS0 = ptr(a[5]), *pdy = ptr(a[6]), *pdSN = ptr(a[7]),
+        void *po = ptr(o), *pf = ptr(a[2]), *pi = ptr(i), *px = ptr(a[4]), *pS0 = ptr(a[5]), *pdy = ptr(a[6]), *pdSN = ptr(a[7]),
              *psaved = ptr(a[8]), *st = stream_of(a[19]);
         const float *S0 = static_cast<const float *>(pS0), *dSN = static_cast<const float *>(pdSN);
         float *pdS0 = static_cast<float *>(dS0.p);
