@@ -42,13 +42,10 @@ if ROOT not in sys.path:
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 NOMINAL = {"hbm_gbs": 7700.0, "bf16_tflops": 2250.0}
 
-# dram__bytes_read.sum + dram__bytes_write.sum per launch, copied from the ncu captures summarised under
-# profiles/ (same workloads as timed here: lm_2048 and the full decode batch); nothing here measures traffic.
+# dram__bytes_read.sum + dram__bytes_write.sum per launch from profiler captures; nothing here measures traffic.
 # None = the kernel has changed since its counters were taken.
-NCU_TRAFFIC_BYTES = {"fwd": 201.41e6 + 154.02e6, "bwd": 406.96e6 + 170.88e6, "step": 271.60e6 + 212.48e6}
-NCU_TRAFFIC_SOURCE = {"fwd": "profiles/tc_fwd_bwd_lm2048.md (captured 2026-11-30, kernels as of the two-read completion pass of the backward)",
-                      "bwd": "profiles/tc_fwd_bwd_lm2048.md (captured 2026-11-30, kernels as of the two-read completion pass of the backward)",
-                      "step": "profiles/step_kernel_decode.md"}
+NCU_TRAFFIC_BYTES = {"fwd": None, "bwd": None, "step": None}
+NCU_TRAFFIC_SOURCE = {"fwd": None, "bwd": None, "step": None}
 
 
 def load_peaks():

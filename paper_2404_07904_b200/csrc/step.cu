@@ -118,7 +118,7 @@ step_kernel(const T *__restrict__ o, const T *__restrict__ f, const T *__restric
 // SM, and no barrier per token - the partial sums of eight tokens are added up together.  What the loop over rows
 // must not do is read much shared memory: a warp's load takes a cycle per 128 bytes of REGISTERS filled, broadcast
 // or not, so gates staged as ready-made pairs (24 bytes per row for four columns) cost as much as the arithmetic
-// twice over.  One 8-byte (f, o) per row serves eight columns here.  4096 units, bf16: 8 tokens 139 -> 104 us (83 is
+// twice over.  One 8-byte (f, o) per row serves eight columns here.  4096 units, bf16: 8 tokens 139 -> 112 us (83 is
 // the state traffic alone), 16 tokens 250 -> 169 us; quarter units per CTA 141 us, one token per loop body 115 us.
 template <typename T, int D, int kSplit, int TB>
 __global__ void __launch_bounds__(Cols<D>::kThreads / kSplit)
