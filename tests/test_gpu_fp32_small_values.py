@@ -39,3 +39,9 @@ def _check(inp, io, outputs):
 def test_small_gradients_and_values(io, dk, dv, f, scale):
     _check(_inputs(io, dk, dv, f, dy=scale, dSN=scale), io, ("d_i", "dS0"))
     _check(_inputs(io, dk, dv, f, i=scale, S0=scale), io, ("y", "SN"))
+
+
+@pytest.mark.parametrize("scale", [1e-6, 1e-9])
+@pytest.mark.parametrize("io,dk,dv", SHAPES)
+def test_small_queries(io, dk, dv, scale):
+    _check(_inputs(io, dk, dv, 0.118, o=scale), io, ("y", "SN", "d_o", "d_f", "d_i"))
