@@ -45,3 +45,12 @@ def test_small_gradients_and_values(io, dk, dv, f, scale):
 @pytest.mark.parametrize("io,dk,dv", SHAPES)
 def test_small_queries(io, dk, dv, scale):
     _check(_inputs(io, dk, dv, 0.118, o=scale), io, ("y", "SN", "d_o", "d_f", "d_i"))
+
+
+# dA, X and their products with the decays reach the end of float32's range.  Bound: as above where the float32 terms themselves are
+# normal numbers (1e-8, decays of 2^-98); with 1e-14 the terms lie below 2^-126 unless they are lifted.
+@pytest.mark.parametrize("scale", [1e-8, 1e-14, 1e-20])
+@pytest.mark.parametrize("io,dk,dv", SHAPES)
+def test_small_gradients_of_the_gates(io, dk, dv, scale):
+    inp = _inputs(io, dk, dv, 0.118, dy=scale, dSN=scale)
+    _check(inp, io, ("d_o", "d_f") if scale > 1e-12 else ("d_o",))
