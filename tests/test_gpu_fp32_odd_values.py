@@ -35,3 +35,31 @@ def test_forward_with_one_odd_value(io, d, flags, t, bad):
     want_y, want_SN = ref.hgrn2_fwd(x["o"], x["f"], x["i"], x["S0"])
     assert G.rel_err(y, want_y[0, 1, t:, 5]) <= G.TOL[io]
     assert G.rel_err(SN, want_SN[0, 1, :, 5]) <= 1e-4
+
+
+# Bound of the finite values: the path's.
+@pytest.mark.parametrize("gamma", [0.5, 0.0])                                  # 0.0 with a hard gate: the pairwise form
+@pytest.mark.parametrize("t,s", [(100, 97), (100, 100), (20, 18)])            # (further apart, d_f before s cancels to less than its rounding)
+@pytest.mark.parametrize("io,d,flags", [("f32", 128, 0), ("f32", 64, 0), ("bf16", 64, 0)])
+def test_an_overflow_in_the_backward_stays_with_what_depends_on_it(io, d, flags, t, s, gamma):
+    # dY_t . V_s leaves float32 although every element of dY and V is finite
+    inp = W.make_inputs(W.scaled(W.CONFIGS["tiny_f32"], B=1, H=2, N=150, dk=d, dv=d, io=io, has_S0=True, has_dSN=True,
+                                 seed=71, gamma=gamma, scale=d ** -0.5))
+    if gamma == 0.0:
+        inp["f"][..., 3] = 0.03125
+    clean = G.gpu_fwd_bwd(inp, io, flags=flags)
+    big = W.round_to_bf16(np.float32([1e25]))[0]
+    x = dict(inp, i=inp["i"].copy(), dy=inp["dy"].copy())
+    x["i"][0, 1, s, 5] = big
+    x["dy"][0, 1, t, 5] = big
+    got, want = G.gpu_fwd_bwd(x, io, flags=flags), G.oracle_fwd_bwd(x)
+    keys = [c for c in range(d) if gamma or c != 3]                            # (the hard gate forgets V_s before t)
+    assert not np.isfinite(got["d_o"][0, 1, t, keys]).any()
+    assert not np.isfinite(got["d_f"][0, 1, s:t + 1, keys]).any()
+    for k in ("d_o", "d_f"):
+        np.testing.assert_array_equal(got[k][:, 0], clean[k][:, 0])
+    np.testing.assert_array_equal(got["d_o"][0, 1, :s], clean["d_o"][0, 1, :s])
+    rest = {"d_o": [n for n in range(150) if n != t], "d_f": [n for n in range(150) if not s <= n <= t]}
+    for k, rows in rest.items():
+        assert np.isfinite(got[k][0, 1, rows]).all(), k
+        assert G.rel_err(got[k][0, 1, rows], want[k][0, 1, rows]) <= G.TOL[io], k
