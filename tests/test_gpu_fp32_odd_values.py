@@ -2,9 +2,10 @@
 leading part would round to Inf."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import ref
-from paper_2404_07904_b200 import workloads as W
+from paper_2404_07904_b200 import binding, workloads as W
 from tests import gpu_util as G
 
 pytestmark = pytest.mark.gpu
@@ -63,3 +64,49 @@ def test_an_overflow_in_the_backward_stays_with_what_depends_on_it(io, d, flags,
     for k, rows in rest.items():
         assert np.isfinite(got[k][0, 1, rows]).all(), k
         assert G.rel_err(got[k][0, 1, rows], want[k][0, 1, rows]) <= G.TOL[io], k
+
+
+def _classes(x):
+    return np.where(np.isnan(x), 3, np.where(np.isinf(x), np.where(x > 0, 1, 2), 0))
+
+
+# What an Inf makes of the outputs, by the recurrence in float64: NaN, Inf and its sign where it is a sum of Inf alone.
+@pytest.mark.parametrize("name,t", [("i", 10), ("i", 100), ("o", 10), ("o", 100), ("dy", 10), ("dy", 100), ("S0", None), ("dSN", None)])
+@pytest.mark.parametrize("io,dk,dv", [("f32", 128, 128), ("f32", 64, 64), ("f32", 32, 128), ("bf16", 64, 64)])
+def test_one_inf_and_what_depends_on_it(io, dk, dv, name, t):
+    inp = W.make_inputs(W.scaled(W.CONFIGS["tiny_f32"], B=1, H=2, N=150, dk=dk, dv=dv, io=io, has_S0=True, has_dSN=True,
+                                 seed=73, gamma=0.5, scale=dk ** -0.5))
+    for k in ("o", "dy", "i"):
+        inp[k] = np.abs(inp[k])                                                # no two Inf of opposite sign meet in y, SN, d_o, d_i, dS0
+    x = dict(inp, **{name: inp[name].copy()})
+    if t is None:
+        x[name][0, 1, 7, 5] = np.inf
+    else:
+        x[name][0, 1, t, 5] = -np.inf
+    got, want = G.gpu_fwd_bwd(x, io), G.oracle_fwd_bwd(x)
+    for k in want:
+        np.testing.assert_array_equal(np.isfinite(got[k]), np.isfinite(want[k]), err_msg=k)
+        if k != "d_f":
+            np.testing.assert_array_equal(_classes(got[k]), _classes(want[k]), err_msg=k)
+        ok = np.isfinite(want[k])
+        assert G.rel_err(got[k][ok], want[k][ok]) <= G.TOL[io], k
+
+
+def test_an_inf_in_every_sequence_does_not_hold_the_call_up():
+    # with every output that depends on it summed in full such a call took 300 times as long
+    w = W.scaled(W.CONFIGS["tiny_f32"], B=2, H=16, N=1024, dk=128, dv=128, gamma=0.5, scale=128 ** -0.5)
+    t = G.to_dev(W.make_inputs(w), "f32")
+    bad = t["i"].clone()
+    bad[:, :, 10, 5] = float("inf")
+
+    def once(i):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        _, _, saved, ws, _ = binding.hgrn2_fwd(t["o"], t["f"], i, None)
+        binding.hgrn2_bwd(t["o"], t["f"], i, None, t["dy"], None, saved, ws=ws)
+        b.record()
+        torch.cuda.synchronize()
+        return a.elapsed_time(b)
+
+    clean = min(once(t["i"]) for _ in range(5))
+    assert min(once(bad) for _ in range(3)) <= 40 * clean
