@@ -6,7 +6,7 @@ import torch
 
 from oracle import ref
 from paper_2404_07904_b200 import binding, workloads as W
-from tests import gpu_util as G
+from tests import gpu_util as G, test_gpu_gated as gated, test_gpu_varlen as varlen
 
 pytestmark = pytest.mark.gpu
 
@@ -110,3 +110,51 @@ def test_an_inf_in_every_sequence_does_not_hold_the_call_up():
 
     clean = min(once(t["i"]) for _ in range(5))
     assert min(once(bad) for _ in range(3)) <= 40 * clean
+
+
+def _check(got, want, clean, want_clean, tol):
+    """Every output of a call with one odd value: Inf or NaN where the recurrence in float64 has it, what the value does not reach as
+    without it, the rest to the path's bound.  Beyond 1e37 (sums of the largest floats) it is Inf, NaN or at least large."""
+    for k in want:
+        g, w = got[k], want[k]
+        large = np.isfinite(w) & (np.abs(w) >= 1e37)
+        assert (~np.isfinite(g[large]) | (np.abs(g[large]) > 1e36)).all(), k
+        np.testing.assert_array_equal(np.isfinite(g[~large]), np.isfinite(w[~large]), err_msg=k)
+        same = w == want_clean[k]
+        assert np.abs(g[same] - clean[k][same]).max(initial=0) <= tol * np.abs(want_clean[k]).max(), k
+        rest = ~same & ~large & np.isfinite(w)
+        assert np.abs(g[rest] - w[rest]).max(initial=0) <= tol * np.abs(w[rest]).max(initial=0), k
+
+
+BAD = [np.inf, np.nan, np.finfo(np.float32).max, np.finfo(np.float32).min]
+SHAPES = [(io, dk, dv, bad) for io, dk, dv in (("f32", 128, 128), ("f32", 64, 64), ("f32", 32, 128), ("bf16", 64, 64), ("bf16", 128, 16))
+          for bad in BAD if io == "f32" or not np.isfinite(bad)]             # (the tiles hold every finite bf16)
+
+
+@pytest.mark.parametrize("name,t", [("i", 10), ("i", 100), ("o", 10), ("o", 100), ("dy", 10), ("dy", 100), ("S0", None), ("dSN", None)])
+@pytest.mark.parametrize("io,dk,dv,bad", SHAPES)
+def test_every_output_with_one_odd_value(io, dk, dv, name, t, bad):
+    inp = W.make_inputs(W.scaled(W.CONFIGS["tiny_f32"], B=1, H=2, N=150, dk=dk, dv=dv, io=io, has_S0=True, has_dSN=True,
+                                 seed=74, gamma=0.5, scale=dk ** -0.5))
+    inp["dy"] = inp["dy"] * np.float32(0.125)                                  # (below 1: no product with the largest float overflows)
+    x = dict(inp, **{name: inp[name].copy()})
+    x[name][(0, 1, 7, 5) if t is None else (0, 1, t, 5)] = bad
+    _check(G.gpu_fwd_bwd(x, io), G.oracle_fwd_bwd(x), G.gpu_fwd_bwd(inp, io), G.oracle_fwd_bwd(inp), G.TOL[io])
+
+
+@pytest.mark.parametrize("name,bad", [("zi", np.inf), ("zi", np.nan), ("zo", np.inf), ("zo", np.nan), ("zf", np.inf), ("dy", np.inf), ("dy", np.nan)])
+@pytest.mark.parametrize("io,d", [("f32", 128), ("bf16", 64)])
+def test_every_output_of_the_gated_call_with_one_odd_value(io, d, name, bad):
+    inp = gated._inputs(1, 2, 150, d, io, 75, 0.5, 0.9)
+    x = dict(inp, **{name: inp[name].copy()})
+    x[name][0, 1, 70, 5] = bad
+    _check(gated._run(x, io)[0], gated._oracle(x), gated._run(inp, io)[0], gated._oracle(inp), G.TOL[io])
+
+
+@pytest.mark.parametrize("bad", BAD)
+@pytest.mark.parametrize("name", ["i", "o", "dy"])
+def test_every_output_of_a_packed_batch_with_one_odd_value(name, bad):
+    inp = varlen._packed_inputs([70, 0, 130, 1, 64], 2, 64, "f32", 76, gamma=0.5)
+    x = dict(inp, **{name: inp[name].copy()})
+    x[name][1, 150, 5] = bad
+    _check(varlen._run_gpu(x, "f32")[0], varlen._oracle(x), varlen._run_gpu(inp, "f32")[0], varlen._oracle(inp), G.TOL["f32"])
